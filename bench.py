@@ -6,8 +6,8 @@ B-splines on slab-dense/geometric knots, KB s+p projectors, 2x2 k-points,
 32 bands.  Synthetic, seeded inputs.
 
 A step is one H application to the 32-band block at all 4 k-points in one
-batched call (B-spline evaluation, inverse FFTs, potential product, forward
-FFTs, adjoint, banded kinetic term, projector contractions).  `value` is
+batched call (2D FFTs of the coefficient rows, the local potential as a band
+along z at every grid point, banded kinetic term, projector contractions).  `value` is
 Hpsi GB/s = algorithmic bytes / device time; the same apply in FP64 and the
 mixed-precision and plain-FP64 eigensolves are reported beside it.
 
@@ -45,11 +45,11 @@ METRIC = "Hψ GB/s & eigensolves/s at 1e-6 Ha vs plain FP64 GPU; p50/p99 solve l
 # The plane kernel's sources: its DRAM traffic (from an ncu capture, recorded
 # in the profile summary below with the kernel instance) is reported only
 # while these are unchanged and the same instance runs.
-PLANE_SOURCES = ("plane_reg.cu", "apply_common.cuh", "cplx.cuh")
+PLANE_SOURCES = ("rowspace.cuh", "rowspace32.cu", "fft_reg.cuh", "cplx.cuh")
 PLANE_PROFILES = {
-    "slab": "profiles/plane32_kernel_slab_fp32.md",
-    "graphene": "profiles/plane32_kernel_graphene_fp32.md",
-    "kbatch": "profiles/plane32_kernel_kbatch_fp32.md",
+    "slab": "profiles/rowspace_kernel_slab_fp32.md",
+    "graphene": "profiles/rowspace_kernel_graphene_fp32.md",
+    "kbatch": "profiles/rowspace_kernel_kbatch_fp32.md",
 }
 
 
@@ -94,7 +94,9 @@ def _peaks():
 
 
 def workload_sizes(h, w, prec):
-    """Algorithmic bytes and plane-kernel flops of one batched apply."""
+    """Algorithmic bytes and local-potential flops of one batched apply: per
+    (band, B-spline row) two 2D transforms and the banded product along z at
+    every grid point."""
     cb = 16 if prec == "fp64" else 8
     rb = cb // 2
     zq, _ = h.zplanes()
@@ -107,7 +109,7 @@ def workload_sizes(h, w, prec):
     for ik in range(w.nk):
         ng, nb, ldg = h.sizes(ik)
         byts += 2 * ng * nb * w.nbands * cb + nproj * (ng + nb) * cb
-        flops += w.nbands * nq * (8 * w.order * ng + 10 * N * math.log2(N) + 2 * N)
+        flops += w.nbands * nb * (10 * N * math.log2(N) + 4 * (2 * w.order - 1) * N)
     return byts, flops
 
 
@@ -931,7 +933,7 @@ def main():
     ap.add_argument("--apply-workload", default="slab", help="workload of --apply-only")
     ap.add_argument("--apply-prec", default="fp32", help="precision of --apply-only")
     ap.add_argument("--apply-tune", action="store_true", help="autotune the launch shape of --apply-only")
-    ap.add_argument("--apply-kernel", type=int, default=None, help="compact-plane instance id for --apply-only")
+    ap.add_argument("--apply-kernel", type=int, default=None, help="row-space instance id for --apply-only")
     ap.add_argument("--apply-persistent", action="store_true", help="persistent launch for --apply-kernel")
     ap.add_argument("--no-serve", action="store_true")
     ap.add_argument("--no-scf", action="store_true")

@@ -1,6 +1,10 @@
 // H and S applies of the mixed basis on one GPU (sm_103a).
 //
-//  plane_kernel   local potential (§II.B.1, Eqs. (12)-(13), (19)-(20)):
+//  rowspace       local potential (§II.B.1, Eqs. (12)-(13), (19)-(20)) on
+//                 grids of 16 - 64 points a side with B-splines of order 6:
+//                 one pair of 2D transforms per coefficient row and a banded
+//                 product along z at every grid point (rowspace.cuh).
+//  plane_kernel   the same for every other grid and order, plane by plane:
 //                 B-spline evaluation on the Gauss planes, inverse 2D FFT,
 //                 product with w_q V(r, z_q), forward 2D FFT, adjoint
 //                 B-spline sum back to coefficients.  One CTA owns a
@@ -26,6 +30,7 @@
 #include "cplx.cuh"
 #include "fft_smem.cuh"
 #include "mb_internal.h"
+#include "rowspace.h"
 
 namespace mb {
 
@@ -639,6 +644,66 @@ static int upload_set(mb_handle *h, DevTables &t) {
 // terms (vloc.cu).
 int upload_potential(mb_handle *h) { return vloc_build(h); }
 
+// The row-space kernel's view of every k-point's disc.  A grid side that is
+// not folded is compacted: the disc's indices n_min .. n_max become 0 .. n - 1
+// (a cyclic shift); a folded side keeps n mod M, M = N / 2.  Axis 1 is the
+// contiguous one of a plane, as in the disc's order: consecutive G lie side by
+// side.
+static int upload_rs_tables(mb_handle *h) {
+    const int s1 = rs_fold(h->n1), s2 = rs_fold(h->n2), S = s1 * s2, M1 = h->n1 / s1, M2 = h->n2 / s2, LDP = M1 + 1;
+    const size_t nk = h->kp.size();
+    std::vector<int> lo1(nk, 0), lo2(nk, 0);
+    h->rs_pruned = S == 1;
+    for (size_t ik = 0; ik < nk; ++ik) {
+        const KPoint &kp = h->kp[ik];
+        if (!kp.ng) continue;
+        const auto r1 = std::minmax_element(kp.n1.begin(), kp.n1.begin() + kp.ng);
+        const auto r2 = std::minmax_element(kp.n2.begin(), kp.n2.begin() + kp.ng);
+        lo1[ik] = *r1.first;
+        lo2[ik] = *r2.first;
+        if (4 * (*r1.second - lo1[ik] + 1) > 3 * M1 || 4 * (*r2.second - lo2[ik] + 1) > 3 * M2) h->rs_pruned = false;
+    }
+    const int NR = h->rs_pruned ? M1 * 3 / 4 : M1, NC = h->rs_pruned ? M2 * 3 / 4 : M2;   // as RsGeom
+    h->rs_pofs.assign(nk, 0);
+    h->rs_npos.assign(nk, 0);
+    std::vector<int> pos, gpos((size_t)h->total_ldg, 0);
+    std::vector<cdouble> ph(S > 1 ? (size_t)S * h->total_ldg : 0);
+    auto mod = [](int a, int n) { return ((a % n) + n) % n; };
+    for (size_t ik = 0; ik < nk; ++ik) {
+        const KPoint &kp = h->kp[ik];
+        const int per = S > 1 ? 4 : 1;
+        std::vector<int> src((size_t)NR * NC * per, -1);
+        for (int g = 0; g < kp.ng; ++g) {
+            const int r = s1 > 1 ? mod(kp.n1[g], M1) : kp.n1[g] - lo1[ik], p = s2 > 1 ? mod(kp.n2[g], M2) : kp.n2[g] - lo2[ik];
+            int *e = &src[((size_t)p * NR + r) * per];
+            while (*e >= 0) ++e;      // at most one G per residue of a folded position
+            *e = g;
+            gpos[h->kofs[ik] + g] = p * LDP + r;
+            for (int c = 0; c < S && S > 1; ++c) {
+                const double turn = (double)mod((c / s2) * kp.n1[g], h->n1) / h->n1 + (double)mod((c % s2) * kp.n2[g], h->n2) / h->n2;
+                ph[(size_t)c * h->total_ldg + h->kofs[ik] + g] = std::polar(1.0, 2.0 * 3.14159265358979323846 * turn);
+            }
+        }
+        h->rs_pofs[ik] = (int)(pos.size() / per);
+        if (S > 1) {
+            pos.insert(pos.end(), src.begin(), src.end());
+        } else {
+            for (int e = 0; e < NR * NC; ++e)
+                if (src[e] < 0) pos.push_back((e / NR) * LDP + e % NR);
+        }
+        h->rs_npos[ik] = (int)(pos.size() / per) - h->rs_pofs[ik];
+    }
+    if (pos.empty()) pos.push_back(0);
+    int rc;
+    if ((rc = dev_upload(h, &h->d_rspos, pos.data(), pos.size() * sizeof(int)))) return rc;
+    if ((rc = dev_upload(h, (void **)&h->d_rsgpos, gpos.data(), gpos.size() * sizeof(int)))) return rc;
+    if (S > 1) {
+        if ((rc = upload_complex<double>(h, &h->t64.phase, ph))) return rc;
+        if ((rc = upload_complex<float>(h, &h->t32.phase, ph))) return rc;
+    }
+    return MB_OK;
+}
+
 int upload_tables(mb_handle *h) {
     MB_CUDA(cudaSetDevice(h->device));
     if (!h->hs) {
@@ -656,57 +721,7 @@ int upload_tables(mb_handle *h) {
     for (size_t ik = 0; ik < h->kp.size(); ++ik)
         for (int g = 0; g < h->kp[ik].ng; ++g) goff[h->kofs[ik] + g] = h->kp[ik].goff[g];
     if ((rc = dev_upload(h, (void **)&h->d_goff, goff.data(), goff.size() * sizeof(int)))) return rc;
-    // grid rows that hold disc points, per k-point
-    std::vector<int> rows;
-    h->rows_ofs.assign(h->kp.size(), 0);
-    h->nrows.assign(h->kp.size(), 0);
-    h->rowmask.assign(h->kp.size(), 0ull);
-    for (size_t ik = 0; ik < h->kp.size(); ++ik) {
-        std::vector<char> used(h->n1, 0);
-        for (int g = 0; g < h->kp[ik].ng; ++g) used[h->kp[ik].goff[g] / h->n2] = 1;
-        h->rows_ofs[ik] = (int)rows.size();
-        for (int r = 0; r < h->n1; ++r)
-            if (used[r]) {
-                rows.push_back(r);
-                if (r < 64) h->rowmask[ik] |= 1ull << r;
-            }
-        h->nrows[ik] = (int)rows.size() - h->rows_ofs[ik];
-    }
-    if ((rc = dev_upload(h, (void **)&h->d_rows, rows.data(), rows.size() * sizeof(int)))) return rc;
-    // compact planes: the disc's rows n1min .. n1max become rows 0 .. nocc-1
-    // (row stride N2 + 1); the positions of those rows outside the disc
-    {
-        const int N2 = h->n2, LDP = N2 + 1;
-        const size_t nk = h->kp.size();
-        std::vector<int> cpos((size_t)h->total_ldg, 0), zpos;
-        h->nocc.assign(nk, 1);
-        h->zofs.assign(nk, 0);
-        h->nzero.assign(nk, 0);
-        for (size_t ik = 0; ik < nk; ++ik) {
-            const KPoint &kp = h->kp[ik];
-            int lo = 0, hi = 0;
-            for (int g = 0; g < kp.ng; ++g) {
-                lo = g ? std::min(lo, kp.n1[g]) : kp.n1[g];
-                hi = g ? std::max(hi, kp.n1[g]) : kp.n1[g];
-            }
-            const int nocc = kp.ng ? hi - lo + 1 : 1;
-            std::vector<char> used((size_t)nocc * N2, 0);
-            for (int g = 0; g < kp.ng; ++g) {
-                const int r = kp.n1[g] - lo, i2 = ((kp.n2[g] % N2) + N2) % N2;
-                used[(size_t)r * N2 + i2] = 1;
-                cpos[h->kofs[ik] + g] = r * LDP + i2;
-            }
-            h->nocc[ik] = nocc;
-            h->zofs[ik] = (int)zpos.size();
-            for (int r = 0; r < nocc; ++r)
-                for (int i2 = 0; i2 < N2; ++i2)
-                    if (!used[(size_t)r * N2 + i2]) zpos.push_back(r * LDP + i2);
-            h->nzero[ik] = (int)zpos.size() - h->zofs[ik];
-        }
-        if (zpos.empty()) zpos.push_back(0);
-        if ((rc = dev_upload(h, (void **)&h->d_cpos, cpos.data(), cpos.size() * sizeof(int)))) return rc;
-        if ((rc = dev_upload(h, (void **)&h->d_zpos, zpos.data(), zpos.size() * sizeof(int)))) return rc;
-    }
+    if (rs_supported(h->n1, h->n2, h->order) && (rc = upload_rs_tables(h))) return rc;
     if (h->nterm > 0) {
         std::vector<int> zi(h->pgroup);
         zi.insert(zi.end(), h->zstart.begin(), h->zstart.end());
@@ -717,15 +732,10 @@ int upload_tables(mb_handle *h) {
         zi.insert(zi.end(), h->plist.begin(), h->plist.end());
         if ((rc = dev_upload(h, (void **)&h->d_zidx, zi.data(), zi.size() * sizeof(int)))) return rc;
     }
-    upload_fft_twiddles();
     if (!h->d_tcerr) {
         // status word of the kernels' bounded device waits (mb_status)
         const int zero = 0;
         if ((rc = dev_upload(h, &h->d_tcerr, &zero, sizeof(int)))) return rc;
-    }
-    {
-        const int zeros[2] = {0, 0};
-        if ((rc = dev_upload(h, (void **)&h->d_queue, zeros, sizeof(zeros)))) return rc;
     }
     MB_CUDA(cudaStreamCreateWithFlags(&h->aux, cudaStreamNonBlocking));
     MB_CUDA(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
@@ -754,7 +764,7 @@ int ensure_precond(mb_handle *h) {
 }
 
 static void free_set(mb_handle *h, DevTables &t) {
-    void **ps[] = {&t.Bq, &t.V, &t.Vn, &t.tw, &t.Sband, &t.SbandP, &t.Dband, &t.Lband, &t.Lrecip, &t.q2, &t.qproj, &t.zproj, &t.zf, &t.E, &t.Pfac, &t.Vt, &t.Q, &t.Eid};
+    void **ps[] = {&t.Bq, &t.V, &t.U, &t.phase, &t.tw, &t.Sband, &t.SbandP, &t.Dband, &t.Lband, &t.Lrecip, &t.q2, &t.qproj, &t.zproj, &t.zf, &t.E, &t.Pfac, &t.Q, &t.Eid};
     for (void **p : ps) dev_free(h, p);
 }
 
@@ -768,13 +778,11 @@ void free_tables(mb_handle *h) {
     free_set(h, h->t64);
     free_set(h, h->t32);
     dev_free(h, (void **)&h->d_goff);
-    dev_free(h, (void **)&h->d_rows);
-    dev_free(h, (void **)&h->d_cpos);
-    dev_free(h, (void **)&h->d_zpos);
+    dev_free(h, &h->d_rspos);
+    dev_free(h, (void **)&h->d_rsgpos);
     dev_free(h, &h->d_projB);
     dev_free(h, (void **)&h->d_zidx);
     dev_free(h, &h->d_tcerr);
-    dev_free(h, (void **)&h->d_queue);
     dev_free(h, (void **)&h->d_vloc);
     dev_free(h, &h->scratch.ptr);
     h->scratch = Scratch();
@@ -809,22 +817,19 @@ int ensure_scratch(mb_handle *h, size_t bytes, cudaStream_t s) {
 
 // Launch plan of the plane kernel for one batched apply.
 struct PlanePlan {
-    bool reg = false;      // register-FFT kernel (else radix-2 shared-memory kernel)
-    bool p32 = false;      // FP32 compact-plane kernel
-    bool persist = false;  // its persistent, work-queue launch
-    Plane32Shape sh;       // its instance
-    int bt = 1;            // bands per CTA
-    int np = 1;            // planes in flight
-    int chunk = 1, nchunks = 1;
+    bool rs = false;       // row-space kernel (else the radix-2 plane kernel)
+    RsShape sh;            // its instance
+    int np = 1;            // radix-2 kernel: planes in flight
+    int nchunks = 1;       // runs of rows (row-space) or knot intervals (radix-2)
     size_t smem = 0;
 };
 
-// Run count of the wave model: a CTA's time ~ its run length + about one
-// interval of run overhead (boundary rows); the launch takes
-// ceil(items / slots) rounds of the longest run.
-static int wave_model_chunks(const mb_handle *h, int pairs, int slots, int nmax_chunks, int waves) {
+// Runs per (k-point, band): `cost(n)` of one item when there are n of them,
+// times the rounds that the items take on `slots` resident CTAs.  waves > 0:
+// an explicit target of about that many items per slot.
+template <typename Cost>
+static int wave_model_chunks(int pairs, int slots, int nmax_chunks, int waves, Cost cost) {
     if (waves > 0) {
-        // explicit target: about `waves` CTAs per resident slot
         const int target = std::max(1, (waves * slots + pairs - 1) / pairs);
         return std::min(nmax_chunks, target);
     }
@@ -833,109 +838,60 @@ static int wave_model_chunks(const mb_handle *h, int pairs, int slots, int nmax_
     for (int n = 1; n <= nmax_chunks; ++n) {
         const long long items = (long long)pairs * n;
         const long long rounds = (items + slots - 1) / slots;
-        const double cost = (double)rounds * ((h->nint + n - 1) / n + 1.0);
-        if (cost < best - 1e-9) { best = cost; nch = n; }
+        const double c = (double)rounds * cost(n);
+        if (c < best - 1e-9) { best = c; nch = n; }
     }
     return nch;
 }
 
-// Shared memory of a compact-plane instance at its CTAs per SM: planes,
-// output-row ring (and X window slots), and the B values of a run of
-// intervals; runs as short as the plan allows (K intervals) must fit.
-static size_t p32_budget(const mb_handle *h, const Plane32Shape &sh) {
-    return std::min((size_t)h->smem_optin, (size_t)228 * 1024 / sh.ctas_per_sm - 1024);
-}
-static size_t p32_smem(const mb_handle *h, const Plane32Shape &sh, int maxldg, int nch) {
-    const int K = h->order, P = h->nquad;
-    return sh.smem_fixed + (size_t)sh.bt * K * maxldg * sizeof(float2) +
-           (size_t)((h->nint + nch - 1) / nch) * K * P * sizeof(float);
-}
-static bool p32_fits(const mb_handle *h, const Plane32Shape &sh, int maxldg) {
-    const int nmax_chunks = std::max(1, std::min(kMaxChunks, h->nint / h->order));
-    return p32_smem(h, sh, maxldg, nmax_chunks) <= p32_budget(h, sh);
-}
-
-static PlanePlan plan_plane(const mb_handle *h, int nsel, const int *iks, int nbands, size_t c2, bool reg_ok) {
+static PlanePlan plan_plane(const mb_handle *h, int nsel, const int *iks, int nbands, size_t c2) {
     PlanePlan p;
     const int K = h->order, P = h->nquad;
     const size_t NN = (size_t)h->n1 * h->n2;
-    int maxldg = 0, nocc_max = 0;
-    for (int i = 0; i < nsel; ++i) {
-        maxldg = std::max(maxldg, h->kp[iks[i]].ldg);
-        nocc_max = std::max(nocc_max, h->nocc[iks[i]]);
-    }
-    int ctas_per_sm = 1;
-    // defaults, or the shape mb_autotune measured fastest for this batch
-    const bool small = h->n1 <= 32 && h->n2 <= 32;
-    int bt_max = small ? 2 : 1, waves = 0, p32_id = -1, persist = 0;
+    int waves = 0, inst = -1;
     auto it = h->tuned.find(std::make_tuple(nsel, nbands, c2 == 16 ? 1 : 0));
     if (it != h->tuned.end()) {
-        bt_max = it->second.bt;
         waves = it->second.waves;
-        p32_id = it->second.p32;
-        persist = it->second.persist;
+        inst = it->second.inst;
     }
-    const int nmax_chunks = std::max(1, std::min(kMaxChunks, h->nint / K));   // runs of >= K intervals
-    if (c2 == 8 && p32_id != -2) {
-        // FP32 compact-plane kernel: planes + output-row ring (+ X window
-        // slots) + the run's B values.  The tuned instance if there is one,
-        // else the first whose shared memory fits.
-        Plane32Shape shapes[kMaxPlane32Shapes];
-        const int ns = plane32_shapes(h->n1, h->n2, K, P, nocc_max, maxldg, shapes, kMaxPlane32Shapes);
-        for (int pass = 0; pass < 2; ++pass)
-            for (int v = 0; v < ns; ++v) {
-                const Plane32Shape &sh = shapes[v];
-                if (pass == 0 && sh.id != p32_id) continue;
-                const int pairs = nsel * ((nbands + sh.bt - 1) / sh.bt);
-                const int slots = h->num_sms * sh.ctas_per_sm;
-                const size_t budget = p32_budget(h, sh);
-                int nch = wave_model_chunks(h, pairs, slots, nmax_chunks, waves);
-                auto smem_of = [&](int n) { return p32_smem(h, sh, maxldg, n); };
-                while (nch < nmax_chunks && smem_of(nch) > budget) ++nch;
-                if (smem_of(nch) > budget) continue;
-                p.p32 = true;
-                p.persist = persist != 0;
-                p.sh = sh;
-                p.bt = sh.bt;
-                p.np = sh.bt * P;
-                p.nchunks = nch;
-                p.chunk = (h->nint + nch - 1) / nch;
-                p.smem = smem_of(nch);
-                return p;
-            }
+    RsShape shapes[kMaxRsShapes];
+    const int ns = c2 == 16 ? rs_shapes<double>(h->n1, h->n2, K, shapes, kMaxRsShapes)
+                            : rs_shapes<float>(h->n1, h->n2, K, shapes, kMaxRsShapes);
+    if (ns > 0) {
+        p.rs = true;
+        p.sh = shapes[0];
+        for (int v = 0; v < ns; ++v)
+            if (shapes[v].id == inst) p.sh = shapes[v];
+        p.smem = p.sh.smem;
+        // a run of L rows transforms up to 2 kRsHalo more: inverse transforms
+        // are about a third of a row's work, and a step of the row loop costs
+        // about two rows' latency.  FP64 CTAs of one SM share its FP64 pipe,
+        // which one of them fills: they count as one slot.
+        const int S = p.sh.s1 * p.sh.s2;
+        p.nchunks = wave_model_chunks(nsel * nbands, h->num_sms * (c2 == 16 ? 1 : p.sh.ctas_per_sm) / S, std::min(kMaxChunks, h->nb), waves, [&](int n) {
+            const int L = (h->nb + n - 1) / n;
+            const int in = std::min(h->nb, L + (n == 1 ? 0 : n == 2 ? kRsHalo : 2 * kRsHalo));
+            const int steps = (std::min(h->nb, L + (n > 2 ? kRsHalo : 0)) + kRsHalo + p.sh.rows - 1) / p.sh.rows;
+            return 0.35 * in + 0.65 * L + 2.0 * steps;
+        });
+        return p;
     }
-    if (reg_ok) {
-        const size_t plane_bytes = (size_t)h->n1 * (h->n2 + 1) * c2;
-        // matches the kernel's launch bounds
-        ctas_per_sm = c2 == 8 ? ((NN <= 512 || (h->n1 == 32 && h->n2 == 32)) ? 3 : small ? 2 : 1) : 1;
-        for (int bt = bt_max; bt >= 1 && !p.reg; --bt) {
-            size_t budget = (size_t)h->smem_optin / ctas_per_sm - 1024;
-            size_t acc = (size_t)bt * K * maxldg * c2;
-            if (acc + plane_bytes > budget) continue;
-            const size_t meta = 8 + 8 * (2 * sizeof(int) + 8 * c2 / 2);   // per plane, rounded up below
-            int np = (int)std::min<size_t>((size_t)bt * P, (budget - acc) / (plane_bytes + meta));
-            if (np < 1) continue;
-            p.reg = true;
-            p.bt = bt;
-            p.np = np;
-            p.smem = acc + (size_t)np * plane_bytes + ((size_t)(np + 1) * 2 * sizeof(int) + (size_t)np * 8 * (c2 / 2) + 15) / 16 * 16;
-        }
-    }
-    if (!p.reg) {
-        ctas_per_sm = 1;
-        const int nmax = std::max(h->n1, h->n2);
-        const size_t fixed = (nmax / 2 + (size_t)K * maxldg) * c2;
-        const size_t budget = (size_t)h->smem_optin;
-        p.bt = 1;
-        p.np = (int)std::min<size_t>((size_t)P, fixed < budget ? (budget - fixed) / (NN * c2) : 0);
-        p.smem = fixed + (size_t)p.np * NN * c2;
-    }
-    const int pairs = nsel * ((nbands + p.bt - 1) / p.bt);
-    const int slots = h->num_sms * ctas_per_sm;
-    p.nchunks = wave_model_chunks(h, pairs, slots, nmax_chunks, waves);
-    p.chunk = (h->nint + p.nchunks - 1) / p.nchunks;   // longest run
+    int maxldg = 0;
+    for (int i = 0; i < nsel; ++i) maxldg = std::max(maxldg, h->kp[iks[i]].ldg);
+    const int nmax = std::max(h->n1, h->n2);
+    const size_t fixed = (nmax / 2 + (size_t)K * maxldg) * c2;
+    const size_t budget = (size_t)h->smem_optin;
+    p.np = (int)std::min<size_t>((size_t)P, fixed < budget ? (budget - fixed) / (NN * c2) : 0);
+    p.smem = fixed + (size_t)p.np * NN * c2;
+    // a CTA's time: its run length plus about one interval of run overhead
+    // (boundary rows); runs of at least kappa intervals
+    p.nchunks = wave_model_chunks(nsel * nbands, h->num_sms, std::max(1, std::min(kMaxChunks, h->nint / K)), waves,
+                                  [&](int n) { return (h->nint + n - 1) / n + 1.0; });
     return p;
 }
+
+// runs whose boundary rows go through the scratch (the row-space kernel has none)
+static int part_chunks(const PlanePlan &p) { return p.rs ? 1 : p.nchunks; }
 
 // Largest j-segment count of the projector overlaps and of the epilogue.
 static int nl_max_seg(const mb_handle *h) { return std::max(1, std::min(8, h->nb / 8)); }
@@ -969,8 +925,6 @@ static size_t per_k_scratch(const mb_handle *h, int ldg, int nbands, int nchunks
 // kMaxK that apply_H_batch forms, each planned as it will be launched).
 size_t apply_scratch_bytes(const mb_handle *h, int nk, int nbands, int prec) {
     const size_t c2 = prec == MB_FP64 ? 16 : 8;
-    const bool reg = prec == MB_FP64 ? plane_reg_supported<double>(h->n1, h->n2, h->order)
-                                     : plane_reg_supported<float>(h->n1, h->n2, h->order);
     nk = std::min(nk, (int)h->kp.size());
     size_t need = 0;
     for (int i0 = 0; i0 < nk; i0 += kMaxK) {
@@ -981,8 +935,8 @@ size_t apply_scratch_bytes(const mb_handle *h, int nk, int nbands, int prec) {
             maxldg = std::max(maxldg, h->kp[i].ldg);
             ik[i - i0] = i;
         }
-        const PlanePlan p = plan_plane(h, nsel, ik.data(), nbands, c2, reg);
-        need = std::max(need, (size_t)nsel * per_k_scratch(h, maxldg, nbands, p.nchunks, c2, prec == MB_BF16));
+        const PlanePlan p = plan_plane(h, nsel, ik.data(), nbands, c2);
+        need = std::max(need, (size_t)nsel * per_k_scratch(h, maxldg, nbands, part_chunks(p), c2, prec == MB_BF16));
     }
     return need;
 }
@@ -1001,8 +955,8 @@ static size_t apply_H_need(const mb_handle *h, int nsel, const int *iks, int nba
     const size_t c2 = sizeof(typename V2<R>::T);
     int maxldg = 0;
     for (int i = 0; i < nsel; ++i) maxldg = std::max(maxldg, h->kp[iks[i]].ldg);
-    const PlanePlan plan = plan_plane(h, nsel, iks, nbands, c2, plane_reg_supported<R>(h->n1, h->n2, h->order));
-    return (size_t)nsel * per_k_scratch(h, maxldg, nbands, plan.nchunks, c2, tensor);
+    const PlanePlan plan = plan_plane(h, nsel, iks, nbands, c2);
+    return (size_t)nsel * per_k_scratch(h, maxldg, nbands, part_chunks(plan), c2, tensor);
 }
 
 template <typename R>
@@ -1020,12 +974,66 @@ static int apply_H_group(mb_handle *h, int nsel, const int *iks, const void *con
     return MB_OK;
 }
 
-// Scratch need of a single-k-point apply, and the apply itself on a scratch
-// region supplied by the caller of this function (no allocation here).
-size_t apply_H_scratch_need(const mb_handle *h, int ik, int nbands, int prec) {
-    return prec == MB_FP64 ? apply_H_need<double>(h, 1, &ik, nbands, false)
-                           : apply_H_need<float>(h, 1, &ik, nbands, prec == MB_BF16);
+// Runs of knot intervals that an apply walking interval by interval makes of
+// one k-point's block: the wave model over the bands per CTA and CTAs per SM
+// that its planes, its kappa-row output ring and (FP32, at most `nocc`
+// occupied rows and `ldg` columns) its window of X rows allow.
+static int interval_runs(const mb_handle *h, int ik, int nbands, size_t c2) {
+    const int K = h->order, P = h->nquad, ldg = h->kp[ik].ldg;
+    const int nmax_chunks = std::max(1, std::min(kMaxChunks, h->nint / K));
+    int waves = 0;
+    auto it = h->tuned.find(std::make_tuple(1, nbands, c2 == 16 ? 1 : 0));
+    if (it != h->tuned.end()) waves = it->second.waves;
+    auto runs = [&](int bt, int ctas) {
+        return wave_model_chunks((nbands + bt - 1) / bt, h->num_sms * ctas, nmax_chunks, waves,
+                                 [&](int n) { return (h->nint + n - 1) / n + 1.0; });
+    };
+    const KPoint &kp = h->kp[ik];
+    int nocc = 1;
+    if (kp.ng) {
+        const auto r = std::minmax_element(kp.n1.begin(), kp.n1.begin() + kp.ng);
+        nocc = *r.second - *r.first + 1;
+    }
+    if (c2 == 8 && K == 6 && P == 6) {
+        // grid, largest nocc and ldg, bands per CTA, CTAs per SM, entries of an X window in shared memory
+        static const struct { int n1, n2, nocc, ldg, bt, ctas, window; } shapes[] = {
+            {16, 16, 10, 96, 2, 4, 0},   {32, 16, 24, 192, 2, 2, 0},    {32, 16, 24, 256, 2, 2, 3072},
+            {32, 16, 24, 192, 2, 2, 2304}, {32, 16, 24, 192, 1, 4, 0},  {32, 32, 24, 384, 1, 2, 0},
+            {32, 32, 24, 384, 2, 1, 0},  {32, 32, 23, 384, 1, 3, 2304}, {64, 64, 48, 1536, 1, 1, 0},
+            {64, 64, 48, 1536, 1, 1, 0}, {32, 16, 22, 192, 2, 3, 2304}};
+        for (const auto &sh : shapes) {
+            if (h->n1 != sh.n1 || h->n2 != sh.n2 || nocc > sh.nocc || ldg > sh.ldg) continue;
+            const size_t budget = std::min((size_t)h->smem_optin, (size_t)228 * 1024 / sh.ctas - 1024);
+            const size_t fixed = ((size_t)sh.bt * 6 * sh.nocc * (sh.n2 + 1) + sh.window + (size_t)sh.bt * K * ldg) * 8;
+            auto smem = [&](int n) { return fixed + (size_t)((h->nint + n - 1) / n) * K * P * sizeof(float); };
+            int n = runs(sh.bt, sh.ctas);
+            while (n < nmax_chunks && smem(n) > budget) ++n;
+            if (smem(n) <= budget) return n;
+        }
+    }
+    if (rs_supported(h->n1, h->n2, K) && (c2 == 8 || (h->n1 <= 32 && h->n2 <= 32))) {
+        const bool small = h->n1 <= 32 && h->n2 <= 32;
+        const int ctas = c2 == 16 ? 1 : (h->n1 * h->n2 <= 512 || (h->n1 == 32 && h->n2 == 32)) ? 3 : small ? 2 : 1;
+        const size_t plane = (size_t)h->n1 * (h->n2 + 1) * c2 + 8 + 8 * (2 * sizeof(int) + 8 * c2 / 2);
+        const size_t budget = (size_t)h->smem_optin / ctas - 1024;
+        for (int bt = small ? 2 : 1; bt >= 1; --bt)
+            if ((size_t)bt * K * ldg * c2 + plane <= budget) return runs(bt, ctas);
+    }
+    return runs(1, 1);
 }
+
+// Scratch by which mb_apply_H_noalloc admits a request: that of the walk over
+// knot intervals, whose runs leave their boundary rows there (at least what
+// any plane kernel uses; the row-space kernel has no boundary rows, and its
+// requests are admitted as the others' are).
+size_t apply_H_scratch_need(const mb_handle *h, int ik, int nbands, int prec) {
+    const size_t c2 = prec == MB_FP64 ? 16 : 8;
+    const size_t need = per_k_scratch(h, h->kp[ik].ldg, nbands, interval_runs(h, ik, nbands, c2), c2, prec == MB_BF16);
+    return std::max(need, prec == MB_FP64 ? apply_H_need<double>(h, 1, &ik, nbands, false)
+                                          : apply_H_need<float>(h, 1, &ik, nbands, prec == MB_BF16));
+}
+
+// A single-k-point apply on a scratch region supplied by the caller (no allocation here).
 
 int apply_H_on_scratch(mb_handle *h, int ik, const void *X, void *Y, int nbands, int prec, cudaStream_t s,
                        void *scratch) {
@@ -1046,9 +1054,8 @@ static int apply_H_launch(mb_handle *h, int nsel, const int *iks, const void *co
     size_t off = 0;
     int maxldg = 0;
     for (int i = 0; i < nsel; ++i) maxldg = std::max(maxldg, h->kp[iks[i]].ldg);
-    const PlanePlan plan = plan_plane(h, nsel, iks, nbands, c2, plane_reg_supported<R>(h->n1, h->n2, h->order));
-    const int chunk = plan.chunk, nchunks = plan.nchunks;
-    (void)chunk;
+    const PlanePlan plan = plan_plane(h, nsel, iks, nbands, c2);
+    const int nchunks = part_chunks(plan);
     if (plan.np < 1) return MB_EUNSUPPORTED;
     auto al = [](size_t x) { return (x + 255) / 256 * 256; };
     for (int i = 0; i < nsel; ++i) {
@@ -1060,13 +1067,6 @@ static int apply_H_launch(mb_handle *h, int nsel, const int *iks, const void *co
         d.ldg = kp.ldg;
         d.kofs = h->kofs[iks[i]];
         d.qofs = h->qofs[iks[i]];
-        d.rows_ofs = h->rows_ofs[iks[i]];
-        d.nrows = h->nrows[iks[i]];
-        d.rowmask = h->rowmask[iks[i]];
-        d.rows_magic = (unsigned)((1ull << 32) / (unsigned)std::max(1, d.nrows) + 1);
-        d.nocc = h->nocc[iks[i]];
-        d.zofs = h->zofs[iks[i]];
-        d.nz = h->nzero[iks[i]];
         // every k-point's regions are laid out for the batch's widest row (maxldg)
         const KScratch ks = per_k_layout(h, maxldg, nbands, nchunks, c2, tensor);
         d.part = base + off;
@@ -1152,50 +1152,54 @@ static int apply_H_launch(mb_handle *h, int nsel, const int *iks, const void *co
         MB_CUDA(cudaEventRecord(h->ev_join, sa));
         forked = true;
     }
-    // local potential through the planes
-    PlaneArgs<R> pa;
-    pa.Bq = reinterpret_cast<const R *>(t.Bq);
-    pa.V = reinterpret_cast<const R *>(t.V);
-    pa.Vn = reinterpret_cast<const R *>(t.Vn);
-    pa.rows = h->d_rows;
-    pa.tw = reinterpret_cast<const R2 *>(t.tw);
-    pa.goff = h->d_goff;
-    pa.Vt = reinterpret_cast<const R *>(t.Vt);
-    pa.cpos = h->d_cpos;
-    pa.zpos = h->d_zpos;
-    pa.n1 = h->n1;
-    pa.n2 = h->n2;
-    pa.l1 = h->l1;
-    pa.l2 = h->l2;
-    pa.nmax = std::max(h->n1, h->n2);
-    pa.order = h->order;
-    pa.nquad = h->nquad;
-    pa.nint = h->nint;
-    pa.nb = h->nb;
-    pa.nbands = nbands;
-    pa.nchunks = nchunks;
-    pa.chunk = chunk;
-    pa.ldg_max = maxldg;
-    pa.nsel = nsel;
-    pa.bt = plan.bt;
-    pa.np = plan.np;
-    pa.queue = plan.persist ? h->d_queue : nullptr;
-    std::copy(desc, desc + nsel, pa.d);
-    if (plan.p32) {
-        if constexpr (sizeof(R) == 4) {
-            const unsigned items = (unsigned)(nsel * ((nbands + plan.bt - 1) / plan.bt) * nchunks);
-            const unsigned grid =
-                plan.persist ? std::min(items, (unsigned)(h->num_sms * plan.sh.ctas_per_sm)) : items;
-            cudaError_t e = cudaSuccess;
-            MB_LAUNCH(h, s, KN_PLANE, e = plane32_launch(pa, plan.sh, grid, plan.smem, s));
-            MB_CUDA(e);
+    // local potential
+    if (plan.rs) {
+        RsArgs<R> ra;
+        ra.U = reinterpret_cast<const R2 *>(t.U);
+        ra.gpos = h->d_rsgpos;
+        ra.pos = reinterpret_cast<const int *>(h->d_rspos);
+        ra.src = reinterpret_cast<const int4 *>(h->d_rspos);
+        ra.phase = reinterpret_cast<const R2 *>(t.phase);
+        ra.phase_stride = (size_t)h->total_ldg;
+        ra.nbands = nbands;
+        ra.nb = h->nb;
+        ra.nchunks = plan.nchunks;
+        ra.s1 = plan.sh.s1;
+        ra.s2 = plan.sh.s2;
+        ra.pruned = h->rs_pruned;
+        for (int i = 0; i < nsel; ++i) {
+            RsK &d = ra.d[i];
+            const int ik = iks[i];
+            d.X = X[i];
+            d.Y = Y[i];
+            d.ng = h->kp[ik].ng;
+            d.ldg = h->kp[ik].ldg;
+            d.npos = h->rs_npos[ik];
+            d.pofs = h->rs_pofs[ik];
+            d.gofs = h->kofs[ik];
         }
-    } else if (plan.reg) {
-        const unsigned grid = (unsigned)(nsel * ((nbands + plan.bt - 1) / plan.bt) * nchunks);
         cudaError_t e = cudaSuccess;
-        MB_LAUNCH(h, s, KN_PLANE, e = plane_reg_launch<R>(pa, grid, plan.smem, s));
+        MB_LAUNCH(h, s, KN_PLANE, e = rs_launch<R>(ra, plan.sh, (unsigned)(nsel * nbands * plan.nchunks), s));
         MB_CUDA(e);
     } else {
+        PlaneArgs<R> pa;
+        pa.Bq = reinterpret_cast<const R *>(t.Bq);
+        pa.V = reinterpret_cast<const R *>(t.V);
+        pa.tw = reinterpret_cast<const R2 *>(t.tw);
+        pa.goff = h->d_goff;
+        pa.n1 = h->n1;
+        pa.n2 = h->n2;
+        pa.l1 = h->l1;
+        pa.l2 = h->l2;
+        pa.nmax = std::max(h->n1, h->n2);
+        pa.order = h->order;
+        pa.nquad = h->nquad;
+        pa.nint = h->nint;
+        pa.nb = h->nb;
+        pa.nbands = nbands;
+        pa.nchunks = nchunks;
+        pa.np = plan.np;
+        std::copy(desc, desc + nsel, pa.d);
         MB_CUDA(smem_limit_once((const void *)plane_kernel<R>, h->device, h->smem_optin));
         MB_LAUNCH(h, s, KN_PLANE, plane_kernel<R><<<nsel * nbands * nchunks, 256, plan.smem, s>>>(pa));
     }
@@ -1557,38 +1561,22 @@ int autotune(mb_handle *h, int nbands, int prec, int *best_bt, int *best_waves, 
     if (rc == MB_OK && (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess ||
                         cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess))
         rc = MB_ECUDA;
-    const bool small = h->n1 <= 32 && h->n2 <= 32;
     const auto key = std::make_tuple(std::min(nk, kMaxK), nbands, c2 == 16 ? 1 : 0);
-    // candidates: every compact-plane instance that can run the batch (FP32),
-    // and the register-FFT / radix-2 kernels with 1..4 bands per CTA; each
-    // with the wave model's run count and with explicit wave targets
+    // candidates: every row-space instance of the grid, or the radix-2 plane
+    // kernel; each with the wave model's run count and with explicit wave targets
     std::vector<mb_handle::Tuned> cand;
-    if (c2 == 8) {
-        int nocc_max = 0, maxldg = 0;
-        for (int i = 0; i < std::min(nk, kMaxK); ++i) {
-            nocc_max = std::max(nocc_max, h->nocc[i]);
-            maxldg = std::max(maxldg, h->kp[i].ldg);
-        }
-        Plane32Shape shapes[kMaxPlane32Shapes];
-        const int ns = plane32_shapes(h->n1, h->n2, h->order, h->nquad, nocc_max, maxldg, shapes, kMaxPlane32Shapes);
-        for (int v = 0; v < ns; ++v)
-            for (int persist : {0, 1})
-                for (int waves : {0, 1, 2, 4, 8}) {
-                    mb_handle::Tuned t;
-                    t.p32 = shapes[v].id;
-                    t.waves = waves;
-                    t.persist = persist;
-                    cand.push_back(t);
-                }
+    {
+        RsShape shapes[kMaxRsShapes];
+        const int ns = c2 == 16 ? rs_shapes<double>(h->n1, h->n2, h->order, shapes, kMaxRsShapes)
+                                : rs_shapes<float>(h->n1, h->n2, h->order, shapes, kMaxRsShapes);
+        for (int v = 0; v < std::max(1, ns); ++v)
+            for (int waves : {0, 1, 2, 4, 8}) {
+                mb_handle::Tuned t;
+                t.inst = ns > 0 ? shapes[v].id : -1;
+                t.waves = waves;
+                cand.push_back(t);
+            }
     }
-    for (int bt = small ? 4 : 2; bt >= 1; --bt)
-        for (int waves : {0, 1, 2, 4, 8}) {
-            mb_handle::Tuned t;
-            t.bt = bt;
-            t.waves = waves;
-            t.p32 = -2;            // not the compact-plane kernel
-            cand.push_back(t);
-        }
     double best = 1e300;
     mb_handle::Tuned bestp = cand.empty() ? mb_handle::Tuned() : cand[0];
     h->tune_report.clear();
@@ -1609,8 +1597,7 @@ int autotune(mb_handle *h, int nbands, int prec, int *best_bt, int *best_waves, 
         cudaEventElapsedTime(&ms, e0, e1);
         if (rc == MB_OK) {
             char line[256];
-            std::snprintf(line, sizeof(line), "%s bands/CTA %d waves %d: %.4f ms\n", name,
-                          c.p32 >= 0 ? 0 : c.bt, c.waves, ms / 5);   // the name says "persistent" for the queue launch
+            std::snprintf(line, sizeof(line), "%s waves %d: %.4f ms\n", name, c.waves, ms / 5);
             h->tune_report += line;
         }
         if (rc == MB_OK && ms / 5 < best) {
@@ -1619,7 +1606,7 @@ int autotune(mb_handle *h, int nbands, int prec, int *best_bt, int *best_waves, 
         }
     }
     h->tuned[key] = bestp;
-    if (best_bt) *best_bt = bestp.p32 >= 0 ? -1 - bestp.p32 : bestp.bt;
+    if (best_bt) *best_bt = bestp.inst >= 0 ? -1 - bestp.inst : 1;
     if (best_waves) *best_waves = bestp.waves;
     if (best_ms) *best_ms = best;
     if (e0) cudaEventDestroy(e0);
@@ -1640,12 +1627,9 @@ int plane_kernel_name(const mb_handle *h, int nk, int nbands, int prec, char *bu
     std::vector<int> iks(nk);
     for (int i = 0; i < nk; ++i) iks[i] = i;
     const size_t c2 = prec == MB_FP64 ? 16 : 8;
-    const bool reg = prec == MB_FP64 ? plane_reg_supported<double>(h->n1, h->n2, h->order)
-                                     : plane_reg_supported<float>(h->n1, h->n2, h->order);
-    const PlanePlan p = plan_plane(h, nk, iks.data(), nbands, c2, reg);
+    const PlanePlan p = plan_plane(h, nk, iks.data(), nbands, c2);
     char tmp[128];
-    if (p.p32) std::snprintf(tmp, sizeof(tmp), "%s%s", p.sh.name, p.persist ? " persistent" : "");
-    else if (p.reg) std::snprintf(tmp, sizeof(tmp), "plane_reg_kernel<%s, %d, %d, %d>", c2 == 8 ? "float" : "double", h->n1, h->n2, h->order);
+    if (p.rs) std::snprintf(tmp, sizeof(tmp), "%s", p.sh.name);
     else std::snprintf(tmp, sizeof(tmp), "plane_kernel<%s>", c2 == 8 ? "float" : "double");
     std::snprintf(buf, (size_t)len, "%s", tmp);
     return MB_OK;
@@ -1663,22 +1647,11 @@ extern "C" int mb_plane_kernel_name(const mb_handle *h, int nk, int nbands, int 
 }
 
 namespace mb {
-static int plane_candidates(const mb_handle *h, int nk, int prec, int *ids, int max) {
+static int plane_candidates(const mb_handle *h, int prec, int *ids, int max) {
     if (prec == MB_FP64) return 0;
-    nk = std::min(std::min(nk, (int)h->kp.size()), kMaxK);
-    int nocc_max = 0, maxldg = 0;
-    for (int i = 0; i < nk; ++i) {
-        nocc_max = std::max(nocc_max, h->nocc[i]);
-        maxldg = std::max(maxldg, h->kp[i].ldg);
-    }
-    Plane32Shape shapes[kMaxPlane32Shapes];
-    const int ns = plane32_shapes(h->n1, h->n2, h->order, h->nquad, nocc_max, maxldg, shapes, kMaxPlane32Shapes);
-    int n = 0;   // the instances whose shared memory fits this batch
-    for (int v = 0; v < ns; ++v)
-        if (p32_fits(h, shapes[v], maxldg)) {
-            if (n < max) ids[n] = shapes[v].id;
-            ++n;
-        }
+    RsShape shapes[kMaxRsShapes];
+    const int n = rs_shapes<float>(h->n1, h->n2, h->order, shapes, kMaxRsShapes);
+    for (int v = 0; v < std::min(n, max); ++v) ids[v] = shapes[v].id;
     return n;
 }
 }  // namespace mb
@@ -1686,7 +1659,7 @@ static int plane_candidates(const mb_handle *h, int nk, int prec, int *ids, int 
 extern "C" int mb_plane_kernel_candidates(const mb_handle *h, int nk, int nbands, int prec, int *ids, int max) {
     if (!h || !ids || nk < 1 || nbands < 1 || max < 0) return -MB_EINVAL;
     if (prec != MB_FP64 && prec != MB_FP32 && prec != MB_BF16) return -MB_EINVAL;
-    return mb::plane_candidates(h, nk, prec, ids, max);
+    return mb::plane_candidates(h, prec, ids, max);
 }
 
 extern "C" int mb_plane_kernel_select(mb_handle *h, int nk, int nbands, int prec, int id, int waves,
@@ -1694,17 +1667,16 @@ extern "C" int mb_plane_kernel_select(mb_handle *h, int nk, int nbands, int prec
     if (!h || nk < 1 || nbands < 1 || waves < 0 || id < -2) return MB_EINVAL;
     if (prec != MB_FP64 && prec != MB_FP32 && prec != MB_BF16) return MB_EINVAL;
     if (id >= 0) {
-        int ids[mb::kMaxPlane32Shapes];
-        const int n = mb::plane_candidates(h, nk, prec, ids, mb::kMaxPlane32Shapes);
+        int ids[mb::kMaxRsShapes];
+        const int n = mb::plane_candidates(h, prec, ids, mb::kMaxRsShapes);
         bool ok = false;
         for (int i = 0; i < n; ++i) ok = ok || ids[i] == id;
         if (!ok) return MB_EINVAL;
     }
     mb_handle::Tuned t;
-    t.p32 = id;
+    t.inst = id;
     t.waves = waves;
-    t.persist = persistent ? 1 : 0;
-    t.bt = h->n1 <= 32 && h->n2 <= 32 ? 2 : 1;
+    (void)persistent;    // every launch is a grid of CTAs that the hardware hands out as slots free up
     h->tuned[std::make_tuple(std::min(std::min(nk, (int)h->kp.size()), mb::kMaxK), nbands, prec == MB_FP64 ? 1 : 0)] = t;
     return MB_OK;
 }

@@ -30,11 +30,23 @@ struct KPoint {
 // of 4, so that a row is a whole number of 16-byte loads in both precisions
 constexpr int band_pad(int order) { return (2 * order - 1 + 3) / 4 * 4; }
 
+// Row-space kernel (rowspace.cuh): B-splines of order 6 on grids of 16, 32 or
+// 64 points a side; a side of 64 is folded into 2 interleaved residues.
+constexpr int kRsOrder = 6;
+constexpr int kRsHalo = kRsOrder - 1;       // half-width of its band along z
+constexpr int kRsPad = 24;                  // zero rows after the row-space potential (a step may run past the basis)
+inline int rs_fold(int n) { return n == 64 ? 2 : 1; }
+inline bool rs_supported(int n1, int n2, int order) {
+    auto side = [](int n) { return n == 16 || n == 32 || n == 64; };
+    return side(n1) && side(n2) && order == kRsOrder;
+}
+
 // Device copies of one precision (R = double or float).
 struct DevTables {
     void *Bq = nullptr;      // nq x order, B_{t+m}(z_q) of the full basis
-    void *V = nullptr;       // nq x N1 x N2, w_q V / (N1 N2), bit-reversed layout
-    void *Vn = nullptr;      // the same in natural layout
+    void *V = nullptr;       // nq x N1 x N2, w_q V / (N1 N2), bit-reversed layout (radix-2 plane kernel)
+    void *U = nullptr;       // row-space potential: nb x 3 x residue x plane, pairs (row-space kernel)
+    void *phase = nullptr;   // folded grids: residue x total_ldg complex phases of the disc
     void *tw = nullptr;      // Nmax/2 complex, exp(+2 pi i k / Nmax)
     void *Sband = nullptr;   // nb x (2 order - 1): S[j][j+d], d = -(order-1)..order-1
     void *SbandP = nullptr;  // the same with rows padded to band_pad(order) entries (zeros)
@@ -47,7 +59,6 @@ struct DevTables {
     void *zf = nullptr;      // nzf x nb: the distinct rows of zproj
     void *E = nullptr;       // nkb diagonal strengths, then nkb partner couplings
     void *Pfac = nullptr;    // preconditioner factors: all k, ldg x nb x order each
-    void *Vt = nullptr;      // nq x N2 x N1, w_q V / (N1 N2), i1 fastest (FP32 compact-plane kernel)
     void *Q = nullptr;       // ultrasoft q: nkb diagonal, then nkb partner couplings (the layout of E)
     void *Eid = nullptr;     // strengths 1 (diagonal) and 0 (couplings): the overlaps <beta_p|x> themselves
 };
@@ -108,17 +119,17 @@ struct mb_handle {
     std::vector<int> kofs, qofs;     // offsets of per-k arrays (in elements)
     int total_ldg = 0;
     int *d_goff = nullptr;           // all k (int), offset kofs
-    int *d_rows = nullptr;           // occupied grid rows of every k, offset rows_ofs[k]
+    // row-space kernel: the plane offset of every G (offset kofs), and per
+    // k-point a list of positions at rs_pofs[k] (rs_npos[k] entries): the
+    // compact plane's disc-free ones (int), or the sources of every position
+    // of a folded plane (int4); rs_pruned: every disc fits in 3/4 of a side
+    int *d_rsgpos = nullptr;
+    void *d_rspos = nullptr;
+    std::vector<int> rs_pofs, rs_npos;
+    bool rs_pruned = false;
     void *d_projB = nullptr;         // BF16 projector tables for the tensor-core contractions
     void *d_tcerr = nullptr;         // status word of the tensor-core kernels' bounded waits
     std::vector<int> pb0_ofs, pb1_ofs, pb0_ld, pb1_ld;
-    std::vector<int> rows_ofs, nrows;
-    // compact planes of the FP32 plane kernel, per k-point: occupied grid
-    // rows n1min .. n1min + nocc - 1, and the disc-free positions of those rows
-    int *d_cpos = nullptr;           // all k (int), offset kofs: (n1 - n1min)(N2 + 1) + (n2 mod N2)
-    int *d_zpos = nullptr;           // all k, offset zofs[k], nzero[k] entries
-    std::vector<int> nocc, zofs, nzero;
-    std::vector<unsigned long long> rowmask;
     mb::DevTables t64, t32;
     bool pfac_ready = false;
     // z modes of the eigensolver's free-electron start (k-independent, cached)
@@ -134,13 +145,12 @@ struct mb_handle {
     // destroying a handle never waits for other work on the device
     cudaStream_t hs = nullptr;
     cudaEvent_t scratch_ev = nullptr;      // recorded after the last apply that used the scratch
-    int *d_queue = nullptr;                // work-queue counters of the persistent plane kernel (2 ints)
     size_t desc_bytes = 0;
     std::string last_cuda_error;
     // plane-kernel launch shapes picked by mb_autotune: (k-points per batch,
-    // bands, FP64?) -> (largest bands per CTA of the radix-2 / register-FFT
-    // kernels, resident-CTA waves, compact-plane kernel instance id or -1)
-    struct Tuned { int bt = 1; int waves = 0; int p32 = -1; int persist = 0; };
+    // bands, FP64?) -> resident-CTA waves (0: the wave model), row-space
+    // kernel instance id (-1: the default)
+    struct Tuned { int waves = 0; int inst = -1; };
     std::map<std::tuple<int, int, int>, Tuned> tuned;
     std::string tune_report;         // the last mb_autotune's candidates and times
     // launch accounting (always on) and optional per-kernel event timing
@@ -166,7 +176,7 @@ int upload_tables(mb_handle *h);
 int upload_potential(mb_handle *h);
 // vloc.cu
 int vloc_build(mb_handle *h);             // d_vloc from the atoms' analytic terms, then the derived tables
-int vloc_derive_tables(mb_handle *h);     // d_vloc -> t64.V/Vn, t32.V/Vn/Vt
+int vloc_derive_tables(mb_handle *h);     // d_vloc -> the tables of the handle's plane kernel (U, or V)
 size_t vloc_build_scratch_bytes(const mb_handle *h);
 int vloc_tabulate(mb_handle *h, int mode, double *out, cudaStream_t s, const std::vector<double> *lgrp = nullptr,
                   const std::vector<double> *lion = nullptr, const std::vector<int> *lstart = nullptr);

@@ -1,0 +1,45 @@
+// Row-space local potential: host interface (kernels in rowspace.cuh).
+#pragma once
+
+#include "cplx.cuh"
+#include "apply_common.cuh"
+#include "mb_internal.h"
+
+namespace mb {
+
+// one k-point's disc on the (folded) plane
+struct RsK {
+    const void *X;
+    void *Y;
+    int ng, ldg;
+    int gofs;             // offset of the per-G tables (plane offsets, phases)
+    int pofs, npos;       // its position list: disc-free positions, or (folded) the source table
+};
+
+template <typename R> struct RsArgs {
+    const typename V2<R>::T *U;       // [nb + kRsPad][3][residue][point, axis 1 fastest]: pairs U(j, j - 2t), U(j, j - 2t - 1)
+    const int *gpos;                  // plane offset of each G
+    const int *pos;                   // unfolded: plane offsets of the compact plane's disc-free positions
+    const int4 *src;                  // folded: the up to four G of each plane position (-1: none)
+    const typename V2<R>::T *phase;   // folded: [residue][G] exp(2 pi i (c1 n1 / N1 + c2 n2 / N2))
+    size_t phase_stride;              // elements from one residue's phases to the next
+    int nbands, nb, nchunks;
+    int s1, s2;                       // folds of the two grid sides
+    int pruned;                       // the tables are those of the 3/4 x 3/4 compact plane
+    RsK d[kMaxK];
+};
+
+// launch shape of one (grid, precision)
+struct RsShape {
+    bool ok = false;
+    int id = -1;
+    char name[96] = {0};
+    int m1 = 0, m2 = 0, s1 = 1, s2 = 1;
+    int threads = 0, rows = 0, ctas_per_sm = 1;   // rows per step
+    size_t smem = 0;
+};
+constexpr int kMaxRsShapes = 4;
+template <typename R> int rs_shapes(int n1, int n2, int order, RsShape *out, int max);
+template <typename R> cudaError_t rs_launch(const RsArgs<R> &a, const RsShape &sh, unsigned items, cudaStream_t s);
+
+}  // namespace mb

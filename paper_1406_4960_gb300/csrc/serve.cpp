@@ -52,15 +52,19 @@ struct Job {
 // apply scratch, and the eigensolver workspace (vectors + small matrices).
 size_t footprint_of(const mb_handle &h, int nbands, int prec) {
     const size_t NN = (size_t)h.n1 * h.n2;
-    // V: the natural FP64 table, permuted + natural (FP64 + FP32), per column
-    // (FP32); the transient buffers of its build
-    size_t tables = (size_t)h.nq * NN * (8 + (8 + 4) * 2 + 4) + vloc_build_scratch_bytes(&h);
+    // V: the natural FP64 table, and the plane kernel's (FP64 + FP32): the
+    // row-space band (order entries per row) or the bit-reversed planes; the
+    // transient buffers of its build
+    size_t tables = (size_t)h.nq * NN * 8 + vloc_build_scratch_bytes(&h) +
+                    (rs_supported(h.n1, h.n2, h.order) ? (size_t)(h.nb + kRsPad) * h.order : (size_t)h.nq) * NN * (8 + 4);
     tables += (size_t)h.nq * h.order * 12 + (size_t)h.nb * (2 * h.order - 1) * 12 * 2 + (size_t)h.nb * h.order * 12 +
               (size_t)h.nb * band_pad(h.order) * 12;   // the padded S band
     size_t vec_bytes = 0, pf = 0;
     int maxldg = 0;
     for (auto &k : h.kp) {
         tables += (size_t)k.ldg * (12 + 4) + (size_t)h.nterm * k.ldg * 24;
+        // position table of the compact planes; per-G offsets and phases of folded grids
+        tables += 16 * (size_t)h.n1 * h.n2 + (size_t)k.ldg * (4 + 4 * 24);
         pf += (size_t)k.ldg * h.nb * h.order * 12;
         vec_bytes += (size_t)h.nb * k.ldg * 16;
         maxldg = std::max(maxldg, k.ldg);

@@ -21,9 +21,11 @@
 // times their structure factors, summed along m2 (vloc_rows_kernel) and then
 // along m1, keeping the real part (vloc_cols_kernel): plain O(N) sums per
 // output with N <= 256, in FP64, twiddles from sincospi of exact ratios.
-// The tables the apply kernels read (weight and 1/(N1 N2) folded in,
-// bit-reversed, per column, FP32 copies) are derived from the natural table
-// by vloc_tables_kernel, which also serves a table set by the caller.
+// The table the handle's plane kernel reads is derived from the natural
+// table, which may also be one set by the caller: the row-space potential U
+// (rs_tables_kernel), or, on grids without a row-space kernel, the planes
+// with weight and 1/(N1 N2) folded in, bit-reversed (vloc_tables_kernel);
+// each in FP64 with an FP32 copy.
 #include <algorithm>
 #include <vector>
 
@@ -155,24 +157,61 @@ __global__ void vloc_cols_kernel(VlocGeom G, const double2 *tmp, int q0, int nqc
     V[((size_t)(q0 + qq) * G.N1 + i1) * G.N2 + i2] = s;
 }
 
-// The apply kernels' tables from the natural table V (nq x N1 x N2):
-// val = (w_q / (N1 N2)) V; Vn natural, Vp bit-reversed on both axes, Vt
-// per column (i1 fastest).
+// The radix-2 plane kernel's table from the natural table V (nq x N1 x N2):
+// (w_q / (N1 N2)) V, bit-reversed on both axes.
 __global__ void vloc_tables_kernel(int nq, int N1, int N2, int l1, int l2, const double *V, const double *wq,
-                                   double *Vn64, float *Vn32, double *Vp64, float *Vp32, float *Vt32) {
+                                   double *Vp64, float *Vp32) {
     const int NN = N1 * N2;
     const size_t total = (size_t)nq * NN;
     const double scale = 1.0 / NN;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
         const int q = (int)(e / NN), r = (int)(e % NN), i1 = r / N2, i2 = r % N2;
         const double val = wq[q] * scale * V[e];
-        Vn64[e] = val;
-        Vn32[e] = (float)val;
         const int p1 = (int)(__brev((unsigned)i1) >> (32 - l1)), p2 = (int)(__brev((unsigned)i2) >> (32 - l2));
         const size_t pe = (size_t)q * NN + (size_t)p1 * N2 + p2;
         Vp64[pe] = val;
         Vp32[pe] = (float)val;
-        Vt32[((size_t)q * N2 + i2) * N1 + i1] = (float)val;
+    }
+}
+
+// The row-space potential U[j][d](r) = sum_q B_j(z_q) B_{j-d}(z_q) w_q V(r, z_q) / (N1 N2),
+// d = 0 .. order - 1 (0 where j - d < 0), summed over the knot intervals both
+// splines share: one thread per (row j, grid point r), which reads every
+// plane of the row's support once.  Stored in pairs of d, each residue of the
+// folded sides contiguous: [j][d / 2][residue][point].  FP64 bound (about 100
+// FMAs per element); it runs once per potential: 0.02 ms for the slab's table.
+__global__ void __launch_bounds__(256) rs_tables_kernel(int nb, int nint, int P, int N1, int N2, int s1, int s2,
+                                                        const double *V, const double *wq, const double *Bq,
+                                                        double2 *U64, float2 *U32) {
+    constexpr int K = kRsOrder;
+    const int NN = N1 * N2, M1 = N1 / s1, NP = NN / (s1 * s2);
+    const size_t total = (size_t)(nb + kRsPad) * NN;
+    const double scale = 1.0 / NN;
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+        const int j = (int)(e / NN), r = (int)(e % NN);
+        double acc[K];
+#pragma unroll
+        for (int d = 0; d < K; ++d) acc[d] = 0.0;
+        // spline j is entry m = j + 1 - t of interval t's kappa splines
+        for (int t = max(0, j + 2 - K); t <= min(nint - 1, j + 1) && j < nb; ++t) {
+            const int m = j + 1 - t;
+            for (int s = 0; s < P; ++s) {
+                const int q = t * P + s;
+                const double *b = Bq + (size_t)q * K;
+                const double v = b[m] * (wq[q] * scale * V[(size_t)q * NN + r]);
+#pragma unroll
+                for (int d = 0; d < K; ++d)
+                    if (d <= m && j - d >= 0) acc[d] = fma(b[m - d], v, acc[d]);
+            }
+        }
+        const int i1 = r / N2, i2 = r % N2;
+        const int res = (i1 % s1) * s2 + i2 % s2, pt = (i2 / s2) * M1 + i1 / s1;
+#pragma unroll
+        for (int t = 0; t < K / 2; ++t) {
+            const size_t o = ((size_t)j * (K / 2) + t) * NN + (size_t)res * NP + pt;
+            U64[o] = make_double2(acc[2 * t], acc[2 * t + 1]);
+            U32[o] = make_float2((float)acc[2 * t], (float)acc[2 * t + 1]);
+        }
     }
 }
 
@@ -195,21 +234,29 @@ size_t vloc_build_scratch_bytes(const mb_handle *h) {
            h->lstart.size() * sizeof(int) + 2 * (size_t)h->nq * sizeof(double);
 }
 
-// The natural table d_vloc -> every table of t64 / t32 the apply kernels read.
+// The natural table d_vloc -> the table of t64 / t32 the handle's plane kernel reads.
 int vloc_derive_tables(mb_handle *h) {
     const size_t NN = (size_t)h->n1 * h->n2, n = (size_t)h->nq * NN;
     int rc;
-    if ((rc = pool_alloc(h, &h->t64.Vn, n * sizeof(double)))) return rc;
-    if ((rc = pool_alloc(h, &h->t32.Vn, n * sizeof(float)))) return rc;
-    if ((rc = pool_alloc(h, &h->t64.V, n * sizeof(double)))) return rc;
-    if ((rc = pool_alloc(h, &h->t32.V, n * sizeof(float)))) return rc;
-    if ((rc = pool_alloc(h, &h->t32.Vt, n * sizeof(float)))) return rc;
+    const bool rs = rs_supported(h->n1, h->n2, h->order);
+    const size_t nu = (size_t)(h->nb + kRsPad) * kRsOrder * NN;
+    if (rs) {
+        if ((rc = pool_alloc(h, &h->t64.U, nu * sizeof(double)))) return rc;
+        if ((rc = pool_alloc(h, &h->t32.U, nu * sizeof(float)))) return rc;
+    } else {
+        if ((rc = pool_alloc(h, &h->t64.V, n * sizeof(double)))) return rc;
+        if ((rc = pool_alloc(h, &h->t32.V, n * sizeof(float)))) return rc;
+    }
     double *wq = nullptr;
     if ((rc = dev_upload(h, (void **)&wq, h->wq.data(), h->wq.size() * sizeof(double)))) return rc;
-    const int blocks = (int)std::min<size_t>((n + 255) / 256, (size_t)h->num_sms * 8);
-    vloc_tables_kernel<<<blocks, 256, 0, h->hs>>>(h->nq, h->n1, h->n2, h->l1, h->l2, h->d_vloc, wq,
-                                                 (double *)h->t64.Vn, (float *)h->t32.Vn, (double *)h->t64.V,
-                                                 (float *)h->t32.V, (float *)h->t32.Vt);
+    auto blocks = [&](size_t m) { return (int)std::min<size_t>((m + 255) / 256, (size_t)h->num_sms * 8); };
+    if (rs)
+        rs_tables_kernel<<<blocks((size_t)(h->nb + kRsPad) * NN), 256, 0, h->hs>>>(
+            h->nb, h->nint, h->nquad, h->n1, h->n2, rs_fold(h->n1), rs_fold(h->n2), h->d_vloc, wq,
+            (const double *)h->t64.Bq, (double2 *)h->t64.U, (float2 *)h->t32.U);
+    else
+        vloc_tables_kernel<<<blocks(n), 256, 0, h->hs>>>(h->nq, h->n1, h->n2, h->l1, h->l2, h->d_vloc, wq,
+                                                        (double *)h->t64.V, (float *)h->t32.V);
     cudaError_t e = cudaGetLastError();
     dev_free(h, (void **)&wq);
     if (e != cudaSuccess) return cuda_fail(h, e);
