@@ -214,6 +214,11 @@ size_t apply_H_scratch_need(const mb_handle *h, int ik, int nbands, int prec);
 int apply_H_on_scratch(mb_handle *h, int ik, const void *X, void *Y, int nbands, int prec, cudaStream_t s,
                        void *scratch);
 
+// density.cu: the electron density through row space (rs_supported handles);
+// nonneg: no occupation is negative (the result is then clamped at zero)
+int density_rows(mb_handle *h, const void *evecs, int nbands, const double *occ_dev, bool nonneg, double *rho,
+                 cudaStream_t s);
+
 enum { BAND_S = 0, BAND_SINV = 1, BAND_PREC = 2 };
 
 // eigensolver defaults: Krylov depth and roots per block of the second grand

@@ -6,7 +6,9 @@
 //                      one knot interval, inverse 2D FFT in shared memory,
 //                      f |.|^2 accumulated into the CTA's own partial table;
 //                      density_reduce_kernel sums the partials in a fixed
-//                      order (deterministic, no atomics).
+//                      order (deterministic, no atomics).  Grids of 16 to 64
+//                      points a side with order 6 take the row-space kernels
+//                      of density.cu instead.
 //  hartree_*           the electrons' Coulomb potential through the 2D
 //                      transform of 1/r (the Coulomb integral of §II.B.1):
 //                      per in-plane component g,
@@ -470,7 +472,10 @@ int check_tables(mb_handle *h) {
 
 // rho (device, nq x N1 x N2) from the eigenvectors evecs (the layout of
 // mb_eigsolve's) and the occupations occ_dev (device, nk x nbands).
-int scf_density(mb_handle *h, const void *evecs, int nbands, const double *occ_dev, double *rho, cudaStream_t s) {
+// nonneg: no occupation is negative.
+int scf_density(mb_handle *h, const void *evecs, int nbands, const double *occ_dev, bool nonneg, double *rho,
+                cudaStream_t s) {
+    if (rs_supported(h->n1, h->n2, h->order)) return density_rows(h, evecs, nbands, occ_dev, nonneg, rho, s);
     const int nk = (int)h->kp.size(), NN = h->n1 * h->n2, P = h->nquad;
     const int nmax = std::max(h->n1, h->n2);
     const int np = fft_planes(h, P);
@@ -750,7 +755,8 @@ int mb_density(mb_handle *h, const void *evecs, int nbands, const double *occ, d
     double *d_occ = B.get<double>(nocc);
     if (B.rc) return B.rc;
     MB_CUDA(cudaMemcpyAsync(d_occ, occ, sizeof(double) * nocc, cudaMemcpyHostToDevice, s));
-    if ((rc = scf_density(h, evecs, nbands, d_occ, rho, s))) return rc;
+    const bool nonneg = std::all_of(occ, occ + nocc, [](double f) { return f >= 0.0; });
+    if ((rc = scf_density(h, evecs, nbands, d_occ, nonneg, rho, s))) return rc;
     MB_CUDA(cudaStreamSynchronize(s));   // the host occupations are read by the copy above
     return MB_OK;
 }
@@ -905,7 +911,7 @@ int mb_scf(mb_handle *h, const mb_scf_opts *o, double *evals, double *rho_out, m
             // output density and the mixed next input
             mu = occupations(ev, wk, nbands, nelec, o->sigma, f);
             MB_CUDA(cudaMemcpyAsync(occ, f.data(), sizeof(double) * f.size(), cudaMemcpyHostToDevice, s));
-            if ((rc = scf_density(h, evecs, nbands, occ, rho_o, s))) {
+            if ((rc = scf_density(h, evecs, nbands, occ, true, rho_o, s))) {
                 result = rc;
                 break;
             }

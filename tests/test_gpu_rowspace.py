@@ -4,13 +4,15 @@ sides of 64 points whose disc folds onto itself, runs of one row up to the
 whole basis, steps that end inside and past the basis, and k-points with
 different discs in one batch, against the FP64 oracle.
 
-Tolerances as in test_gpu_apply.py: 1e-10 (FP64) and 2e-5 (FP32) of max |Y|."""
+Tolerances as in test_gpu_apply.py: 1e-10 (FP64) and 2e-5 (FP32) of max |Y|,
+and for the row-space density that of test_gpu_scf.py, 1e-11 of its maximum."""
 import dataclasses
 
 import numpy as np
 import pytest
 
 from oracle import hamiltonian as Hm
+from oracle import scf as F
 from paper_1406_4960_gb300 import workloads as W
 
 from gpu_util import gmap, lib_block, oracle_block, rel_err
@@ -91,3 +93,34 @@ def test_run_lengths_around_a_step(mbmod, n_int, prec):
     # enough bands that a run is the whole basis: 9 to 33 rows, which with the
     # five drain rows end below, at and above multiples of the step (8, 16)
     _check(mbmod, _workload((16, 16), (4.7, 4.7), 5.0, n_int, 100), prec)
+
+
+@pytest.mark.parametrize("case,n_int,nbands", [(c, 9, 3) for c in GRIDS] + [("16x32", 24, 40), ("64x16-fold", 14, 20)])
+def test_density(mbmod, case, n_int, nbands):
+    """The density of random bands on every grid shape, with some bands empty
+    (and a whole k-point) and, in the cells of 3 bands, one of negative weight."""
+    w = _workload(*GRIDS[case], n_int=n_int, nbands=nbands)
+    w = dataclasses.replace(w, kpts=np.array([[0.0, 0.0], [0.11, -0.07], [-0.2, 0.05]]))
+    h = mbmod.Handle.from_workload(w)
+    models, coefs, blocks = [], [], []
+    occ = np.random.default_rng(4).random((w.nk, nbands))
+    occ[1] = 0.0
+    occ[2, 1] = 0.0
+    if nbands == 3:
+        occ[0, 2] = -0.3
+    for ik in range(w.nk):
+        ng, nb, ldg = h.sizes(ik)
+        m = Hm.model_from_workload(w, ik)
+        X = W.random_block(nbands, nb, ng, seed=40 + ik)
+        models.append(m)
+        coefs.append(X)
+        blocks.append(lib_block(X, gmap(h, m, ik), ldg, np.complex128).ravel())
+    evecs = torch.from_numpy(np.concatenate(blocks)).cuda()
+    zq, _ = h.zplanes()
+    rho = torch.full((len(zq),) + w.grid, float("nan"), dtype=torch.float64, device="cuda")
+    h.density(evecs, nbands, occ, rho)
+    ref = F.density(models, coefs, occ)
+    assert np.abs(rho.cpu().numpy() - ref).max() < 1e-11 * np.abs(ref).max()
+    if nbands > 3:
+        assert float(rho.min()) >= 0.0
+    h.close()
