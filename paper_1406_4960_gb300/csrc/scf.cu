@@ -55,6 +55,7 @@ constexpr double kTwoPi = 6.283185307179586476925;
 // Perdew-Zunger (1981) parametrization of the Ceperley-Alder correlation
 // energy per electron of the unpolarized electron gas (Hartree)
 constexpr double kPzGamma = -0.1423, kPzBeta1 = 1.0529, kPzBeta2 = 0.3334;
+constexpr double kExRs = -0.45816529328314289;   // -(3/4) (9 / (4 pi^2))^(1/3)
 constexpr double kPzA = 0.0311, kPzB = -0.048, kPzC = 0.0020, kPzD = -0.0116;
 // The LDA is evaluated at max(rho, kRhoFloor) (bohr^-3): the vacuum's densities
 // of 1e-16 and below are noise of the FP64 sums and of the eigenvectors, and
@@ -209,9 +210,22 @@ __device__ __forceinline__ double2 axpy2(double a, double2 x, double2 y) {
 // combined across the lanes by shuffle scans and then re-run with the carry:
 // V_q = (2 pi/g)(L_q + R_q).  g = 0: -2 pi sum_q' a_q' |z_q - z_q'| from the
 // prefix sums of a and a z, scanned the same way.
+// Each lane keeps its chunk's a, f and (between the re-runs) L in shared
+// memory: one read of rho, all its loads in flight together, and one
+// exponential per plane (FP64 bound: about 40 FP64 instructions a plane and
+// component, 23 us on the slab's 512 x 702; 109 us when every sweep read rho
+// and evaluated the exponentials again).  With more planes than fit, `C` is
+// the chunk's length and the arrays are in the warp's part of `spill`.
+struct SweepChunk {
+    double2 *a, *L;
+    double *f;
+};
+constexpr int kSweepBytes = 2 * sizeof(double2) + sizeof(double);   // per lane and plane of a chunk
+
 __global__ void __launch_bounds__(128) hartree_sweep_kernel(const double2 *rg, double2 *vg, const double *zq,
                                                             const double *wq, int nq, int N1, int N2, double b1x,
-                                                            double b1y, double b2x, double b2y) {
+                                                            double b1y, double b2x, double b2y, unsigned char *spill) {
+    extern __shared__ __align__(16) unsigned char ssm[];
     const int NN = N1 * N2;
     const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (e >= NN) return;                         // whole warps
@@ -219,17 +233,34 @@ __global__ void __launch_bounds__(128) hartree_sweep_kernel(const double2 *rg, d
     const int m1 = u < N1 / 2 ? u : u - N1, m2 = v < N2 / 2 ? v : v - N2;
     const double gx = m1 * b1x + m2 * b2x, gy = m1 * b1y + m2 * b2y;
     const double g = sqrt(gx * gx + gy * gy);
-    const int C = (nq + 31) / 32, q0 = min(nq, lane * C), q1 = min(nq, q0 + C);
-    auto a_at = [&](int q) {
-        const double2 r = rg[(size_t)q * NN + e];
-        return make_double2(wq[q] * r.x, wq[q] * r.y);
-    };
+    const int C = (nq + 31) / 32, q0 = min(nq, lane * C), n = min(nq, q0 + C) - q0;
+    SweepChunk ch;                               // entry i of this lane at [i * 32]
+    {
+        unsigned char *base = spill ? spill + (size_t)e * C * 32 * kSweepBytes
+                                    : ssm + (size_t)(threadIdx.x >> 5) * C * 32 * kSweepBytes;
+        ch.a = reinterpret_cast<double2 *>(base) + lane;
+        ch.L = ch.a + C * 32;
+        ch.f = reinterpret_cast<double *>(base + (size_t)2 * C * 32 * sizeof(double2)) + lane;
+    }
+    for (int i0 = 0; i0 < n; i0 += 8) {
+        double2 r[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) r[i] = i0 + i < n ? rg[(size_t)(q0 + i0 + i) * NN + e] : czero<double2>();
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i0 + i < n) {
+                const int q = q0 + i0 + i;
+                const double w = wq[q];
+                ch.a[(i0 + i) * 32] = make_double2(w * r[i].x, w * r[i].y);
+                if (g != 0.0) ch.f[(i0 + i) * 32] = q > 0 ? exp(-g * (zq[q] - zq[q - 1])) : 0.0;
+            }
+    }
     if (g == 0.0) {
         double2 P = czero<double2>(), Pz = czero<double2>();
-        for (int q = q0; q < q1; ++q) {
-            const double2 a = a_at(q);
+        for (int i = 0; i < n; ++i) {
+            const double2 a = ch.a[i * 32];
             P = P + a;
-            Pz = axpy2(zq[q], a, Pz);
+            Pz = axpy2(zq[q0 + i], a, Pz);
         }
         // inclusive sums over the lanes, totals from the last lane
         for (int d = 1; d < 32; d <<= 1) {
@@ -244,27 +275,26 @@ __global__ void __launch_bounds__(128) hartree_sweep_kernel(const double2 *rg, d
         P = shfl_up2(P, 1);
         Pz = shfl_up2(Pz, 1);
         if (lane == 0) P = Pz = czero<double2>();
-        for (int q = q0; q < q1; ++q) {
-            const double2 a = a_at(q);
-            const double z = zq[q];
+        for (int i = 0; i < n; ++i) {
+            const double2 a = ch.a[i * 32];
+            const double z = zq[q0 + i];
             P = P + a;
             Pz = axpy2(z, a, Pz);
             const double re = z * P.x - Pz.x + (PzT.x - Pz.x) - z * (PT.x - P.x);
             const double im = z * P.y - Pz.y + (PzT.y - Pz.y) - z * (PT.y - P.y);
-            vg[(size_t)q * NN + e] = make_double2(-kTwoPi * re, -kTwoPi * im);
+            vg[(size_t)(q0 + i) * NN + e] = make_double2(-kTwoPi * re, -kTwoPi * im);
         }
         return;
     }
-    auto f_at = [&](int q) { return q > 0 ? exp(-g * (zq[q] - zq[q - 1])) : 0.0; };
     // this chunk's maps: forward L and backward R (same multiplier A)
     double A = 1.0;
     double2 BL = czero<double2>(), BR = czero<double2>();
-    if (q1 > q0) {
-        A = q0 > 0 ? exp(-g * (zq[q1 - 1] - zq[q0 - 1])) : 0.0;
-        for (int q = q0; q < q1; ++q) BL = axpy2(f_at(q), BL, a_at(q));
-        for (int q = q1 - 1; q >= q0; --q) {
-            const double2 a = a_at(q);
-            const double f = f_at(q);
+    if (n > 0) {
+        A = q0 > 0 ? exp(-g * (zq[q0 + n - 1] - zq[q0 - 1])) : 0.0;
+        for (int i = 0; i < n; ++i) BL = axpy2(ch.f[i * 32], BL, ch.a[i * 32]);
+        for (int i = n - 1; i >= 0; --i) {
+            const double2 a = ch.a[i * 32];
+            const double f = ch.f[i * 32];
             BR = make_double2(f * (BR.x + a.x), f * (BR.y + a.y));
         }
     }
@@ -281,9 +311,9 @@ __global__ void __launch_bounds__(128) hartree_sweep_kernel(const double2 *rg, d
     }
     double2 L = shfl_up2(IB, 1);
     if (lane == 0) L = czero<double2>();
-    for (int q = q0; q < q1; ++q) {
-        L = axpy2(f_at(q), L, a_at(q));
-        vg[(size_t)q * NN + e] = L;
+    for (int i = 0; i < n; ++i) {
+        L = axpy2(ch.f[i * 32], L, ch.a[i * 32]);
+        ch.L[i * 32] = L;
     }
     // backward: inclusive scan from lane 31 (later chunks applied first)
     double JA = A;
@@ -299,11 +329,10 @@ __global__ void __launch_bounds__(128) hartree_sweep_kernel(const double2 *rg, d
     double2 R = shfl_down2(JB, 1);
     if (lane == 31) R = czero<double2>();
     const double c = kTwoPi / g;
-    for (int q = q1 - 1; q >= q0; --q) {
-        const double2 l = vg[(size_t)q * NN + e];
-        vg[(size_t)q * NN + e] = make_double2(c * (l.x + R.x), c * (l.y + R.y));
-        const double2 a = a_at(q);
-        const double f = f_at(q);
+    for (int i = n - 1; i >= 0; --i) {
+        const double2 l = ch.L[i * 32], a = ch.a[i * 32];
+        vg[(size_t)(q0 + i) * NN + e] = make_double2(c * (l.x + R.x), c * (l.y + R.y));
+        const double f = ch.f[i * 32];
         R = make_double2(f * (R.x + a.x), f * (R.y + a.y));
     }
 }
@@ -311,8 +340,9 @@ __global__ void __launch_bounds__(128) hartree_sweep_kernel(const double2 *rg, d
 __global__ void xc_lda_kernel(const double *rho, double *vxc, double *exc, size_t n) {
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
         const double d = fmax(rho[e], kRhoFloor);
+        // e_x = -(3/4) (3 d / pi)^(1/3) = -(3/4) (9 / (4 pi^2))^(1/3) / r_s
         const double rs = cbrt(3.0 / (4.0 * 3.14159265358979323846 * d));
-        const double ex = -0.75 * cbrt(3.0 * d / 3.14159265358979323846);
+        const double ex = kExRs / rs;
         double ec, vc;
         if (rs >= 1.0) {
             const double sr = sqrt(rs), den = 1.0 + kPzBeta1 * sr + kPzBeta2 * rs;
@@ -536,7 +566,9 @@ int scf_density(mb_handle *h, const void *evecs, int nbands, const double *occ_d
 static int plane_fft2(mb_handle *h, bool inv, const double *in_r, const double2 *in_c, double *out_r, double2 *out_c,
                       double scale, cudaStream_t s) {
     const int NN = h->n1 * h->n2, nmax = std::max(h->n1, h->n2);
-    const int np = fft_planes(h, 8);
+    // few enough planes per CTA that the CTAs fill the SMs twice (8 planes:
+    // 88 CTAs and 62 us on the slab's 702 planes)
+    const int np = fft_planes(h, std::max(1, std::min(8, h->nq / (2 * h->num_sms))));
     const size_t smem = (size_t)(nmax / 2 + (size_t)np * NN) * sizeof(double2);
     const int grid = (h->nq + np - 1) / np;
     const double2 *tw = reinterpret_cast<const double2 *>(h->t64.tw);
@@ -559,9 +591,18 @@ struct ScfPlanes {
 };
 
 static int hartree_g(mb_handle *h, const double2 *rg, double2 *vg, const ScfPlanes &pl, cudaStream_t s) {
-    const int NN = h->n1 * h->n2;
-    hartree_sweep_kernel<<<(NN + 3) / 4, 128, 0, s>>>(rg, vg, pl.zq, pl.wq, h->nq, h->n1, h->n2, h->b1[0],
-                                                       h->b1[1], h->b2[0], h->b2[1]);
+    const int NN = h->n1 * h->n2, C = (h->nq + 31) / 32;
+    size_t smem = (size_t)4 * 32 * C * kSweepBytes;
+    Buf B{h, s};
+    unsigned char *spill = nullptr;
+    if (smem > (size_t)h->smem_optin) {          // beyond about 1400 planes
+        spill = B.get<unsigned char>((size_t)NN * 32 * C * kSweepBytes);
+        if (B.rc) return B.rc;
+        smem = 0;
+    }
+    MB_CUDA(smem_limit_once((const void *)hartree_sweep_kernel, h->device, h->smem_optin));
+    hartree_sweep_kernel<<<(NN + 3) / 4, 128, smem, s>>>(rg, vg, pl.zq, pl.wq, h->nq, h->n1, h->n2, h->b1[0],
+                                                          h->b1[1], h->b2[0], h->b2[1], spill);
     MB_CUDA(cudaGetLastError());
     ++h->launches;
     return MB_OK;
