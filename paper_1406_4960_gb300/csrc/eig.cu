@@ -192,10 +192,13 @@ __global__ void residual_kernel(const EigK *ks, int M, int oX, int oHX, int oSX,
     (void)oX;
 }
 
-// out[prob*m + i] = Re <A_i, B_i>   (block reduction with warp shuffles)
+// Re <A_i, B_i> over one of gridDim.z chunks of the vector into part[(prob m + i)
+// chunks + chunk] (block reduction with warp shuffles); coldot_sum_kernel adds
+// the chunks in order.  Bound by the read of the vectors: one CTA a vector
+// (73 us for 90 vectors of 115 k elements) left half the SMs idle.
 // F32: on the FP32 copies, per-thread sums in FP32 and the rest in FP64
 template <bool F32>
-__global__ void coldot_kernel(const EigK *ks, int nch, VSet A, VSet B, double *out) {
+__global__ void coldot_kernel(const EigK *ks, int nch, VSet A, VSet B, double *part) {
     typedef typename std::conditional<F32, float2, double2>::type T2;
     typedef typename std::conditional<F32, float, double>::type T;
     const int i = blockIdx.x, prob = blockIdx.y;
@@ -204,8 +207,10 @@ __global__ void coldot_kernel(const EigK *ks, int nch, VSet A, VSet B, double *o
     const T2 *vb = F32 ? reinterpret_cast<const T2 *>(d.v32) : reinterpret_cast<const T2 *>(d.base);
     const T2 *a = vb + (long long)A.at(i, ch) * d.nvec;
     const T2 *b = vb + (long long)B.at(i, ch) * d.nvec;
+    const long long t0 = blockIdx.z * d.nvec / gridDim.z, t1 = (blockIdx.z + 1) * d.nvec / gridDim.z;
     T st = T(0);
-    for (long long t = threadIdx.x; t < d.nvec; t += blockDim.x) st = fma(a[t].x, b[t].x, fma(a[t].y, b[t].y, st));
+#pragma unroll 4
+    for (long long t = t0 + threadIdx.x; t < t1; t += blockDim.x) st = fma(a[t].x, b[t].x, fma(a[t].y, b[t].y, st));
     double s = (double)st;
     for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
     __shared__ double ws[32];
@@ -214,8 +219,15 @@ __global__ void coldot_kernel(const EigK *ks, int nch, VSet A, VSet B, double *o
     if (threadIdx.x < 32) {
         s = threadIdx.x < (blockDim.x >> 5) ? ws[threadIdx.x] : 0.0;
         for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-        if (threadIdx.x == 0) out[(size_t)prob * A.count() + i] = s;
+        if (threadIdx.x == 0) part[((size_t)prob * A.count() + i) * gridDim.z + blockIdx.z] = s;
     }
+}
+__global__ void coldot_sum_kernel(const double *part, int chunks, int n, double *out) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    double s = 0.0;
+    for (int c = 0; c < chunks; ++c) s += part[(size_t)e * chunks + c];
+    out[e] = s;
 }
 
 // new Krylov vector: K = W / ||W||_S, SK = SW / ||W||_S, HK slot cleared;
@@ -648,66 +660,91 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_mixed_kernel(const doub
     }
 }
 
-// U = L^{-H} with G = L L^H (G Hermitian positive definite, m <= JMAX).
-// L lives in shared memory; U is written row by row to global memory.
+// U = L^{-H} with G = L L^H (G Hermitian positive definite, m <= JMAX), one
+// CTA per problem, the matrix in shared memory throughout: right-looking
+// Cholesky (a warp per row of the trailing update), then the lower triangle
+// inverted in place row by row (row i of L^{-1} needs row i of L and the rows
+// above it: kCholSplit threads per column share the sum).  Latency bound, two
+// barriers a column: m = 90 in FP32 took 0.66 ms with one thread per column
+// of the inverse reading it back from global memory; now 0.10 ms.
 // T = float: the arithmetic in FP32 (the bulk cycles' S-Grams, which are the
 // identity up to the FP32 Gram-Schmidt error).
+constexpr int kCholThreads = 512, kCholSplit = 4;
+template <typename T> constexpr size_t cholinv_smem(int m) {
+    return ((size_t)m * (m + 1) + m + (size_t)kCholSplit * JMAX) * 2 * sizeof(T);
+}
 template <typename T>
-__global__ void __launch_bounds__(128) cholinv_kernel(const double2 *G, int m, double2 *U, int *status) {
+__global__ void __launch_bounds__(kCholThreads) cholinv_kernel(const double2 *G, int m, double2 *U, int *status) {
     typedef typename std::conditional<std::is_same<T, float>::value, float2, double2>::type T2;
     extern __shared__ __align__(16) unsigned char sm[];
-    T2 *L = reinterpret_cast<T2 *>(sm);     // m x m, lower
-    T *rdiag = reinterpret_cast<T *>(L + m * m);
-    const int prob = blockIdx.x;
+    const int ld = m + 1;                   // rows padded by one: columns are free of bank conflicts
+    T2 *L = reinterpret_cast<T2 *>(sm);     // m x ld, lower
+    T2 *row = L + m * ld;                   // m
+    T2 *red = row + m;                      // kCholSplit x JMAX
+    __shared__ T rpiv;
+    const int prob = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const double2 *g = G + (size_t)prob * LD * LD;
     double2 *u = U + (size_t)prob * LD * LD;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        int i = e / m, j = e % m;
-        const double2 v = i >= j ? g[i * LD + j] : make_double2(0.0, 0.0);
-        L[e] = mk((T)v.x, (T)v.y);
-    }
+    for (int i = warp; i < m; i += kCholThreads / 32)
+        for (int j = lane; j <= i; j += 32) {
+            const double2 v = g[i * LD + j];
+            L[i * ld + j] = mk((T)v.x, (T)v.y);
+        }
     __syncthreads();
-    __shared__ T rpiv;
     for (int j = 0; j < m; ++j) {
-        if (threadIdx.x == 0) {
-            T d = L[j * m + j].x;
+        if (tid == 0) {
+            T d = L[j * ld + j].x;
             if (!(d > T(0))) {
                 status[prob] = 1;
                 d = std::is_same<T, float>::value ? T(1e-30) : T(1e-300);
             }
             const T piv = sqrt(d);
             rpiv = T(1) / piv;
-            L[j * m + j] = mk(piv, T(0));
+            L[j * ld + j] = mk(piv, T(0));
         }
         __syncthreads();
         const T r = rpiv;
-        for (int i = j + 1 + threadIdx.x; i < m; i += blockDim.x) L[i * m + j] = rscale(r, L[i * m + j]);
+        // column j scaled into `row`, then the trailing update L[i][c] -= l_i conj(l_c), j < c <= i
+        for (int i = j + 1 + tid; i < m; i += kCholThreads) {
+            const T2 v = rscale(r, L[i * ld + j]);
+            L[i * ld + j] = v;
+            row[i] = v;
+        }
         __syncthreads();
-        // trailing update: L[i][c] -= L[i][j] conj(L[c][j]) for j < c <= i
-        for (int e = threadIdx.x; e < (m - j - 1) * (m - j - 1); e += blockDim.x) {
-            int i = j + 1 + e / (m - j - 1), c = j + 1 + e % (m - j - 1);
-            if (c > i) continue;
-            T2 lij = L[i * m + j], lcj = L[c * m + j];
-            L[i * m + c] = L[i * m + c] - cmul_c(lij, lcj);
+        for (int i = j + 1 + warp; i < m; i += kCholThreads / 32) {
+            const T2 li = row[i];
+            for (int c = j + 1 + lane; c <= i; c += 32) L[i * ld + c] = L[i * ld + c] - cmul_c(li, row[c]);
         }
         __syncthreads();
     }
-    for (int i = threadIdx.x; i < m; i += blockDim.x) rdiag[i] = T(1) / L[i * m + i].x;
-    __syncthreads();
-    // column c of Z = L^{-1} by forward substitution (one thread per column);
-    // U[c][i] = conj(Z[i][c]), and Z[q][c] is read back as conj(U[c][q])
-    for (int c = threadIdx.x; c < m; c += blockDim.x) {
-        for (int i = 0; i < c; ++i) u[c * LD + i] = make_double2(0.0, 0.0);
-        for (int i = c; i < m; ++i) {
-            T2 acc = mk(T(i == c ? 1 : 0), T(0));
-            for (int q = c; q < i; ++q) {
-                const double2 uq = u[c * LD + q];
-                acc = acc - cmul(L[i * m + q], mk((T)uq.x, (T)-uq.y));
-            }
-            const T2 z = rscale(rdiag[i], acc);
+    // row i of Z = L^{-1}: Z[i][c] = -(1 / L_ii) sum_{c <= q < i} L[i][q] Z[q][c]
+    const int part = tid / (kCholThreads / kCholSplit), c0 = tid % (kCholThreads / kCholSplit);
+    static_assert(kCholThreads / kCholSplit >= JMAX, "a thread per column and part");
+    for (int i = 0; i < m; ++i) {
+        const T r = T(1) / L[i * ld + i].x;
+        if (c0 < i) {
+            T2 s = mk(T(0), T(0));
+            // an equal share of the column's terms for every part
+            const int n = i - c0, q1 = c0 + (part + 1) * n / kCholSplit;
+            for (int q = c0 + part * n / kCholSplit; q < q1; ++q) cfma(s, L[i * ld + q], L[q * ld + c0]);
+            red[part * JMAX + c0] = s;
+        }
+        __syncthreads();
+        if (tid < i) {
+            T2 s = red[tid];
+#pragma unroll
+            for (int p = 1; p < kCholSplit; ++p) s = s + red[p * JMAX + tid];
+            L[i * ld + tid] = rscale(-r, s);
+        } else if (tid == i) {
+            L[i * ld + i] = mk(r, T(0));
+        }
+        __syncthreads();
+    }
+    for (int c = warp; c < m; c += kCholThreads / 32)
+        for (int i = lane; i < m; i += 32) {
+            const T2 z = i >= c ? L[i * ld + c] : mk(T(0), T(0));
             u[c * LD + i] = make_double2((double)z.x, (double)-z.y);
         }
-    }
 }
 
 // Maximum-overlap selection of bsz Ritz pairs in a block (+ new roots).
@@ -1717,13 +1754,11 @@ struct Solver {
     // U = L^{-H} of np problems (FP32 arithmetic in the bulk cycles)
     void cholinv(int np, int m, const double2 *G, double2 *U, int *status, bool f32) {
         if (f32) {
-            const size_t smem = (size_t)m * m * sizeof(float2) + m * sizeof(float);
             cuda(smem_limit_once((const void *)cholinv_kernel<float>, h->device, h->smem_optin));
-            MB_LAUNCH_E(KN_SMALL, cholinv_kernel<float><<<np, 128, smem, s>>>(G, m, U, status));
+            MB_LAUNCH_E(KN_SMALL, cholinv_kernel<float><<<np, kCholThreads, cholinv_smem<float>(m), s>>>(G, m, U, status));
         } else {
-            const size_t smem = (size_t)m * m * sizeof(double2) + m * sizeof(double);
             cuda(smem_limit_once((const void *)cholinv_kernel<double>, h->device, h->smem_optin));
-            MB_LAUNCH_E(KN_SMALL, cholinv_kernel<double><<<np, 128, smem, s>>>(G, m, U, status));
+            MB_LAUNCH_E(KN_SMALL, cholinv_kernel<double><<<np, kCholThreads, cholinv_smem<double>(m), s>>>(G, m, U, status));
         }
     }
     void small_gemm(const double2 *A, const double2 *B, double2 *C, int m, int conjA, int np = 0) {
@@ -1757,9 +1792,15 @@ struct Solver {
         if (r && rc == MB_OK) rc = r;
     }
     void coldot(int nch, VSet A, VSet B, double *out, bool f32 = false) {
-        const dim3 grid(A.count(), nk * nch);
-        if (f32) MB_LAUNCH_E(KN_SMALL, coldot_kernel<true><<<grid, 256, 0, s>>>(d_k, nch, A, B, out));
-        else MB_LAUNCH_E(KN_SMALL, coldot_kernel<false><<<grid, 256, 0, s>>>(d_k, nch, A, B, out));
+        // chunks of at least 2048 elements, until there are about four CTAs per SM
+        const int n = A.count() * nk * nch;
+        const int chunks = (int)std::max<long long>(1, std::min<long long>((4 * h->num_sms + n - 1) / n, nmax / 2048));
+        double *part = chunks > 1 ? reinterpret_cast<double *>(d_part) : out;
+        const dim3 grid(A.count(), nk * nch, chunks);
+        if (f32) MB_LAUNCH_E(KN_SMALL, coldot_kernel<true><<<grid, 256, 0, s>>>(d_k, nch, A, B, part));
+        else MB_LAUNCH_E(KN_SMALL, coldot_kernel<false><<<grid, 256, 0, s>>>(d_k, nch, A, B, part));
+        if (chunks > 1)
+            MB_LAUNCH_E(KN_SMALL, coldot_sum_kernel<<<(n + 127) / 128, 128, 0, s>>>(part, chunks, n, out));
     }
     // Y = H X on the FP32 copies (bulk cycles): nv vectors from src32 to dst32
     void apply32(int src32, int dst32, int nv) {
