@@ -1355,47 +1355,128 @@ __global__ void __launch_bounds__(256) combine_ff_kernel(const EigK *ks, int nch
     }
 }
 
-// C_j = beta C_j + alpha sum_i A_i Y[i][j]: one element t per thread, JC
-// output columns at a time with their coefficients staged in shared memory.
-template <int JC, bool F32>
-__global__ void __launch_bounds__(256) combine2_kernel(const EigK *ks, int nch, VSet A, VSet C,
-                                                       const double2 *Y, double alpha, double beta) {
+// C_j = beta C_j + alpha sum_i A_i Y[i][j]: TE elements per thread (blockDim.x
+// apart) and JC output columns per CTA (blockIdx.z: the column group), their
+// coefficients staged in shared memory and read two columns at a time, so that
+// a pair of 16-byte loads serves 4 TE complex products.  FP32 (F32): bound by
+// the FMA pipe for many columns; FP64: by the FP64 pipe, so small problems
+// take narrow groups to reach every SM.
+constexpr int kCombThreads = 128;
+template <int JC, int TE, bool F32>
+__global__ void __launch_bounds__(kCombThreads) combine2_kernel(const EigK *ks, int nch, VSet A, VSet C,
+                                                                const double2 *Y, double alpha, double beta) {
     typedef typename std::conditional<F32, float2, double2>::type T2;
     typedef typename std::conditional<F32, float, double>::type T;
-    __shared__ T2 Ys[JMAX][JC];
+    __shared__ __align__(16) T2 Ys[JMAX][JC];
+    const int prob = blockIdx.y, j0 = blockIdx.z * JC;
+    const int k = prob / nch, ch = prob % nch;
+    const EigK d = ks[k];
+    const long long t0 = (long long)blockIdx.x * (kCombThreads * TE) + threadIdx.x;
+    if (t0 - threadIdx.x >= d.nvec) return;               // the batch's longest vectors size the grid
+    const int ma = A.count(), mc = C.count();
+    const double2 *y = Y + (size_t)prob * LD * LD;
+    for (int e = threadIdx.x; e < ma * JC; e += kCombThreads) {
+        const int i = e / JC, jj = e % JC;
+        const double2 yv = j0 + jj < mc ? y[i * LD + j0 + jj] : make_double2(0.0, 0.0);
+        Ys[i][jj] = mk((T)yv.x, (T)yv.y);
+    }
+    __syncthreads();
+    T2 *vb = F32 ? reinterpret_cast<T2 *>(d.v32) : reinterpret_cast<T2 *>(d.base);
+    T2 acc[TE][JC];
+#pragma unroll
+    for (int u = 0; u < TE; ++u)
+#pragma unroll
+        for (int jj = 0; jj < JC; ++jj) acc[u][jj] = czero<T2>();
+    auto step = [&](int i, const T2(&av)[TE]) {
+#pragma unroll
+        for (int jj = 0; jj < JC; jj += 2) {
+            T2 w0, w1;
+            if constexpr (F32) {
+                const float4 w = *reinterpret_cast<const float4 *>(&Ys[i][jj]);
+                w0 = make_float2(w.x, w.y);
+                w1 = make_float2(w.z, w.w);
+            } else {
+                w0 = Ys[i][jj];
+                w1 = Ys[i][jj + 1];
+            }
+#pragma unroll
+            for (int u = 0; u < TE; ++u) {
+                cfma(acc[u][jj], av[u], w0);
+                cfma(acc[u][jj + 1], av[u], w1);
+            }
+        }
+    };
+    auto load = [&](int i, T2(&av)[TE]) {
+        const T2 *v = vb + (long long)A.at(i, ch) * d.nvec + t0;
+#pragma unroll
+        for (int u = 0; u < TE; ++u) av[u] = t0 + u * kCombThreads < d.nvec ? v[u * kCombThreads] : czero<T2>();
+    };
+    constexpr int PF = 4;                                 // vectors in flight
+    for (int i = 0; i < ma; i += PF) {
+        T2 av[PF][TE];
+#pragma unroll
+        for (int p = 0; p < PF; ++p)
+            if (i + p < ma) load(i + p, av[p]);
+#pragma unroll
+        for (int p = 0; p < PF; ++p)
+            if (i + p < ma) step(i + p, av[p]);
+    }
+#pragma unroll
+    for (int jj = 0; jj < JC; ++jj) {
+        if (j0 + jj >= mc) break;
+        T2 *c = vb + (long long)C.at(j0 + jj, ch) * d.nvec + t0;
+#pragma unroll
+        for (int u = 0; u < TE; ++u) {
+            if (t0 + u * kCombThreads >= d.nvec) break;
+            const T2 v = rscale((T)alpha, acc[u][jj]);
+            c[u * kCombThreads] = beta == 0.0 ? v : rscale((T)beta, c[u * kCombThreads]) + v;
+        }
+    }
+}
+
+// The same for one output column (a chain's Gram-Schmidt update): 16 bytes
+// of every vector per thread, eight vectors in flight.  Bound by the read of
+// the vectors.
+template <bool F32>
+__global__ void __launch_bounds__(kCombThreads) combine1_kernel(const EigK *ks, int nch, VSet A, VSet C,
+                                                                const double2 *Y, double alpha, double beta) {
+    typedef typename std::conditional<F32, float2, double2>::type T2;
+    typedef typename std::conditional<F32, float, double>::type T;
+    constexpr int VE = F32 ? 2 : 1;                       // elements per thread (nvec is a multiple of 32)
+    __shared__ T2 Ys[JMAX];
     const int prob = blockIdx.y;
     const int k = prob / nch, ch = prob % nch;
     const EigK d = ks[k];
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = t < d.nvec;
-    const int ma = A.count(), mc = C.count();
+    const long long t = ((long long)blockIdx.x * kCombThreads + threadIdx.x) * VE;
+    const int ma = A.count();
     const double2 *y = Y + (size_t)prob * LD * LD;
-    for (int j0 = 0; j0 < mc; j0 += JC) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < ma * JC; e += blockDim.x) {
-            const int i = e / JC, jj = e % JC;
-            const double2 yv = j0 + jj < mc ? y[i * LD + j0 + jj] : make_double2(0.0, 0.0);
-            Ys[i][jj] = mk((T)yv.x, (T)yv.y);
-        }
-        __syncthreads();
-        if (!live) continue;
-        T2 *vb = F32 ? reinterpret_cast<T2 *>(d.v32) : reinterpret_cast<T2 *>(d.base);
-        T2 acc[JC];
+    for (int i = threadIdx.x; i < ma; i += kCombThreads) Ys[i] = mk((T)(alpha * y[i * LD].x), (T)(alpha * y[i * LD].y));
+    __syncthreads();
+    if (t >= d.nvec) return;
+    T2 *vb = F32 ? reinterpret_cast<T2 *>(d.v32) : reinterpret_cast<T2 *>(d.base);
+    struct __align__(16) Pack { T2 v[VE]; };
+    Pack *c = reinterpret_cast<Pack *>(vb + (long long)C.at(0, ch) * d.nvec + t);
+    Pack acc;
+    if (beta == 0.0) {
 #pragma unroll
-        for (int jj = 0; jj < JC; ++jj) acc[jj] = czero<T2>();
-        for (int i = 0; i < ma; ++i) {
-            const T2 a = vb[(long long)A.at(i, ch) * d.nvec + t];
+        for (int u = 0; u < VE; ++u) acc.v[u] = czero<T2>();
+    } else {
+        acc = *c;
 #pragma unroll
-            for (int jj = 0; jj < JC; ++jj) cfma(acc[jj], a, Ys[i][jj]);
-        }
-#pragma unroll
-        for (int jj = 0; jj < JC; ++jj) {
-            if (j0 + jj >= mc) break;
-            T2 *c = vb + (long long)C.at(j0 + jj, ch) * d.nvec + t;
-            const T2 v = rscale((T)alpha, acc[jj]);
-            *c = beta == 0.0 ? v : rscale((T)beta, *c) + v;
-        }
+        for (int u = 0; u < VE; ++u) acc.v[u] = rscale((T)beta, acc.v[u]);
     }
+    for (int i0 = 0; i0 < ma; i0 += 8) {
+        Pack a[8];
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+            if (i0 + p < ma) a[p] = *reinterpret_cast<const Pack *>(vb + (long long)A.at(i0 + p, ch) * d.nvec + t);
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+            if (i0 + p < ma)
+#pragma unroll
+                for (int u = 0; u < VE; ++u) cfma(acc.v[u], a[p].v[u], Ys[i0 + p]);
+    }
+    *c = acc;
 }
 
 // [X|K]^H H [X|K] (and the S counterpart) when X holds Ritz vectors of the
@@ -1735,21 +1816,35 @@ struct Solver {
             combine_t<false>(nch, A, C, Y, alpha, beta);
         }
     }
+    template <int JC, int TE, bool F32> void combine_j(int nch, VSet A, VSet C, const double2 *Y, double alpha, double beta) {
+        const dim3 grid((unsigned)((nmax + kCombThreads * TE - 1) / (kCombThreads * TE)), nk * nch, (C.count() + JC - 1) / JC);
+        MB_LAUNCH_E(F32 ? KN_COMBINE32 : KN_COMBINE,
+                    (combine2_kernel<JC, TE, F32><<<grid, kCombThreads, 0, s>>>(d_k, nch, A, C, Y, alpha, beta)));
+    }
     template <bool F32> void combine_t(int nch, VSet A, VSet C, const double2 *Y, double alpha, double beta) {
-        const dim3 grid((unsigned)((nmax + 255) / 256), nk * nch);
         const int mc = C.count();
-        // column width with the least padding (12 divides the common 36)
+        if (mc == 1) {
+            const int per = kCombThreads * (F32 ? 2 : 1);
+            MB_LAUNCH_E(F32 ? KN_COMBINE32 : KN_COMBINE,
+                        (combine1_kernel<F32><<<dim3((unsigned)((nmax + per - 1) / per), nk * nch), kCombThreads, 0, s>>>(
+                            d_k, nch, A, C, Y, alpha, beta)));
+            return;
+        }
+        // the widest column group (least re-reading of A) among those with the
+        // least padding, narrow ones where wide ones would leave SMs idle
+        const long long ctas = (nmax + kCombThreads - 1) / kCombThreads * nk * nch;
         auto waste = [&](int jc) { return (mc + jc - 1) / jc * jc - mc; };
-        if (mc == 1)
-            MB_LAUNCH_E(F32 ? KN_COMBINE32 : KN_COMBINE, (combine2_kernel<1, F32><<<grid, 256, 0, s>>>(d_k, nch, A, C, Y, alpha, beta)));
-        else if (mc <= 4)
-            MB_LAUNCH_E(F32 ? KN_COMBINE32 : KN_COMBINE, (combine2_kernel<4, F32><<<grid, 256, 0, s>>>(d_k, nch, A, C, Y, alpha, beta)));
-        else if (mc <= 8)
-            MB_LAUNCH_E(F32 ? KN_COMBINE32 : KN_COMBINE, (combine2_kernel<8, F32><<<grid, 256, 0, s>>>(d_k, nch, A, C, Y, alpha, beta)));
-        else if (waste(12) < waste(16))
-            MB_LAUNCH_E(F32 ? KN_COMBINE32 : KN_COMBINE, (combine2_kernel<12, F32><<<grid, 256, 0, s>>>(d_k, nch, A, C, Y, alpha, beta)));
-        else
-            MB_LAUNCH_E(F32 ? KN_COMBINE32 : KN_COMBINE, (combine2_kernel<16, F32><<<grid, 256, 0, s>>>(d_k, nch, A, C, Y, alpha, beta)));
+        if (mc <= 2 || (!F32 && ctas * ((mc + 11) / 12) < 2 * h->num_sms)) {
+            combine_j<2, 1, F32>(nch, A, C, Y, alpha, beta);
+        } else if (mc <= 4 || ctas * ((mc + 11) / 12) < 2 * h->num_sms) {
+            combine_j<4, 1, F32>(nch, A, C, Y, alpha, beta);
+        } else if (mc <= 8) {
+            combine_j<8, 1, F32>(nch, A, C, Y, alpha, beta);
+        } else if (waste(10) < waste(12)) {
+            combine_j<10, F32 ? 2 : 1, F32>(nch, A, C, Y, alpha, beta);
+        } else {
+            combine_j<12, F32 ? 2 : 1, F32>(nch, A, C, Y, alpha, beta);
+        }
     }
     // U = L^{-H} of np problems (FP32 arithmetic in the bulk cycles)
     void cholinv(int np, int m, const double2 *G, double2 *U, int *status, bool f32) {
