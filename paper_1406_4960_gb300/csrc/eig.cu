@@ -804,92 +804,129 @@ __global__ void take_evals_kernel(const double *evals, int M, int nk, double *ep
     if (e < M * nk) eps[e] = evals[(size_t)(e / M) * LD + (e % M)];
 }
 
-// banded solves on vector ranges of every k-point (FP64)
-// L L^T y = x, one thread per (vector, G) column; the last K-1 solution values
-// ride in registers.  per_g: the k-point's factors L_G[j][d] stored as
-// pfac[(j*K + d)*ldg + G] (coalesced over G); else the G-independent L_z.
-// F32: on the FP32 Gram-Schmidt copies with FP32 factors (a preconditioner
-// solve, whose rounding only changes which Krylov space is built).
-template <int K, bool F32>
-__global__ void eig_banded_solve_kernel(const EigK *ks, const void *Lbv, int per_g, int nb, int src, int dst,
-                                        int nv) {
+// Banded solves on vector ranges of every k-point: L L^T y = x, one thread per
+// G column and NV vectors; the last K-1 solution values ride in registers.
+// per_g: the k-point's factors L_G[j][d] stored as pfac[(j*K + d)*ldg + G]
+// (coalesced over G); else the G-independent L_z.  F32: on the FP32
+// Gram-Schmidt copies with FP32 factors (a preconditioner solve, whose
+// rounding only changes which Krylov space is built).
+// Rows go in tiles of PD: while a tile's recurrence runs, the next tile's
+// right-hand sides and factors (none of which depends on it) are in flight,
+// and NV vectors share every factor: with one vector per thread the factors
+// were 7 of 9 bytes read, from L2, and each tile waited for its own loads.
+template <int K, bool F32, int NV>
+__global__ void __launch_bounds__(64) eig_banded_solve_kernel(const EigK *ks, const void *Lbv, int per_g, int nb, int src,
+                                                              int dst, int nv) {
     typedef typename std::conditional<F32, float2, double2>::type T2;
     typedef typename std::conditional<F32, float, double>::type T;
-    const int k = blockIdx.z / nv, v = blockIdx.z % nv;
+    const int nvt = (nv + NV - 1) / NV;
+    const int k = blockIdx.z / nvt, v0 = blockIdx.z % nvt * NV, nvl = min(NV, nv - v0);
     const EigK d = ks[k];
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= d.ldg) return;
     T2 *vb = F32 ? reinterpret_cast<T2 *>(d.v32) : reinterpret_cast<T2 *>(d.base);
     const T *Lb = reinterpret_cast<const T *>(Lbv);
     const T *pf = F32 ? reinterpret_cast<const T *>(d.pfac32) : reinterpret_cast<const T *>(d.pfac);
-    const T2 *x = vb + (long long)(src + v) * d.nvec;
-    T2 *y = vb + (long long)(dst + v) * d.nvec;
-    const size_t ldg = d.ldg;
+    const int ldg = d.ldg;
+    // vector v of the thread (past the last one: the last one again, not written)
+    const T2 *xv[NV];
+    T2 *yv[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        xv[v] = vb + (long long)(src + v0 + min(v, nvl - 1)) * d.nvec + g;
+        yv[v] = vb + (long long)(dst + v0 + min(v, nvl - 1)) * d.nvec + g;
+    }
     if (g >= d.ng) {
-        for (int j = 0; j < nb; ++j) y[(size_t)j * ldg + g] = czero<T2>();
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+            for (int j = 0; j < nb; ++j) yv[v][j * ldg] = czero<T2>();
         return;
     }
-    // factors hold L[j][j-d] for d >= 1 and 1 / L[j][j] at d = 0
-    auto L = [&](int j, int dd) -> T {
-        return per_g ? pf[((size_t)j * K + dd) * ldg + g] : __ldg(&Lb[(size_t)j * K + dd]);
+    // factors hold L[j][j-d] for d >= 1 (0 where j < d) and 1 / L[j][j] at
+    // d = 0; fd: entry (j, d) is fp[j * fr + d * fd]
+    const T *fp = per_g ? pf + g : Lb;
+    const int fd = per_g ? ldg : 1, fr = K * fd;
+    constexpr int PD = F32 ? 4 : 2;
+    struct Tile {
+        T2 x[NV][PD];
+        T f[PD][K];
     };
-    // rows are handled in tiles of PD: every load of a tile (right-hand
-    // sides and factors, none of which depends on the recurrence) is issued
-    // before the tile's recurrence runs
-    constexpr int PD = F32 ? 8 : 4;
-    T2 win[K];
+    T2 win[NV][K];                                  // win[v][i]: solution i + 1 rows back
+    auto clear = [&]() {
 #pragma unroll
-    for (int i = 0; i < K; ++i) win[i] = czero<T2>();
-    for (int j0 = 0; j0 < nb; j0 += PD) {
-        T2 xs[PD];
-        T fs[PD][K];
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+            for (int i = 0; i < K; ++i) win[v][i] = czero<T2>();
+    };
+    // one row: s - sum_d f_d win_d, the newest solution last (only its FMA waits for the previous row)
+    auto solve = [&](int v, T2 s, const T(&f)[K]) {
+#pragma unroll
+        for (int dd = K - 1; dd >= 1; --dd) rfma(s, -f[dd], win[v][dd - 1]);
+        s = rscale(f[0], s);
+#pragma unroll
+        for (int i = K - 1; i > 0; --i) win[v][i] = win[v][i - 1];
+        win[v][0] = s;
+        return s;
+    };
+    auto load_f = [&](Tile &t, int j0) {
 #pragma unroll
         for (int u = 0; u < PD; ++u) {
-            const int j = j0 + u;
-            xs[u] = j < nb ? x[(size_t)j * ldg + g] : czero<T2>();
+            const int j = min(j0 + u, nb - 1), o = j * fr;
 #pragma unroll
-            for (int dd = 0; dd < K; ++dd) fs[u][dd] = (j < nb && j - dd >= 0) ? L(j, dd) : T(0);
+            for (int dd = 0; dd < K; ++dd) t.f[u][dd] = fp[o + dd * fd];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) t.x[v][u] = xv[v][j * ldg];
         }
+    };
+    auto load_b = [&](Tile &t, int j1) {
 #pragma unroll
         for (int u = 0; u < PD; ++u) {
-            const int j = j0 + u;
-            if (j >= nb) break;
-            T2 s = xs[u];
+            // (past the last row the solutions are still zero: any finite factor will do)
+            const int j = max(j1 - u, 0), o = j * fr;
 #pragma unroll
-            for (int dd = 1; dd < K; ++dd) rfma(s, -fs[u][dd], win[dd - 1]);
-            const T2 yj = rscale(fs[u][0], s);
-            y[(size_t)j * ldg + g] = yj;
+            for (int dd = 0; dd < K; ++dd) t.f[u][dd] = fp[j + dd < nb ? o + dd * (fr + fd) : o];
 #pragma unroll
-            for (int i = K - 1; i > 0; --i) win[i] = win[i - 1];
-            win[0] = yj;
+            for (int v = 0; v < NV; ++v) t.x[v][u] = yv[v][j * ldg];
         }
+    };
+    auto run_f = [&](const Tile &t, int j0) {
+#pragma unroll
+        for (int u = 0; u < PD; ++u) {
+            if (j0 + u >= nb) break;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                const T2 r = solve(v, t.x[v][u], t.f[u]);
+                if (NV == 1 || v < nvl) yv[v][(j0 + u) * ldg] = r;
+            }
+        }
+    };
+    auto run_b = [&](const Tile &t, int j1) {
+#pragma unroll
+        for (int u = 0; u < PD; ++u) {
+            if (j1 - u < 0) break;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                const T2 r = solve(v, t.x[v][u], t.f[u]);
+                if (NV == 1 || v < nvl) yv[v][(j1 - u) * ldg] = r;
+            }
+        }
+    };
+    Tile ta, tb;
+    clear();
+    load_f(ta, 0);
+    for (int j0 = 0; j0 < nb; j0 += 2 * PD) {
+        if (j0 + PD < nb) load_f(tb, j0 + PD);
+        run_f(ta, j0);
+        if (j0 + 2 * PD < nb) load_f(ta, j0 + 2 * PD);
+        if (j0 + PD < nb) run_f(tb, j0 + PD);
     }
-#pragma unroll
-    for (int i = 0; i < K; ++i) win[i] = czero<T2>();
-    for (int j1 = nb - 1; j1 >= 0; j1 -= PD) {
-        T2 xs[PD];
-        T fs[PD][K];
-#pragma unroll
-        for (int u = 0; u < PD; ++u) {
-            const int j = j1 - u;
-            xs[u] = j >= 0 ? y[(size_t)j * ldg + g] : czero<T2>();
-            fs[u][0] = j >= 0 ? L(j, 0) : T(0);
-#pragma unroll
-            for (int dd = 1; dd < K; ++dd) fs[u][dd] = (j >= 0 && j + dd < nb) ? L(j + dd, dd) : T(0);
-        }
-#pragma unroll
-        for (int u = 0; u < PD; ++u) {
-            const int j = j1 - u;
-            if (j < 0) break;
-            T2 s = xs[u];
-#pragma unroll
-            for (int dd = 1; dd < K; ++dd) rfma(s, -fs[u][dd], win[dd - 1]);
-            const T2 zj = rscale(fs[u][0], s);
-            y[(size_t)j * ldg + g] = zj;
-#pragma unroll
-            for (int i = K - 1; i > 0; --i) win[i] = win[i - 1];
-            win[0] = zj;
-        }
+    clear();
+    load_b(ta, nb - 1);
+    for (int j1 = nb - 1; j1 >= 0; j1 -= 2 * PD) {
+        if (j1 - PD >= 0) load_b(tb, j1 - PD);
+        run_b(ta, j1);
+        if (j1 - 2 * PD >= 0) load_b(ta, j1 - 2 * PD);
+        if (j1 - PD >= 0) run_b(tb, j1 - PD);
     }
 }
 
@@ -1913,18 +1950,24 @@ struct Solver {
         applies += nv * nk;
     }
     void bandSolve(int per_g, int src, int dst, int nv, bool f32 = false) {
-        const dim3 grid((maxldg + 63) / 64, 1, nk * nv);
         const void *Lb = f32 ? h->t32.Lrecip : h->t64.Lrecip;
+        // four (two) vectors per thread where that leaves at least 96 threads an SM
+        const long long cols = (long long)nk * nv * maxldg;
+        const int nvt = !f32 ? 1 : cols >= 4ll * 96 * h->num_sms ? 4 : cols >= 2ll * 96 * h->num_sms ? 2 : 1;
+        const dim3 grid((maxldg + 63) / 64, 1, nk * ((nv + nvt - 1) / nvt));
         switch (h->order) {
-#define MB_BL(KK)                                                                                                 \
-    case KK:                                                                                                      \
-        if (f32)                                                                                                  \
-            MB_LAUNCH_E(KN_BANDED, (eig_banded_solve_kernel<KK, true><<<grid, 64, 0, s>>>(d_k, Lb, per_g, h->nb, src, dst, nv))); \
-        else                                                                                                      \
-            MB_LAUNCH_E(KN_BANDED, (eig_banded_solve_kernel<KK, false><<<grid, 64, 0, s>>>(d_k, Lb, per_g, h->nb, src, dst, nv))); \
+#define MB_BLV(KK, F, NVV)                                                                              \
+    MB_LAUNCH_E(KN_BANDED, (eig_banded_solve_kernel<KK, F, NVV><<<grid, 64, 0, s>>>(d_k, Lb, per_g, h->nb, src, dst, nv)))
+#define MB_BL(KK)                              \
+    case KK:                                   \
+        if (!f32) MB_BLV(KK, false, 1);        \
+        else if (nvt == 4) MB_BLV(KK, true, 4); \
+        else if (nvt == 2) MB_BLV(KK, true, 2); \
+        else MB_BLV(KK, true, 1);              \
         break;
             MB_BL(3) MB_BL(4) MB_BL(5) MB_BL(6) MB_BL(7) MB_BL(8)
 #undef MB_BL
+#undef MB_BLV
         }
     }
     int nc_stage() const { return std::max(M, nc); }
