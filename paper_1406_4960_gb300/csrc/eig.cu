@@ -987,18 +987,22 @@ __global__ void __launch_bounds__(256) gram_rows_kernel(const EigK *ks, int nch,
     }
 }
 
-// A^H B for small ma, mb (<= 48) on the FP32 Gram-Schmidt copies: a CTA
-// takes one chunk of the vector length for the whole ma x mb product,
-// staging KC elements of every A and B vector in shared memory; each thread
-// keeps a 3 x 3 block of outputs in registers.  Partial sums per chunk go to
-// `part` (FP64) and are reduced in a fixed order by gram_reduce_kernel.
-constexpr int GT_KC = 32, GT_MAX = 48;
-// Larger products are covered by GT_MAX x GT_MAX tiles (blockIdx.z).
-__global__ void __launch_bounds__(256) gram_tile32_kernel(const EigK *ks, int nch, VSet A, VSet B, int nsplit,
-                                                          double2 *part) {
-    __shared__ float2 As[GT_KC][GT_MAX + 1];
-    __shared__ float2 Bs[GT_KC][GT_MAX + 1];
-    const int split = blockIdx.x, prob = blockIdx.y;
+// A^H B on the FP32 copies for products wider than the tensor-core kernel's
+// tile: a CTA takes one chunk of the vector length for a 96 x 96 tile of the
+// product, 6 x 6 complex outputs per thread (rows ti + 16 i, columns tj + 16 j:
+// 144 FMAs for 12 shared-memory reads), the next KC elements of every vector
+// copied to shared memory (cp.async) while the staged ones are used.  Bound by the FMA pipe.
+// Partial sums per chunk go to `part` (FP64) and are reduced in a fixed order
+// by gram_reduce_kernel; larger products are covered by tiles (blockIdx.z).
+// (With 3 x 3 outputs per thread on 48 x 48 tiles and no loads in flight:
+// 418 us for 90 x 90 over 115 k elements.)
+constexpr int GT_KC = 16, GT_MAX = 96, GT_R = GT_MAX / 16;
+__global__ void __launch_bounds__(256, 2) gram_tile32_kernel(const EigK *ks, int nch, VSet A, VSet B, int nsplit,
+                                                             double2 *part) {
+    extern __shared__ __align__(16) unsigned char gtsm[];
+    typedef float2 Stage[GT_KC][GT_MAX + 1];
+    Stage *As = reinterpret_cast<Stage *>(gtsm), *Bs = As + 2;     // two buffers each
+    const int split = blockIdx.x, prob = blockIdx.y, tid = threadIdx.x;
     const int k = prob / nch, ch = prob % nch;
     const EigK d = ks[k];
     const int MA = A.count(), MB = B.count();
@@ -1008,48 +1012,57 @@ __global__ void __launch_bounds__(256) gram_tile32_kernel(const EigK *ks, int nc
     const long long n = d.nvec;
     const long long chunk = (n + nsplit - 1) / nsplit;
     const long long t0 = split * chunk, t1 = min(n, t0 + chunk);
-    const int ti = threadIdx.x / 16, tj = threadIdx.x % 16;   // rows 3*ti.., columns 3*tj..
-    float2 acc[3][3];
+    const int ti = tid / 16, tj = tid % 16;
+    // staging: element kk = tid % KC of vectors tid / KC + 16 u
+    const int kk = tid % GT_KC, v0 = tid / GT_KC;
+    auto fetch = [&](long long tb, int buf) {
+        const int in = tb + kk < t1 ? 8 : 0;              // bytes read; the rest is zero
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) acc[i][j] = make_float2(0.f, 0.f);
-    for (long long tb = t0; tb < t1; tb += GT_KC) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < (ma + mb) * GT_KC; e += blockDim.x) {
-            const int v = e / GT_KC, kk = e % GT_KC;
-            const long long t = tb + kk;
-            float2 val = make_float2(0.f, 0.f);
-            if (v < ma) {
-                if (t < t1) val = d.v32[(long long)A.at(r0 + v, ch) * n + t];
-                As[kk][v] = val;
-            } else {
-                if (t < t1) val = d.v32[(long long)B.at(c0 + v - ma, ch) * n + t];
-                Bs[kk][v - ma] = val;
-            }
+        for (int u = 0; u < GT_R; ++u) {
+            const int v = v0 + 16 * u;
+            const float2 *a = d.v32 + (long long)A.at(r0 + min(v, ma - 1), ch) * n + (in ? tb + kk : 0);
+            const float2 *b = d.v32 + (long long)B.at(c0 + min(v, mb - 1), ch) * n + (in ? tb + kk : 0);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(tc::smem_u32(&As[buf][kk][v])), "l"(a),
+                         "r"(v < ma ? in : 0)
+                         : "memory");
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(tc::smem_u32(&Bs[buf][kk][v])), "l"(b),
+                         "r"(v < mb ? in : 0)
+                         : "memory");
         }
-        __syncthreads();
-#pragma unroll 4
-        for (int kk = 0; kk < GT_KC; ++kk) {
-            float2 a[3], b[3];
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float2 acc[GT_R][GT_R];
 #pragma unroll
-            for (int i = 0; i < 3; ++i) a[i] = As[kk][min(3 * ti + i, GT_MAX)];
+    for (int i = 0; i < GT_R; ++i)
 #pragma unroll
-            for (int j = 0; j < 3; ++j) b[j] = Bs[kk][min(3 * tj + j, GT_MAX)];
+        for (int j = 0; j < GT_R; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    int buf = 0;
+    if (t0 < t1) fetch(t0, 0);
+    for (long long tb = t0; tb < t1; tb += GT_KC, buf ^= 1) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();                // this buffer is complete, and the other one's readers have passed
+        if (tb + GT_KC < t1) fetch(tb + GT_KC, buf ^ 1);
+#pragma unroll 2
+        for (int q = 0; q < GT_KC; ++q) {
+            float2 a[GT_R], b[GT_R];
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
+            for (int i = 0; i < GT_R; ++i) a[i] = As[buf][q][ti + 16 * i];
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
+            for (int j = 0; j < GT_R; ++j) b[j] = Bs[buf][q][tj + 16 * j];
+#pragma unroll
+            for (int i = 0; i < GT_R; ++i)
+#pragma unroll
+                for (int j = 0; j < GT_R; ++j) {
                     acc[i][j].x = fmaf(a[i].x, b[j].x, fmaf(a[i].y, b[j].y, acc[i][j].x));
                     acc[i][j].y = fmaf(a[i].x, b[j].y, fmaf(-a[i].y, b[j].x, acc[i][j].y));
                 }
         }
     }
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < GT_R; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const int r = 3 * ti + i, c = 3 * tj + j;
+        for (int j = 0; j < GT_R; ++j) {
+            const int r = ti + 16 * i, c = tj + 16 * j;
             if (r < ma && c < mb)
                 part[((size_t)prob * nsplit + split) * MA * MB + (size_t)(r0 + r) * MB + c0 + c] =
                     make_double2(acc[i][j].x, acc[i][j].y);
@@ -1147,7 +1160,7 @@ __global__ void __launch_bounds__(128) pencil_gram32_kernel(const EigK *ks, int 
 // Requires 2 mb <= 128 and ma <= GTC_NMAX.  Partials go to `part` like the
 // CUDA-core Gram kernels' (reduced by gram_reduce_kernel); a wait on the MMA
 // barrier that runs out sets *err and skips the rest.
-constexpr int GTC_KC = 32;                    // complex elements per step (64 TF32 values per row)
+constexpr int GTC_KC = 16;                    // complex elements per step (32 TF32 values per row)
 constexpr int GTC_NMAX = 64;
 constexpr int GTC_LBO = 128, GTC_SBO = (2 * GTC_KC / 4) * 128;
 __host__ __device__ constexpr size_t gtc_smem_bytes(int ntile) {
@@ -1800,9 +1813,9 @@ struct Solver {
         const int nprob = nk * nch;
         const int ma = A.count(), mbc = B.count();
         if (f32 && mbc >= 4 && 2 * mbc <= 128 && ma <= GTC_NMAX && ma * mbc >= 64) {
-            // tensor cores: two resident CTAs per SM over the whole grid
+            // tensor cores: four resident CTAs per SM over the whole grid
             const int ntile = std::max(16, (ma + 15) / 16 * 16);
-            int nsplit = std::max(1, std::min(1024, (2 * h->num_sms + nprob - 1) / nprob));
+            int nsplit = std::max(1, std::min(1024, (4 * h->num_sms + nprob - 1) / nprob));
             nsplit = std::min<long long>(nsplit, std::max<long long>(1, nmax / (2 * GTC_KC)));
             while ((size_t)nprob * nsplit * ma * mbc > part_cap && nsplit > 1) --nsplit;
             const size_t smem = gtc_smem_bytes(ntile);
@@ -1820,8 +1833,10 @@ struct Solver {
             int nsplit = std::max(1, std::min(1024, (2 * h->num_sms + nprob * tiles - 1) / (nprob * tiles)));
             nsplit = std::min<long long>(nsplit, std::max<long long>(1, nmax / (4 * GT_KC)));
             while ((size_t)nprob * nsplit * ma * mbc > part_cap && nsplit > 1) --nsplit;
-            MB_LAUNCH_E(KN_GRAM32, gram_tile32_kernel<<<dim3(nsplit, nprob, tiles), 256, 0, s>>>(d_k, nch, A, B, nsplit,
-                                                                                               d_part));
+            const size_t smem = (size_t)4 * GT_KC * (GT_MAX + 1) * sizeof(float2);
+            cuda(smem_limit_once((const void *)gram_tile32_kernel, h->device, h->smem_optin));
+            MB_LAUNCH_E(KN_GRAM32, gram_tile32_kernel<<<dim3(nsplit, nprob, tiles), 256, smem, s>>>(d_k, nch, A, B, nsplit,
+                                                                                                  d_part));
             MB_LAUNCH_E(KN_GRAM32,
                         gram_reduce_kernel<<<dim3((ma * mbc + 7) / 8, nprob), 256, 0, s>>>(d_part, nsplit, ma, mbc, G,
                                                                                            lower ? 1 : 0));
