@@ -1225,7 +1225,7 @@ __global__ void __launch_bounds__(128) gram_tc32_kernel(const EigK *ks, int nch,
     // and element (e/8) % KC (a warp reads 8 rows x 4 consecutive elements);
     // each thread holds its elements of one step in registers, loaded while
     // the previous step's products run
-    constexpr int UMAX = GTC_NMAX * GTC_KC / 128;     // 16
+    constexpr int UMAX = GTC_NMAX * GTC_KC / 128;     // 8
     const int nem = ((mb + 7) / 8) * 8 * GTC_KC, nea = ((ma + 7) / 8) * 8 * GTC_KC;
     float2 bv[UMAX], av[UMAX];
     auto fetch = [&](long long tb) {
@@ -1353,64 +1353,122 @@ __device__ __forceinline__ void ff_mac(FF &acc, FF u, FF v) {
 }
 __device__ __forceinline__ FF ff_neg(FF a) { return {-a.h, -a.l}; }
 
+// The combine kernels' tiles of te elements x tc columns lie on blockIdx.x
+// (the only grid axis without a 65535 limit), the column groups of one run of
+// elements side by side, so that they share its reads through L2.
+static unsigned tile_grid(long long n, int te, int mc, int tc) {
+    return (unsigned)((n + te - 1) / te * ((mc + tc - 1) / tc));
+}
+__device__ __forceinline__ int tile_col(int mc, int tc) { return (int)(blockIdx.x % ((mc + tc - 1) / tc)) * tc; }
+__device__ __forceinline__ long long tile_elem(int mc, int tc, int te) {
+    return (long long)(blockIdx.x / ((mc + tc - 1) / tc)) * te;
+}
+
 // C_j = beta C_j + alpha sum_i A_i Y[i][j] on FP64 vectors with the products
 // and sums in float-float arithmetic (the mixed solver's FP64 root rotations:
-// FP64-level results at the FP32 rate).  Same layout and launch as
-// combine2_kernel.
-template <int JC>
-__global__ void __launch_bounds__(256) combine_ff_kernel(const EigK *ks, int nch, VSet A, VSet C,
-                                                         const double2 *Y, double alpha, double beta) {
-    __shared__ float4 Ys[JMAX][JC];     // (re.h, re.l, im.h, im.l)
-    const int prob = blockIdx.y;
+// FP64-level results at the FP32 rate).  Tiles of 64 elements x 48 columns,
+// 4 x 3 outputs per thread (elements tx + 16 i, columns ty + 16 j), so that an
+// element of A is read and split into float-float once for 48 columns: the
+// split runs at the FP64 rate.  Stages of CF_KC vectors go from registers into
+// two buffers, the next one loaded during the products.  Bound by the FP32
+// pipe (13 operations a real product): 90 x 90 over 115 k elements 2.04 ms,
+// 2.94 ms with 12 columns per pass and a split for each.
+constexpr int CF_T = 64, CF_KC = 8, CF_RI = 4, CF_RJ = 3, CF_C = 16 * CF_RJ;
+__global__ void __launch_bounds__(256, 2) combine_ff_kernel(const EigK *ks, int nch, VSet A, VSet C,
+                                                            const double2 *Y, double alpha, double beta) {
+    __shared__ float4 As[2][CF_KC][CF_T], Ys[2][CF_KC][CF_C];        // (re.h, re.l, im.h, im.l)
+    const int ma = A.count(), mc = C.count(), prob = blockIdx.y, tid = threadIdx.x;
     const int k = prob / nch, ch = prob % nch;
     const EigK d = ks[k];
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = t < d.nvec;
-    const int ma = A.count(), mc = C.count();
+    const int j0 = tile_col(mc, CF_C);
+    const long long t0 = tile_elem(mc, CF_C, CF_T);
+    if (t0 >= d.nvec) return;                                        // the batch's longest vectors size the grid
+    const int nt = (int)min((long long)CF_T, d.nvec - t0);
     const double2 *y = Y + (size_t)prob * LD * LD;
-    for (int j0 = 0; j0 < mc; j0 += JC) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < ma * JC; e += blockDim.x) {
-            const int i = e / JC, jj = e % JC;
-            const double2 yv = j0 + jj < mc ? y[i * LD + j0 + jj] : make_double2(0.0, 0.0);
-            const FF re = ff_from(yv.x), im = ff_from(yv.y);
-            Ys[i][jj] = make_float4(re.h, re.l, im.h, im.l);
+    constexpr int NA = CF_KC * CF_T / 256, NY = (CF_KC * CF_C + 255) / 256;
+    double2 ra[NA], ry[NY];
+    auto load = [&](int i0) {
+#pragma unroll
+        for (int u = 0; u < NA; ++u) {
+            const int q = (tid + u * 256) / CF_T, t = (tid + u * 256) % CF_T;
+            ra[u] = i0 + q < ma && t < nt ? d.base[(long long)A.at(i0 + q, ch) * d.nvec + t0 + t] : make_double2(0.0, 0.0);
         }
+#pragma unroll
+        for (int u = 0; u < NY; ++u) {
+            const int q = (tid + u * 256) / CF_C, j = (tid + u * 256) % CF_C;
+            ry[u] = q < CF_KC && i0 + q < ma && j0 + j < mc ? y[(i0 + q) * LD + j0 + j] : make_double2(0.0, 0.0);
+        }
+    };
+    auto split = [](double2 v) {
+        const FF re = ff_from(v.x), im = ff_from(v.y);
+        return make_float4(re.h, re.l, im.h, im.l);
+    };
+    auto stage = [&](int buf) {
+#pragma unroll
+        for (int u = 0; u < NA; ++u) As[buf][(tid + u * 256) / CF_T][(tid + u * 256) % CF_T] = split(ra[u]);
+#pragma unroll
+        for (int u = 0; u < NY; ++u) {
+            const int q = (tid + u * 256) / CF_C;
+            if (q < CF_KC) Ys[buf][q][(tid + u * 256) % CF_C] = split(ry[u]);
+        }
+    };
+    const int tx = tid % 16, ty = tid / 16;
+    FF ar[CF_RI][CF_RJ], ai[CF_RI][CF_RJ];
+#pragma unroll
+    for (int i = 0; i < CF_RI; ++i)
+#pragma unroll
+        for (int j = 0; j < CF_RJ; ++j) ar[i][j] = ai[i][j] = FF{0.f, 0.f};
+    int buf = 0;
+    load(0);
+    for (int i0 = 0; i0 < ma; i0 += CF_KC, buf ^= 1) {
+        stage(buf);                     // its readers passed the barrier of the stage between
         __syncthreads();
-        if (!live) continue;
-        FF ar[JC], ai[JC];
+        if (i0 + CF_KC < ma) load(i0 + CF_KC);
+        const int nq = min(CF_KC, ma - i0);
+        for (int q = 0; q < nq; ++q) {
+            float4 av[CF_RI];
 #pragma unroll
-        for (int jj = 0; jj < JC; ++jj) ar[jj] = ai[jj] = FF{0.f, 0.f};
-        for (int i = 0; i < ma; ++i) {
-            const double2 av = d.base[(long long)A.at(i, ch) * d.nvec + t];
-            const FF xr = ff_from(av.x), xi = ff_from(av.y);
+            for (int i = 0; i < CF_RI; ++i) av[i] = As[buf][q][tx + 16 * i];
 #pragma unroll
-            for (int jj = 0; jj < JC; ++jj) {
-                const float4 w = Ys[i][jj];
+            for (int j = 0; j < CF_RJ; ++j) {
+                if (j0 + 16 * j + (ty & ~1) >= mc) continue;          // uniform in the warp
+                const float4 w = Ys[buf][q][ty + 16 * j];
                 const FF yr{w.x, w.y}, yi{w.z, w.w};
-                ff_mac(ar[jj], xr, yr);          // re += xr yr - xi yi
-                ff_mac(ar[jj], ff_neg(xi), yi);
-                ff_mac(ai[jj], xr, yi);          // im += xr yi + xi yr
-                ff_mac(ai[jj], xi, yr);
+#pragma unroll
+                for (int i = 0; i < CF_RI; ++i) {
+                    const FF xr{av[i].x, av[i].y}, xi{av[i].z, av[i].w};
+                    ff_mac(ar[i][j], xr, yr);          // re += xr yr - xi yi
+                    ff_mac(ar[i][j], ff_neg(xi), yi);
+                    ff_mac(ai[i][j], xr, yi);          // im += xr yi + xi yr
+                    ff_mac(ai[i][j], xi, yr);
+                }
             }
         }
+    }
+    // C is read before any of the stores, which could alias the loads
+    auto col = [&](int j) { return d.base + (long long)C.at(j0 + ty + 16 * j, ch) * d.nvec + t0 + tx; };
 #pragma unroll
-        for (int jj = 0; jj < JC; ++jj) {
-            if (j0 + jj >= mc) break;
-            double2 *c = d.base + (long long)C.at(j0 + jj, ch) * d.nvec + t;
-            const double2 v = make_double2(alpha * ((double)ar[jj].h + (double)ar[jj].l),
-                                           alpha * ((double)ai[jj].h + (double)ai[jj].l));
-            *c = beta == 0.0 ? v : make_double2(beta * c->x + v.x, beta * c->y + v.y);
-        }
+    for (int j = 0; j < CF_RJ; ++j) {
+        if (j0 + ty + 16 * j >= mc) continue;
+        double2 cv[CF_RI];
+#pragma unroll
+        for (int i = 0; i < CF_RI; ++i)
+            cv[i] = beta != 0.0 && tx + 16 * i < nt ? col(j)[16 * i] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int i = 0; i < CF_RI; ++i)
+            if (tx + 16 * i < nt)
+                col(j)[16 * i] = make_double2(beta * cv[i].x + alpha * ((double)ar[i][j].h + (double)ar[i][j].l),
+                                              beta * cv[i].y + alpha * ((double)ai[i][j].h + (double)ai[i][j].l));
     }
 }
 
 // C_j = beta C_j + alpha sum_i A_i Y[i][j]: TE elements per thread (blockDim.x
-// apart) and JC output columns per CTA (blockIdx.z: the column group), their
+// apart) and JC output columns per CTA (blockIdx.x: the column group, so that
+// the groups that read one piece of A run together and share it in L2), their
 // coefficients staged in shared memory and read two columns at a time, so that
-// a pair of 16-byte loads serves 4 TE complex products.  FP32 (F32): bound by
-// the FMA pipe for many columns; FP64: by the FP64 pipe, so small problems
-// take narrow groups to reach every SM.
+// a pair of 16-byte loads serves 4 TE complex products.  FP64: bound by the
+// FP64 pipe, so small problems take narrow groups to reach every SM (15 x 5
+// over 1.5 k elements 41.7 -> 8.9 us); FP32 (F32) for at most 8 columns.
 constexpr int kCombThreads = 128;
 template <int JC, int TE, bool F32>
 __global__ void __launch_bounds__(kCombThreads) combine2_kernel(const EigK *ks, int nch, VSet A, VSet C,
@@ -1418,12 +1476,12 @@ __global__ void __launch_bounds__(kCombThreads) combine2_kernel(const EigK *ks, 
     typedef typename std::conditional<F32, float2, double2>::type T2;
     typedef typename std::conditional<F32, float, double>::type T;
     __shared__ __align__(16) T2 Ys[JMAX][JC];
-    const int prob = blockIdx.y, j0 = blockIdx.z * JC;
+    const int ma = A.count(), mc = C.count(), prob = blockIdx.y;
     const int k = prob / nch, ch = prob % nch;
     const EigK d = ks[k];
-    const long long t0 = (long long)blockIdx.x * (kCombThreads * TE) + threadIdx.x;
+    const int j0 = tile_col(mc, JC);
+    const long long t0 = tile_elem(mc, JC, kCombThreads * TE) + threadIdx.x;
     if (t0 - threadIdx.x >= d.nvec) return;               // the batch's longest vectors size the grid
-    const int ma = A.count(), mc = C.count();
     const double2 *y = Y + (size_t)prob * LD * LD;
     for (int e = threadIdx.x; e < ma * JC; e += kCombThreads) {
         const int i = e / JC, jj = e % JC;
@@ -1461,7 +1519,7 @@ __global__ void __launch_bounds__(kCombThreads) combine2_kernel(const EigK *ks, 
 #pragma unroll
         for (int u = 0; u < TE; ++u) av[u] = t0 + u * kCombThreads < d.nvec ? v[u * kCombThreads] : czero<T2>();
     };
-    constexpr int PF = 4;                                 // vectors in flight
+    constexpr int PF = 6;                                 // vectors in flight
     for (int i = 0; i < ma; i += PF) {
         T2 av[PF][TE];
 #pragma unroll
@@ -1471,17 +1529,121 @@ __global__ void __launch_bounds__(kCombThreads) combine2_kernel(const EigK *ks, 
         for (int p = 0; p < PF; ++p)
             if (i + p < ma) step(i + p, av[p]);
     }
+    // C is read before any of the stores, which could alias the loads
+    auto col = [&](int jj) { return vb + (long long)C.at(j0 + jj, ch) * d.nvec + t0; };
+    T2 cv[TE][JC];
 #pragma unroll
-    for (int jj = 0; jj < JC; ++jj) {
-        if (j0 + jj >= mc) break;
-        T2 *c = vb + (long long)C.at(j0 + jj, ch) * d.nvec + t0;
+    for (int jj = 0; jj < JC; ++jj)
 #pragma unroll
-        for (int u = 0; u < TE; ++u) {
-            if (t0 + u * kCombThreads >= d.nvec) break;
-            const T2 v = rscale((T)alpha, acc[u][jj]);
-            c[u * kCombThreads] = beta == 0.0 ? v : rscale((T)beta, c[u * kCombThreads]) + v;
+        for (int u = 0; u < TE; ++u)
+            cv[u][jj] = beta != 0.0 && j0 + jj < mc && t0 + u * kCombThreads < d.nvec ? col(jj)[u * kCombThreads] : czero<T2>();
+#pragma unroll
+    for (int jj = 0; jj < JC; ++jj)
+#pragma unroll
+        for (int u = 0; u < TE; ++u)
+            if (j0 + jj < mc && t0 + u * kCombThreads < d.nvec)
+                col(jj)[u * kCombThreads] = rscale((T)beta, cv[u][jj]) + rscale((T)alpha, acc[u][jj]);
+}
+
+// The same for many columns of the FP32 copies, as a matrix product in tiles
+// of 128 elements x 16 RJ columns: 8 x RJ complex outputs per thread (elements
+// tx + 16 i, columns ty + 16 j), A staged KC vectors at a time by cp.async,
+// so that every element of A is read once for all its columns.  Yf: the
+// coefficients in FP32 (to_float_kernel; FP64 conversions run at the FP64
+// rate and would cost every CTA a quarter of its time).  Bound by the FMA
+// pipe: 90 x 90 over 115 k elements 341 -> 188 us, four problems of 36 x 36
+// over 23 k 54 -> 39 us against combine2_kernel's 12 columns per CTA.
+constexpr int CT_T = 128, CT_KC = 8;
+template <int RJ> constexpr size_t combine_tile_smem() {
+    return (size_t)2 * CT_KC * (CT_T + 16 * RJ) * sizeof(float2);
+}
+template <int RJ>
+__global__ void __launch_bounds__(256, RJ > 3 ? 1 : 2) combine_tile_kernel(const EigK *ks, int nch, VSet A, VSet C,
+                                                                          const float2 *Yf, float alpha, float beta) {
+    extern __shared__ __align__(16) unsigned char ctsm[];
+    typedef float2 StageA[CT_KC][CT_T];
+    typedef float2 StageY[CT_KC][16 * RJ];
+    StageA *As = reinterpret_cast<StageA *>(ctsm);                 // two buffers each
+    StageY *Ys = reinterpret_cast<StageY *>(As + 2);
+    const int ma = A.count(), mc = C.count(), prob = blockIdx.y, tid = threadIdx.x;
+    const int k = prob / nch, ch = prob % nch;
+    const EigK d = ks[k];
+    const int j0 = tile_col(mc, 16 * RJ);
+    const long long t0 = tile_elem(mc, 16 * RJ, CT_T);
+    if (t0 >= d.nvec) return;                                      // the batch's longest vectors size the grid
+    const int nt = (int)min((long long)CT_T, d.nvec - t0);         // a multiple of 32
+    const float2 *y = Yf + (size_t)prob * LD * LD;
+    // staging: 16 bytes (two elements) of A per copy, one coefficient per copy
+    auto fetch = [&](int i0, int buf) {
+#pragma unroll
+        for (int e = tid; e < CT_KC * CT_T / 2; e += 256) {
+            const int q = e / (CT_T / 2), t = e % (CT_T / 2) * 2;
+            const bool in = i0 + q < ma && t < nt;
+            const float2 *a = d.v32 + (long long)A.at(in ? i0 + q : 0, ch) * d.nvec + (in ? t0 + t : 0);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(&As[buf][q][t])), "l"(a),
+                         "r"(in ? 16 : 0)
+                         : "memory");
+        }
+#pragma unroll
+        for (int e = tid; e < CT_KC * 16 * RJ; e += 256) {
+            const int q = e / (16 * RJ), j = e % (16 * RJ);
+            const bool in = i0 + q < ma && j0 + j < mc;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(tc::smem_u32(&Ys[buf][q][j])),
+                         "l"(y + (in ? (i0 + q) * LD + j0 + j : 0)), "r"(in ? 8 : 0)
+                         : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    const int tx = tid % 16, ty = tid / 16;
+    float2 acc[8][RJ];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < RJ; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    int buf = 0;
+    fetch(0, 0);
+    for (int i0 = 0; i0 < ma; i0 += CT_KC, buf ^= 1) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();                // this buffer is complete, and the other one's readers have passed
+        if (i0 + CT_KC < ma) fetch(i0 + CT_KC, buf ^ 1);
+#pragma unroll 2
+        for (int q = 0; q < CT_KC; ++q) {
+            float2 av[8], w[RJ];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) av[i] = As[buf][q][tx + 16 * i];
+#pragma unroll
+            for (int j = 0; j < RJ; ++j) w[j] = Ys[buf][q][ty + 16 * j];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < RJ; ++j) cfma(acc[i][j], av[i], w[j]);
         }
     }
+    // C is read a column ahead of its stores, which could alias the loads
+    auto col = [&](int j) { return d.v32 + (long long)C.at(j0 + ty + 16 * j, ch) * d.nvec + t0 + tx; };
+    auto old = [&](int j, float2(&cv)[8]) {
+        const bool in = beta != 0.f && j < RJ && j0 + ty + 16 * j < mc;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) cv[i] = in && tx + 16 * i < nt ? col(j)[16 * i] : make_float2(0.f, 0.f);
+    };
+    float2 cv[2][8];
+    old(0, cv[0]);
+#pragma unroll
+    for (int j = 0; j < RJ; ++j) {
+        old(j + 1, cv[(j + 1) & 1]);
+        if (j0 + ty + 16 * j >= mc) continue;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (tx + 16 * i < nt) col(j)[16 * i] = rscale(beta, cv[j & 1][i]) + rscale(alpha, acc[i][j]);
+    }
+}
+
+// rows i < ma, columns j < mc of every problem's matrix in FP32
+__global__ void to_float_kernel(const double2 *Y, float2 *Yf, int ma, int mc) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= ma * mc) return;
+    const size_t o = (size_t)blockIdx.y * LD * LD + (e / mc) * LD + e % mc;
+    Yf[o] = make_float2((float)Y[o].x, (float)Y[o].y);
 }
 
 // The same for one output column (a chain's Gram-Schmidt update): 16 bytes
@@ -1757,6 +1919,7 @@ struct Solver {
     int o32X = 0, o32SX = 0, o32HX = 0, o32W = 0, o32K = 0, o32SK = 0, o32HK = 0, o32T = 0, o32T2 = 0, n32 = 0;
     double2 *d_Sg = nullptr, *d_Ub = nullptr, *d_Tb = nullptr;
     int *d_statb = nullptr;
+    float2 *d_Yf = nullptr;    // FP32 copy of a rotation's coefficients
     int oV, oHV, oSV, oVB, oHVB, oSVB, oQ, oHQ, oW, oSW, oT;
     int nvecs;
     std::vector<EigK> kd_host;
@@ -1862,14 +2025,14 @@ struct Solver {
             combine_t<true>(nch, A, C, Y, alpha, beta);
         } else if (gs32 && C.count() > 8) {
             // mixed solver, FP64 vectors: the root rotations in float-float
-            const dim3 grid((unsigned)((nmax + 255) / 256), nk * nch);
-            MB_LAUNCH_E(KN_COMBINE, (combine_ff_kernel<12><<<grid, 256, 0, s>>>(d_k, nch, A, C, Y, alpha, beta)));
+            const dim3 grid(tile_grid(nmax, CF_T, C.count(), CF_C), nk * nch);
+            MB_LAUNCH_E(KN_COMBINE, combine_ff_kernel<<<grid, 256, 0, s>>>(d_k, nch, A, C, Y, alpha, beta));
         } else {
             combine_t<false>(nch, A, C, Y, alpha, beta);
         }
     }
     template <int JC, int TE, bool F32> void combine_j(int nch, VSet A, VSet C, const double2 *Y, double alpha, double beta) {
-        const dim3 grid((unsigned)((nmax + kCombThreads * TE - 1) / (kCombThreads * TE)), nk * nch, (C.count() + JC - 1) / JC);
+        const dim3 grid(tile_grid(nmax, kCombThreads * TE, C.count(), JC), nk * nch);
         MB_LAUNCH_E(F32 ? KN_COMBINE32 : KN_COMBINE,
                     (combine2_kernel<JC, TE, F32><<<grid, kCombThreads, 0, s>>>(d_k, nch, A, C, Y, alpha, beta)));
     }
@@ -1882,20 +2045,37 @@ struct Solver {
                             d_k, nch, A, C, Y, alpha, beta)));
             return;
         }
+        if (F32 && mc > 8) {
+            // one column tile where 48 or 96 columns hold them all, else the
+            // width with less padding
+            const int np = nk * nch, w48 = (mc + 47) / 48 * 48, w96 = (mc + 95) / 96 * 96;
+            const float fa = (float)alpha, fb = (float)beta;
+            MB_LAUNCH_E(KN_COMBINE32, to_float_kernel<<<dim3((A.count() * mc + 127) / 128, np), 128, 0, s>>>(Y, d_Yf, A.count(), mc));
+            if (w48 < w96) {
+                cuda(smem_limit_once((const void *)combine_tile_kernel<3>, h->device, h->smem_optin));
+                MB_LAUNCH_E(KN_COMBINE32, (combine_tile_kernel<3><<<dim3(tile_grid(nmax, CT_T, mc, 48), np), 256, combine_tile_smem<3>(), s>>>(
+                                              d_k, nch, A, C, d_Yf, fa, fb)));
+            } else {
+                cuda(smem_limit_once((const void *)combine_tile_kernel<6>, h->device, h->smem_optin));
+                MB_LAUNCH_E(KN_COMBINE32, (combine_tile_kernel<6><<<dim3(tile_grid(nmax, CT_T, mc, 96), np), 256, combine_tile_smem<6>(), s>>>(
+                                              d_k, nch, A, C, d_Yf, fa, fb)));
+            }
+            return;
+        }
         // the widest column group (least re-reading of A) among those with the
         // least padding, narrow ones where wide ones would leave SMs idle
         const long long ctas = (nmax + kCombThreads - 1) / kCombThreads * nk * nch;
         auto waste = [&](int jc) { return (mc + jc - 1) / jc * jc - mc; };
         if (mc <= 2 || (!F32 && ctas * ((mc + 11) / 12) < 2 * h->num_sms)) {
             combine_j<2, 1, F32>(nch, A, C, Y, alpha, beta);
-        } else if (mc <= 4 || ctas * ((mc + 11) / 12) < 2 * h->num_sms) {
+        } else if (mc <= 4) {
             combine_j<4, 1, F32>(nch, A, C, Y, alpha, beta);
         } else if (mc <= 8) {
             combine_j<8, 1, F32>(nch, A, C, Y, alpha, beta);
         } else if (waste(10) < waste(12)) {
-            combine_j<10, F32 ? 2 : 1, F32>(nch, A, C, Y, alpha, beta);
+            combine_j<10, 1, false>(nch, A, C, Y, alpha, beta);
         } else {
-            combine_j<12, F32 ? 2 : 1, F32>(nch, A, C, Y, alpha, beta);
+            combine_j<12, 1, false>(nch, A, C, Y, alpha, beta);
         }
     }
     // U = L^{-H} of np problems (FP32 arithmetic in the bulk cycles)
@@ -2430,6 +2610,7 @@ int eigsolve(mb_handle *h, int nbands, double tol, int prec, double *evals, void
         S.d_Ub = S.alloc<double2>((size_t)nprob * LD * LD);
         S.d_Tb = S.alloc<double2>((size_t)nprob * LD * LD);
         S.d_statb = S.alloc<int>(nprob);
+        S.d_Yf = S.alloc<float2>((size_t)nprob * LD * LD);
     }
     if (S.rc) return S.rc;
     S.cuda(cudaMemcpyAsync(S.d_k, S.kd_host.data(), sizeof(EigK) * S.nk, cudaMemcpyHostToDevice, s));
@@ -2721,8 +2902,8 @@ extern "C" int mb_debug_combine_ff(const void *A, const double *Y, long long n, 
     if (e == cudaSuccess) e = cudaMemcpyAsync(Yd, hY.data(), sizeof(double2) * LD * LD, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dk, &hk, sizeof(EigK), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
-        const dim3 grid((unsigned)((n + 255) / 256), 1);
-        combine_ff_kernel<12><<<grid, 256, 0, s>>>(dk, 1, vs(0, ma), vs(ma, mc), Yd, 1.0, 0.0);
+        const dim3 grid(tile_grid(n, CF_T, mc, CF_C), 1);
+        combine_ff_kernel<<<grid, 256, 0, s>>>(dk, 1, vs(0, ma), vs(ma, mc), Yd, 1.0, 0.0);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
