@@ -38,8 +38,7 @@ namespace mb {
 
 constexpr int LD = 128;       // leading dimension of subspace matrices
 constexpr int JMAX = 112;     // largest subspace the Jacobi kernel holds (matrix in shared memory)
-constexpr int JPAIRS = 58;    // rotation slots per Jacobi round (>= JMAX/2 + 1, even so that
-                              // 5*JPAIRS doubles keep the next double2 array 16-byte aligned)
+constexpr int JPAIRS = 56;    // rotation slots per Jacobi round (JMAX / 2)
 
 struct EigK {
     double2 *base;            // FP64 vectors of this k-point, stride nvec
@@ -316,348 +315,268 @@ __global__ void seed_kernel(const double *dots, int M, int mconv, int nk, int nc
 }
 
 // ---------------------------------------------------------------------------
-// Jacobi diagonalization of one Hermitian m x m matrix per CTA (m <= JMAX),
-// parallel (round-robin) ordering: m'/2 disjoint rotations per round.
+// Jacobi diagonalization of Hermitian m x m matrices (m <= JMAX), parallel
+// (round-robin) ordering: m'/2 disjoint rotations per round.
+//
+// A problem takes gridDim.x CTAs.  Every one of them holds all of A in shared
+// memory and computes the same rotations, but only its share of the rows of
+// the eigenvector matrix, which is most of the work of one CTA and needs
+// nothing from the other rows: no communication, and the result does not
+// depend on the number of CTAs.  Bound by instruction issue (FP32) or the
+// FP64 pipe of one SM, so the index arithmetic of the 2 x 2 blocks is done
+// once for all rounds and blocks whose two rotations are the identity are
+// skipped.  The FP32 problems of 90 to 95 columns of a solve took 1.1 ms on the
+// mean with one CTA each and take 0.5 ms with 15.
 
-// Per-round scratch of the sweeps (shared memory, sized for T = double).
-struct JacobiScratch {
-    unsigned char *rc;   // per pair: c, s, t*|apq|, app, aqq   (5 * JPAIRS T)
-    unsigned char *re;   // per pair: phase e                     (JPAIRS T2)
-    int *pp;             // per pair: p, q
-    double *red;         // 32 partial sums
-    int *stop;
+// rotation of pair (p, q): columns times diag(1, conj e) [[c, s], [-s, c]]
+template <typename T> struct __align__(16) JRot {
+    T c, s;
+    typename std::conditional<std::is_same<T, float>::value, float2, double2>::type e;
 };
-constexpr int kJacobiThreads = 512;    // one CTA per problem
-constexpr size_t kJacobiScratchBytes = 5 * JPAIRS * sizeof(double) + JPAIRS * sizeof(double2) + 2 * JPAIRS * sizeof(int);
-
-// Sweeps until the off-diagonal Frobenius norm is <= rel_tol * sqrt(fro2).
-// A (m x m, row-major) in shared memory; V is updated as V <- V J through
-// vget/vset (shared or global memory).
-template <typename T, typename VGet, typename VSet_>
-__device__ void jacobi_sweeps(typename std::conditional<std::is_same<T, float>::value, float2, double2>::type *A,
-                              int m, VGet vget, VSet_ vset, int max_sweeps, double rel_tol, double fro2,
-                              JacobiScratch js) {
-    typedef typename std::conditional<std::is_same<T, float>::value, float2, double2>::type T2;
-    const T skip_rel = std::is_same<T, float>::value ? T(1e-7) : T(1e-15);
-    T *rc = reinterpret_cast<T *>(js.rc);
-    T2 *re = reinterpret_cast<T2 *>(js.re);
-    int *pp = js.pp;
-    const int mp = (m + 1) & ~1;      // players, padded to even
-    const int npair = mp / 2;
-    const int nblk2 = npair * (npair + 1) / 2;   // 2x2 blocks (I >= J) of the pair partition
-    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        for (int r = 0; r < mp - 1; ++r) {
-            // rotation of every pair of the round (q >= m: an index left
-            // alone this round, identity)
-            for (int pi = threadIdx.x; pi < npair; pi += blockDim.x) {
-                int a = pi == 0 ? 0 : ((r + pi - 1) % (mp - 1)) + 1;
-                int b = ((r + mp - 1 - pi - 1) % (mp - 1)) + 1;
-                if (pi == 0) b = ((r + mp - 2) % (mp - 1)) + 1;
-                const int p = min(a, b), q = max(a, b);
-                T c = 1, s = 0, tm = 0;
-                T2 ep = mk(T(1), T(0));
-                if (q < m) {
-                    T2 apq = A[p * m + q];
-                    T mag = hypot(apq.x, apq.y);
-                    T app = A[p * m + p].x, aqq = A[q * m + q].x;
-                    rc[5 * pi + 3] = app;
-                    rc[5 * pi + 4] = aqq;
-                    // rotations below rounding level of the diagonal are skipped
-                    if (mag > skip_rel * sqrt(fabs(app * aqq)) && mag > T(1e-30)) {
-                        ep = mk(apq.x / mag, apq.y / mag);
-                        T th = (aqq - app) / (T(2) * mag);
-                        T t = (th >= 0 ? T(1) : T(-1)) / (fabs(th) + sqrt(th * th + T(1)));
-                        c = T(1) / sqrt(t * t + T(1));
-                        s = t * c;
-                        tm = t * mag;
-                    }
-                }
-                pp[2 * pi] = p;
-                pp[2 * pi + 1] = q;
-                rc[5 * pi] = c;
-                rc[5 * pi + 1] = s;
-                rc[5 * pi + 2] = tm;
-                re[pi] = ep;
-            }
-            __syncthreads();
-            // A <- J^H A J by 2x2 blocks (rows of pair I, columns of pair J,
-            // I >= J; the block above the diagonal is written as the
-            // conjugate transpose), then V <- V J by (pair, row).
-            // J = diag(1, e^-i phi) [[c, s], [-s, c]] on each pair's columns.
-            for (int e = threadIdx.x; e < nblk2 + npair * m; e += blockDim.x) {
-                if (e < nblk2) {
-                    int I = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-                    while (I * (I + 1) / 2 > e) --I;
-                    while ((I + 1) * (I + 2) / 2 <= e) ++I;
-                    const int J = e - I * (I + 1) / 2;
-                    const int pI = pp[2 * I], qI = pp[2 * I + 1], pJ = pp[2 * J], qJ = pp[2 * J + 1];
-                    const bool vI = qI < m, vJ = qJ < m;
-                    const T sI = rc[5 * I + 1], sJ = rc[5 * J + 1];
-                    const bool actI = vI && sI != T(0), actJ = vJ && sJ != T(0);
-                    T2 a00 = A[pI * m + pJ];
-                    T2 a01 = vJ ? A[pI * m + qJ] : czero<T2>();
-                    T2 a10 = vI ? A[qI * m + pJ] : czero<T2>();
-                    T2 a11 = (vI && vJ) ? A[qI * m + qJ] : czero<T2>();
-                    if (I == J && actI) {
-                        a00 = mk(rc[5 * I + 3] - rc[5 * I + 2], T(0));
-                        a11 = mk(rc[5 * I + 4] + rc[5 * I + 2], T(0));
-                        a01 = a10 = czero<T2>();
-                    } else {
-                        if (actJ) {   // columns pJ, qJ
-                            const T cJ = rc[5 * J];
-                            const T2 ec = mk(re[J].x, -re[J].y);
-                            T2 x = a00, y = cmul(ec, a01);
-                            a00 = rscale(cJ, x) - rscale(sJ, y);
-                            a01 = rscale(sJ, x) + rscale(cJ, y);
-                            x = a10;
-                            y = cmul(ec, a11);
-                            a10 = rscale(cJ, x) - rscale(sJ, y);
-                            a11 = rscale(sJ, x) + rscale(cJ, y);
-                        }
-                        if (actI) {   // rows pI, qI
-                            const T cI = rc[5 * I];
-                            T2 x = a00, y = cmul(re[I], a10);
-                            a00 = rscale(cI, x) - rscale(sI, y);
-                            a10 = rscale(sI, x) + rscale(cI, y);
-                            x = a01;
-                            y = cmul(re[I], a11);
-                            a01 = rscale(cI, x) - rscale(sI, y);
-                            a11 = rscale(sI, x) + rscale(cI, y);
-                        }
-                    }
-                    A[pI * m + pJ] = a00;
-                    if (vJ) A[pI * m + qJ] = a01;
-                    if (vI) A[qI * m + pJ] = a10;
-                    if (vI && vJ) A[qI * m + qJ] = a11;
-                    if (I != J) {
-                        A[pJ * m + pI] = mk(a00.x, -a00.y);
-                        if (vJ) A[qJ * m + pI] = mk(a01.x, -a01.y);
-                        if (vI) A[pJ * m + qI] = mk(a10.x, -a10.y);
-                        if (vI && vJ) A[qJ * m + qI] = mk(a11.x, -a11.y);
-                    }
-                } else {
-                    const int e2 = e - nblk2;
-                    const int pi = e2 / m, row = e2 % m;
-                    const int p = pp[2 * pi], q = pp[2 * pi + 1];
-                    if (q >= m || rc[5 * pi + 1] == T(0)) continue;
-                    const T c = rc[5 * pi], s = rc[5 * pi + 1];
-                    const T2 ec = mk(re[pi].x, -re[pi].y);
-                    T2 vp = vget(row, p), vq = cmul(ec, vget(row, q));
-                    vset(row, p, rscale(c, vp) - rscale(s, vq));
-                    vset(row, q, rscale(s, vp) + rscale(c, vq));
-                }
-            }
-            __syncthreads();
-        }
-        // off-diagonal norm
-        double o = 0.0;
-        for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-            int i = e / m, j = e % m;
-            if (i != j) o += (double)A[e].x * A[e].x + (double)A[e].y * A[e].y;
-        }
-        for (int off = 16; off > 0; off >>= 1) o += __shfl_down_sync(0xffffffffu, o, off);
-        if ((threadIdx.x & 31) == 0) js.red[threadIdx.x >> 5] = o;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double s = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += js.red[w];
-            *js.stop = s <= rel_tol * rel_tol * fro2;
-        }
-        __syncthreads();
-        if (*js.stop) break;
-    }
+constexpr int kJacobiThreads = 512;                       // at most
+constexpr int kJacobiBlocks = 4;                         // 2x2 blocks per thread, at most
+static_assert(JPAIRS * (JPAIRS + 1) / 2 <= kJacobiBlocks * kJacobiThreads, "a thread's blocks");
+template <typename T> constexpr size_t jacobi_smem(int m, int rows) {
+    return (((size_t)(m + rows) * m + 1) & ~(size_t)1) * 2 * sizeof(T) + JPAIRS * (sizeof(JRot<T>) + 2 * sizeof(T) + 2 * sizeof(int));
 }
 
-// A (m x m) from the lower triangle of the problem's G (Hermitian
-// completion: with the subspace ordered [roots | Krylov vectors], the
-// coupling block comes from K^H (H X), which uses the roots' HX rather than
-// the Krylov vectors' HK, which may come from a reduced-precision apply);
-// dead slots become decoupled with a huge diagonal.  Returns the squared
-// Frobenius norm of the live part (all threads).
+// A from the lower triangle of the problem's G (Hermitian completion: with the
+// subspace ordered [roots | Krylov vectors], the coupling block comes from
+// K^H (H X), which uses the roots' HX rather than the Krylov vectors' HK,
+// which may come from a reduced-precision apply); dead slots become decoupled
+// with a huge diagonal.  full (or null): the completed matrix, of which this
+// CTA writes rows [r0, r1).  Returns the squared Frobenius norm of the live
+// part (all threads).
 template <typename T2>
-__device__ double jacobi_load(const double2 *g, int m, const int *dead, int dead_stride, int dead_ofs, T2 *A,
+__device__ double jacobi_load(const double2 *g, int m, const int *dead, int dead_ofs, T2 *A, double2 *full, int r0, int r1,
                               double *red) {
-    const int prob = blockIdx.x;
     double f = 0.0;
     for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        int i = e / m, j = e % m;
+        const int i = e / m, j = e % m;
         double2 v = i >= j ? g[i * LD + j] : g[j * LD + i];
         if (i < j) v.y = -v.y;
         if (i == j) v.y = 0.0;
-        bool di = dead && dead[prob * dead_stride + i] == 0 && i >= dead_ofs;
-        bool dj = dead && dead[prob * dead_stride + j] == 0 && j >= dead_ofs;
+        const bool di = dead && dead[i] == 0 && i >= dead_ofs;
+        const bool dj = dead && dead[j] == 0 && j >= dead_ofs;
         if (di || dj) v = make_double2((i == j) ? 1e30 : 0.0, 0.0);
         else f += v.x * v.x + v.y * v.y;
         A[e] = mk((decltype(A[0].x))v.x, (decltype(A[0].x))v.y);
+        if (full && i >= r0 && i < r1) full[i * LD + j] = v;
     }
     for (int off = 16; off > 0; off >>= 1) f += __shfl_down_sync(0xffffffffu, f, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = f;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        red[0] = s;
-    }
+    double s = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
     __syncthreads();
-    const double fro2 = red[0];
-    __syncthreads();
-    return fro2;
+    return s;
 }
 
-// ascending order of the diagonal (selection sort by one thread)
-template <typename T2>
-__device__ void jacobi_sort(const T2 *A, int m, int *perm) {
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < m; ++i) perm[i] = i;
-        for (int i = 0; i < m; ++i) {
-            int b = i;
-            for (int j = i + 1; j < m; ++j)
-                if (A[perm[j] * m + perm[j]].x < A[perm[b] * m + perm[b]].x) b = j;
-            int t = perm[i]; perm[i] = perm[b]; perm[b] = t;
-        }
-    }
-    __syncthreads();
-}
-
-// VS: the eigenvector matrix lives in shared memory beside A (m <= 84);
-// otherwise it overwrites the input matrix G in global memory (m <= JMAX).
-// T = float runs the rotations in FP32 (the mixed solver's bulk cycles).
-template <bool VS, typename T>
-__global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(double2 *G, int m, const int *dead, int dead_stride,
-                                                     int dead_ofs, double *evals, double2 *evecs,
-                                                     int max_sweeps, double rel_tol) {
+// Sweeps until the off-diagonal Frobenius norm is <= rel_tol * that of the
+// matrix.  sort: eigenvalues ascending (else column i stays near slot i, dead
+// slots exactly there).  T = float: the rotations in FP32.
+template <typename T>
+__global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double2 *G, int m, const int *dead, int dead_stride,
+                                                                int dead_ofs, double *evals, double2 *evecs, double2 *full,
+                                                                int sort, int max_sweeps, double rel_tol) {
     typedef typename std::conditional<std::is_same<T, float>::value, float2, double2>::type T2;
     extern __shared__ __align__(16) unsigned char sm[];
-    const int prob = blockIdx.x;
+    const int prob = blockIdx.y, tid = threadIdx.x, nt = blockDim.x;
+    const int r0 = blockIdx.x * m / gridDim.x, r1 = (blockIdx.x + 1) * m / gridDim.x, rows = r1 - r0;
+    const T skip_rel = std::is_same<T, float>::value ? T(1e-7) : T(1e-15);
     T2 *A = reinterpret_cast<T2 *>(sm);
-    T2 *Vs = A + m * m;                                                  // eigenvectors in shared memory (VS)
-    double2 *Vg = G + (size_t)prob * LD * LD;                            // or in place of G
-    const int ldv = VS ? m : LD;
-    unsigned char *scr = reinterpret_cast<unsigned char *>(A + (VS ? 2 : 1) * m * m);
+    T2 *V = A + m * m;                                    // rows r0 .. r1 - 1
+    JRot<T> *rot = reinterpret_cast<JRot<T> *>(A + (((m + (m + gridDim.x - 1) / gridDim.x) * m + 1) & ~1u));
+    T *diag = reinterpret_cast<T *>(rot + JPAIRS);        // per pair: the rotated diagonal
+    int2 *pq = reinterpret_cast<int2 *>(diag + 2 * JPAIRS);
     __shared__ double red[32];
-    __shared__ int stop;
     __shared__ int perm[LD];
-    JacobiScratch js{scr, scr + 5 * JPAIRS * sizeof(double), reinterpret_cast<int *>(scr + 5 * JPAIRS * sizeof(double) + JPAIRS * sizeof(double2)),
-                     red, &stop};
-    auto vget = [&](int r, int c) -> T2 {
-        if (VS) return Vs[r * ldv + c];
-        const double2 v = Vg[r * ldv + c];
-        return mk((T)v.x, (T)v.y);
-    };
-    auto vset = [&](int r, int c, T2 v) {
-        if (VS) Vs[r * ldv + c] = v;
-        else Vg[r * ldv + c] = make_double2((double)v.x, (double)v.y);
-    };
-    const double fro2 = jacobi_load(G + (size_t)prob * LD * LD, m, dead, dead_stride, dead_ofs, A, red);
-    // G is read completely (jacobi_load ends on a barrier) before V, possibly G itself, is initialised
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        int i = e / m, j = e % m;
-        vset(i, j, mk(T(i == j ? 1 : 0), T(0)));
+    const size_t o = (size_t)prob * LD * LD;
+    const double fro2 = jacobi_load(G + o, m, dead ? dead + prob * dead_stride : nullptr, dead_ofs, A,
+                                    full ? full + o : nullptr, r0, r1, red);
+    for (int e = tid; e < rows * m; e += nt) V[e] = mk(T(e % m == r0 + e / m ? 1 : 0), T(0));
+    const int mp = (m + 1) & ~1;      // players, padded to even
+    const int npair = mp / 2;
+    // this thread's 2x2 blocks (I >= J) of the pair partition
+    int bI[kJacobiBlocks], bJ[kJacobiBlocks];
+#pragma unroll
+    for (int k = 0; k < kJacobiBlocks; ++k) {
+        const int e = tid + k * nt;
+        int I = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+        while (I * (I + 1) / 2 > e) --I;
+        while ((I + 1) * (I + 2) / 2 <= e) ++I;
+        bI[k] = I < npair ? I : -1;
+        bJ[k] = e - I * (I + 1) / 2;
     }
     __syncthreads();
-    jacobi_sweeps<T>(A, m, vget, vset, max_sweeps, rel_tol, fro2, js);
-    jacobi_sort(A, m, perm);
-    for (int c = threadIdx.x; c < m; c += blockDim.x) evals[(size_t)prob * LD + c] = A[perm[c] * m + perm[c]].x;
-    double2 *out = evecs + (size_t)prob * LD * LD;
-    if (!VS && out == Vg) {
-        // eigenvectors already in place of G: permute their columns through
-        // the (now free) shared matrix A, one row at a time
-        for (int r = 0; r < m; ++r) {
-            for (int c = threadIdx.x; c < m; c += blockDim.x) A[c] = vget(r, perm[c]);
+    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
+        double off2 = 0.0;
+        for (int e = tid; e < m * m; e += nt)
+            if (e / m > e % m) off2 += (double)(A[e].x * A[e].x + A[e].y * A[e].y);
+        for (int off = 16; off > 0; off >>= 1) off2 += __shfl_down_sync(0xffffffffu, off2, off);
+        if ((tid & 31) == 0) red[tid >> 5] = off2;
+        __syncthreads();
+        off2 = 0.0;
+        for (int w = 0; w < nt / 32; ++w) off2 += 2 * red[w];
+        __syncthreads();                                  // red is free again, and everyone leaves together
+        if (off2 <= rel_tol * rel_tol * fro2) break;
+        for (int r = 0; r < mp - 1; ++r) {
+            // rotation of every pair of the round (q >= m: an index left
+            // alone this round, identity)
+            if (tid < npair) {
+                const int a = tid == 0 ? 0 : ((r + tid - 1) % (mp - 1)) + 1;
+                const int b = tid == 0 ? ((r + mp - 2) % (mp - 1)) + 1 : ((r + mp - 1 - tid - 1) % (mp - 1)) + 1;
+                const int p = min(a, b), q = max(a, b);
+                JRot<T> w;
+                w.c = 1, w.s = 0, w.e = mk(T(1), T(0));
+                if (q < m) {
+                    const T2 apq = A[p * m + q];
+                    const T app = A[p * m + p].x, aqq = A[q * m + q].x;
+                    // rotations below rounding level of the diagonal are
+                    // skipped (in FP64 first by the components' bound: the
+                    // square roots take 64 clocks an operation)
+                    const T big = T(1.5) * max(fabs(apq.x), fabs(apq.y));
+                    if (big > T(1e-30) && (sizeof(T) == 4 || big * big > skip_rel * skip_rel * fabs(app * aqq))) {
+                        const T mag = hypot(apq.x, apq.y);
+                        if (mag > skip_rel * sqrt(fabs(app * aqq)) && mag > T(1e-30)) {
+                            w.e = mk(apq.x / mag, apq.y / mag);
+                            const T th = (aqq - app) / (T(2) * mag);
+                            const T t = (th >= 0 ? T(1) : T(-1)) / (fabs(th) + sqrt(th * th + T(1)));
+                            w.c = T(1) / sqrt(t * t + T(1));
+                            w.s = t * w.c;
+                            diag[2 * tid] = app - t * mag;
+                            diag[2 * tid + 1] = aqq + t * mag;
+                        }
+                    }
+                }
+                pq[tid] = make_int2(p, q);
+                rot[tid] = w;
+            }
             __syncthreads();
-            for (int c = threadIdx.x; c < m; c += blockDim.x) out[r * LD + c] = make_double2(A[c].x, A[c].y);
+            // A <- J^H A J by 2x2 blocks (rows of pair I, columns of pair J,
+            // I >= J; the block above the diagonal is written as the
+            // conjugate transpose)
+#pragma unroll
+            for (int k = 0; k < kJacobiBlocks; ++k) {
+                const int I = bI[k], J = bJ[k];
+                if (I < 0) break;
+                const T sI = rot[I].s, sJ = rot[J].s;
+                if (sI == T(0) && sJ == T(0)) continue;
+                const int pI = pq[I].x, qI = pq[I].y, pJ = pq[J].x, qJ = pq[J].y;
+                const bool vI = qI < m, vJ = qJ < m;
+                if (I == J) {
+                    A[pI * m + pI] = mk(diag[2 * I], T(0));
+                    A[qI * m + qI] = mk(diag[2 * I + 1], T(0));
+                    A[pI * m + qI] = A[qI * m + pI] = czero<T2>();
+                    continue;
+                }
+                T2 a00 = A[pI * m + pJ];
+                T2 a01 = vJ ? A[pI * m + qJ] : czero<T2>();
+                T2 a10 = vI ? A[qI * m + pJ] : czero<T2>();
+                T2 a11 = (vI && vJ) ? A[qI * m + qJ] : czero<T2>();
+                if (sJ != T(0)) {     // columns pJ, qJ
+                    const JRot<T> w = rot[J];
+                    const T2 ec = mk(w.e.x, -w.e.y);
+                    T2 x = a00, y = cmul(ec, a01);
+                    a00 = rscale(w.c, x) - rscale(w.s, y);
+                    a01 = rscale(w.s, x) + rscale(w.c, y);
+                    x = a10;
+                    y = cmul(ec, a11);
+                    a10 = rscale(w.c, x) - rscale(w.s, y);
+                    a11 = rscale(w.s, x) + rscale(w.c, y);
+                }
+                if (sI != T(0)) {     // rows pI, qI
+                    const JRot<T> w = rot[I];
+                    T2 x = a00, y = cmul(w.e, a10);
+                    a00 = rscale(w.c, x) - rscale(w.s, y);
+                    a10 = rscale(w.s, x) + rscale(w.c, y);
+                    x = a01;
+                    y = cmul(w.e, a11);
+                    a01 = rscale(w.c, x) - rscale(w.s, y);
+                    a11 = rscale(w.s, x) + rscale(w.c, y);
+                }
+                A[pI * m + pJ] = a00;
+                A[pJ * m + pI] = mk(a00.x, -a00.y);
+                if (vJ) {
+                    A[pI * m + qJ] = a01;
+                    A[qJ * m + pI] = mk(a01.x, -a01.y);
+                }
+                if (vI) {
+                    A[qI * m + pJ] = a10;
+                    A[pJ * m + qI] = mk(a10.x, -a10.y);
+                }
+                if (vI && vJ) {
+                    A[qI * m + qJ] = a11;
+                    A[qJ * m + qI] = mk(a11.x, -a11.y);
+                }
+            }
+            // V <- V J: half a warp per pair, a lane per row
+            for (int pi = tid / 16; pi < npair; pi += nt / 16) {
+                const JRot<T> w = rot[pi];
+                if (w.s == T(0)) continue;
+                const int2 c = pq[pi];
+                const T2 ec = mk(w.e.x, -w.e.y);
+                for (int row = tid % 16; row < rows; row += 16) {
+                    T2 *v = V + row * m;
+                    const T2 x = v[c.x], y = cmul(ec, v[c.y]);
+                    v[c.x] = rscale(w.c, x) - rscale(w.s, y);
+                    v[c.y] = rscale(w.s, x) + rscale(w.c, y);
+                }
+            }
             __syncthreads();
         }
-    } else {
-        for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-            int r = e / m, c = e % m;
-            const T2 v = vget(r, perm[c]);
-            out[r * LD + c] = make_double2(v.x, v.y);
+    }
+    // slot of every column: its rank on the diagonal (equal values, the dead
+    // slots, in their order)
+    if (tid < m) perm[tid] = tid;
+    __syncthreads();
+    if (sort && tid < m) {
+        const T v = A[tid * m + tid].x;
+        int rank = 0;
+        for (int j = 0; j < m; ++j) {
+            const T u = A[j * m + j].x;
+            rank += u < v || (u == v && j < tid);
         }
+        perm[rank] = tid;
+    }
+    __syncthreads();
+    if (blockIdx.x == 0 && tid < m) evals[(size_t)prob * LD + tid] = A[perm[tid] * m + perm[tid]].x;
+    for (int e = tid; e < rows * m; e += nt) {
+        const T2 v = V[e / m * m + perm[e % m]];
+        evecs[o + (size_t)(r0 + e / m) * LD + e % m] = make_double2(v.x, v.y);
     }
 }
 
-// FP64 result from FP32 sweeps (m <= JMIX_MAX): Jacobi in FP32 gives V0;
-// B = V0^H A V0 is formed in FP64 (off-diagonal at the FP32 level), FP64
-// sweeps on B converge in one or two (quadratic convergence), and the
-// eigenvectors are V0 V1.  Same result as FP64 sweeps from the start, with
-// most rotations at the FP32 rate.
-constexpr int JMIX_MAX = 64;
-__global__ void __launch_bounds__(kJacobiThreads) jacobi_mixed_kernel(const double2 *G, int m, const int *dead, int dead_stride,
-                                                           int dead_ofs, double *evals, double2 *evecs,
-                                                           int max_sweeps, double rel_tol) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    const int prob = blockIdx.x;
-    double2 *A64 = reinterpret_cast<double2 *>(sm);
-    double2 *W64 = A64 + m * m;
-    float2 *A32 = reinterpret_cast<float2 *>(W64 + m * m);
-    float2 *V32 = A32 + m * m;
-    unsigned char *scr = reinterpret_cast<unsigned char *>(V32 + m * m);
-    __shared__ double red[32];
-    __shared__ int stop;
-    __shared__ int perm[LD];
-    JacobiScratch js{scr, scr + 5 * JPAIRS * sizeof(double), reinterpret_cast<int *>(scr + 5 * JPAIRS * sizeof(double) + JPAIRS * sizeof(double2)),
-                     red, &stop};
-    const double fro2 = jacobi_load(G + (size_t)prob * LD * LD, m, dead, dead_stride, dead_ofs, A64, red);
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        const int i = e / m, j = e % m;
-        A32[e] = make_float2((float)A64[e].x, (float)A64[e].y);
-        V32[e] = make_float2(i == j ? 1.f : 0.f, 0.f);
+// FP64 result from FP32 sweeps: X0 of the FP32 sweeps is refined by two steps
+// of the Ogita-Aishima iteration (Iterative refinement for symmetric
+// eigenvalue decomposition, Japan J. Indust. Appl. Math. 35, 2018): with
+// S = X^H A X, P = X^H X, R = I - P and l_i = S_ii / P_ii,
+//   X <- X + X E,  E_ij = (S_ij + l_j R_ij) / (l_j - l_i),  E_ii = R_ii / 2,
+// which squares the error of the vectors and of their orthogonality.  Where
+// that E_ij is above lim (neighbours that FP32 does not separate), R_ij / 2
+// only makes the two orthogonal and the FP64 sweeps on X^H A X rotate them.
+// lim^2 is the loss of orthogonality the next step (or FP64) must absorb:
+// 1e-4 in the first step, 1e-8 in the second.
+__global__ void refine_kernel(const double2 *S, const double2 *P, double2 *E, int m, double lim) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= m * m) return;
+    const size_t o = (size_t)blockIdx.y * LD * LD;
+    const int i = e / m, j = e % m;
+    if (i < j) return;
+    const double2 p = P[o + i * LD + j];
+    if (i == j) {
+        E[o + i * LD + i] = make_double2(0.5 * (1.0 - p.x), 0.0);
+        return;
     }
-    __syncthreads();
-    auto v32get = [&](int r, int c) -> float2 { return V32[r * m + c]; };
-    auto v32set = [&](int r, int c, float2 v) { V32[r * m + c] = v; };
-    jacobi_sweeps<float>(A32, m, v32get, v32set, max_sweeps, 1e-6, fro2, js);
-    // W = A V0, then A <- V0^H W  (FP64)
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        const int i = e / m, j = e % m;
-        double2 s = make_double2(0.0, 0.0);
-        for (int q = 0; q < m; ++q) {
-            const float2 v = V32[q * m + j];
-            cfma(s, A64[i * m + q], make_double2(v.x, v.y));
-        }
-        W64[e] = s;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        const int i = e / m, j = e % m;
-        double2 s = make_double2(0.0, 0.0);
-        for (int q = 0; q < m; ++q) {
-            const float2 v = V32[q * m + i];
-            cfma(s, make_double2(v.x, -v.y), W64[q * m + j]);
-        }
-        A64[e] = s;
-    }
-    __syncthreads();
-    // exact Hermitian symmetry and real diagonal before the FP64 sweeps
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        const int i = e / m, j = e % m;
-        if (i > j) {
-            const double2 lo = A64[e], up = A64[j * m + i];
-            const double2 h = make_double2(0.5 * (lo.x + up.x), 0.5 * (lo.y - up.y));
-            A64[e] = h;
-            A64[j * m + i] = make_double2(h.x, -h.y);
-        } else if (i == j) {
-            A64[e].y = 0.0;
-        }
-        W64[e] = make_double2(i == j ? 1.0 : 0.0, 0.0);
-    }
-    __syncthreads();
-    auto v64get = [&](int r, int c) -> double2 { return W64[r * m + c]; };
-    auto v64set = [&](int r, int c, double2 v) { W64[r * m + c] = v; };
-    jacobi_sweeps<double>(A64, m, v64get, v64set, max_sweeps, rel_tol, fro2, js);
-    jacobi_sort(A64, m, perm);
-    for (int c = threadIdx.x; c < m; c += blockDim.x) evals[(size_t)prob * LD + c] = A64[perm[c] * m + perm[c]].x;
-    double2 *out = evecs + (size_t)prob * LD * LD;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        const int r = e / m, c = e % m, pc = perm[c];
-        double2 s = make_double2(0.0, 0.0);
-        for (int q = 0; q < m; ++q) {
-            const float2 v = V32[r * m + q];
-            cfma(s, make_double2(v.x, v.y), W64[q * m + pc]);
-        }
-        out[r * LD + c] = s;
-    }
+    // the lower triangle, and E_ji = conj(R_ij - E_ij), so that E + E^H = R
+    // holds to rounding however small the gap
+    const double li = S[o + i * LD + i].x / P[o + i * LD + i].x, lj = S[o + j * LD + j].x / P[o + j * LD + j].x;
+    const double2 sv = S[o + i * LD + j];
+    const double nx = sv.x - lj * p.x, ny = sv.y - lj * p.y, gap = lj - li;
+    const bool far = fmax(fabs(nx), fabs(ny)) <= lim * fabs(gap) && gap != 0.0;
+    const double2 v = far ? make_double2(nx / gap, ny / gap) : make_double2(-0.5 * p.x, -0.5 * p.y);
+    E[o + i * LD + j] = v;
+    E[o + j * LD + i] = make_double2(-p.x - v.x, p.y + v.y);
 }
 
 // U = L^{-H} with G = L L^H (G Hermitian positive definite, m <= JMAX), one
@@ -1732,21 +1651,44 @@ __global__ void mask_sgram_kernel(double2 *G, const int *mask, int m) {
     if (di || dj) g[i * LD + j] = make_double2(i == j ? 1.0 : 0.0, 0.0);
 }
 
-// C = op(A) B for small m x m matrices (leading dimension LD), one thread per
-// output element; op = conjugate transpose when conjA.
-__global__ void small_zgemm_kernel(const double2 *A, const double2 *B, double2 *C, int m, int conjA) {
-    const int prob = blockIdx.y;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= m * m) return;
-    const int i = e / m, j = e % m;
-    const double2 *a = A + (size_t)prob * LD * LD, *b = B + (size_t)prob * LD * LD;
-    double2 s = make_double2(0.0, 0.0);
-    for (int q = 0; q < m; ++q) {
-        double2 av = conjA ? a[q * LD + i] : a[i * LD + q];
-        if (conjA) av.y = -av.y;
-        cfma(s, av, b[q * LD + j]);
+// C = op(A) B (+ D) for small m x m matrices (leading dimension LD), op =
+// conjugate transpose when conjA; a second product op(A) B2 into C2 where given.
+// Bound by the FP64 pipe and the latency of the operands: 8 x 8 outputs per
+// CTA, so that 90 x 90 reaches every SM, the sum split over the warps of all
+// four FP64 pipes, all of A's and B's share in shared memory behind one
+// barrier.  (One thread per output on 128-thread CTAs reading both operands
+// through L2: 30 us for m = 95, now 12.)
+__global__ void __launch_bounds__(256) small_zgemm_kernel(const double2 *A, const double2 *B, double2 *C, int m, int conjA,
+                                                          const double2 *D, const double2 *B2, double2 *C2) {
+    __shared__ double2 As[JMAX][9], Bs[JMAX][8], sum[3][64];
+    const size_t o = (size_t)blockIdx.z * LD * LD;
+    const int i0 = blockIdx.y * 8, j0 = blockIdx.x * 8, tid = threadIdx.x, part = tid / 64, t = tid % 64, ti = t / 8, tj = t % 8;
+#pragma unroll 4
+    for (int e = tid; e < 8 * m; e += 256) {
+        const int q = conjA ? e / 8 : e % m, i = conjA ? e % 8 : e / m;      // along the rows of memory
+        double2 v = i0 + i < m ? (conjA ? A[o + q * LD + i0 + i] : A[o + (i0 + i) * LD + q]) : make_double2(0.0, 0.0);
+        if (conjA) v.y = -v.y;
+        As[q][i] = v;
     }
-    C[(size_t)prob * LD * LD + i * LD + j] = s;
+    const int i = i0 + ti, j = j0 + tj;
+    const bool in = part == 0 && i < m && j < m;
+    for (int pass = 0; pass < (B2 ? 2 : 1); ++pass) {
+        const double2 *b = pass ? B2 : B;
+#pragma unroll 4
+        for (int e = tid; e < 8 * m; e += 256) Bs[e / 8][tj] = j < m ? b[o + (e / 8) * LD + j] : make_double2(0.0, 0.0);
+        __syncthreads();
+        double2 s = make_double2(0.0, 0.0);
+#pragma unroll 4
+        for (int q = part; q < m; q += 4) cfma(s, As[q][ti], Bs[q][tj]);
+        if (part > 0) sum[part - 1][t] = s;
+        __syncthreads();
+        if (in) {
+            s = (s + sum[0][t]) + (sum[1][t] + sum[2][t]);
+            if (D) s = s + D[o + i * LD + j];
+            (pass ? C2 : C)[o + i * LD + j] = s;
+        }
+        __syncthreads();
+    }
 }
 
 // dead-slot mask of a subspace: columns < ofs are the block's inputs (the
@@ -2088,9 +2030,10 @@ struct Solver {
             MB_LAUNCH_E(KN_SMALL, cholinv_kernel<double><<<np, kCholThreads, cholinv_smem<double>(m), s>>>(G, m, U, status));
         }
     }
-    void small_gemm(const double2 *A, const double2 *B, double2 *C, int m, int conjA, int np = 0) {
-        MB_LAUNCH_E(KN_SMALL, small_zgemm_kernel<<<dim3((m * m + 127) / 128, np > 0 ? np : nk), 128, 0, s>>>(
-                                  A, B, C, m, conjA));
+    void small_gemm(const double2 *A, const double2 *B, double2 *C, int m, int conjA, int np = 0, const double2 *D = nullptr,
+                    const double2 *B2 = nullptr, double2 *C2 = nullptr) {
+        const unsigned t = (unsigned)(m + 7) / 8;
+        MB_LAUNCH_E(KN_SMALL, small_zgemm_kernel<<<dim3(t, t, np > 0 ? np : nk), 256, 0, s>>>(A, B, C, m, conjA, D, B2, C2));
     }
     void copy(int nch, VSet S, VSet D, int mode) {
         const unsigned bx = (unsigned)std::min<long long>(64, (nmax + 255) / 256);
@@ -2294,34 +2237,51 @@ struct Solver {
         }
         applyH_chain(nch, kd - 1, kV, kH, cs);
     }
+    // eigenpairs of d_G (overwritten unless f32) into d_evals, d_Y
     void jacobi(int nch, int m, bool masked, int ofs, bool f32 = false) {
-        if (f32) jacobi_t<float>(nch, m, masked, ofs, 1e-6);
-        else jacobi_t<double>(nch, m, masked, ofs, 1e-13);
-    }
-    template <typename T> void jacobi_t(int nch, int m, bool masked, int ofs, double tol) {
-        const size_t c2 = 2 * sizeof(T);
-        const size_t stat = 32 * sizeof(double) + sizeof(int) + LD * sizeof(int) + 256;
-        size_t smem2 = (size_t)2 * m * m * c2 + kJacobiScratchBytes;
-        size_t smem1 = (size_t)m * m * c2 + kJacobiScratchBytes;
-        size_t smemx = (size_t)m * m * (2 * sizeof(double2) + 2 * sizeof(float2)) + kJacobiScratchBytes;
-        const bool vs = smem2 + stat <= (size_t)h->smem_optin;
-        const bool mixed = std::is_same<T, double>::value && m <= JMIX_MAX && smemx + stat <= (size_t)h->smem_optin;
-        int np = nk * nch;
+        const int np = nk * nch;
         if (masked)
             MB_LAUNCH_E(KN_SMALL, alive_mask_kernel<<<(np + 63) / 64, 64, 0, s>>>(d_alive, kd, ofs, M, b, nch, m, np, d_mask));
-        if (mixed) {
-            cuda(smem_limit_once((const void *)jacobi_mixed_kernel, h->device, h->smem_optin));
-            MB_LAUNCH_E(KN_JACOBI, (jacobi_mixed_kernel<<<np, kJacobiThreads, smemx, s>>>(d_G, m, masked ? d_mask : nullptr, LD, 0,
-                                                                               d_evals, d_Y, 30, tol)));
-        } else if (vs) {
-            cuda(smem_limit_once((const void *)jacobi_kernel<true, T>, h->device, h->smem_optin));
-            MB_LAUNCH_E(KN_JACOBI, (jacobi_kernel<true, T><<<np, kJacobiThreads, smem2, s>>>(d_G, m, masked ? d_mask : nullptr, LD, 0,
-                                                                                  d_evals, d_Y, 30, tol)));
-        } else {
-            cuda(smem_limit_once((const void *)jacobi_kernel<false, T>, h->device, h->smem_optin));
-            MB_LAUNCH_E(KN_JACOBI, (jacobi_kernel<false, T><<<np, kJacobiThreads, smem1, s>>>(d_G, m, masked ? d_mask : nullptr, LD, 0,
-                                                                                   d_evals, d_Y, 30, tol)));
+        if (f32) {
+            jacobi_t<float>(np, m, masked, d_G, d_Y, nullptr, true, 1e-6);
+            return;
         }
+        // FP32 sweeps, two refinement steps, FP64 sweeps on what they leave
+        // (m = 95: 0.15 to 1.5 ms in all, 6.8 ms with FP64 sweeps throughout,
+        // which the FP64 pipe of one SM bounds at 3 ms a sweep)
+        const size_t one = (size_t)np * LD * LD;
+        double2 *b0 = d_part, *b1 = b0 + one, *b2 = b1 + one, *A = b2 + one;
+        const dim3 ge((m * m + 127) / 128, np);
+        jacobi_t<float>(np, m, masked, d_G, d_Y, A, false, 1e-6);
+        small_gemm(A, d_Y, b0, m, 0, np);                          // A X0
+        small_gemm(d_Y, b0, b1, m, 1, np, nullptr, d_Y, b2);        // S, P
+        MB_LAUNCH_E(KN_JACOBI, refine_kernel<<<ge, 128, 0, s>>>(b1, b2, b0, m, 1e-4));
+        small_gemm(d_Y, b0, b1, m, 0, np, d_Y);                    // X1 = X0 + X0 E
+        small_gemm(A, b1, b0, m, 0, np);
+        small_gemm(b1, b0, b2, m, 1, np, nullptr, b1, d_Y);
+        MB_LAUNCH_E(KN_JACOBI, refine_kernel<<<ge, 128, 0, s>>>(b2, d_Y, b0, m, 1e-8));
+        small_gemm(b1, b0, b2, m, 0, np, b1);                      // X2
+        small_gemm(A, b2, b0, m, 0, np);
+        small_gemm(b2, b0, d_G, m, 1, np);                         // X2^H A X2
+        jacobi_t<double>(np, m, masked, d_G, b0, nullptr, true, 1e-13);
+        small_gemm(b2, b0, d_Y, m, 0, np);
+    }
+    // CTAs per problem: as many as give each 6 rows of eigenvectors (fewer
+    // would not shorten a round) and fit on the SMs, and enough for the
+    // matrix and the rows to fit in shared memory
+    template <typename T>
+    void jacobi_t(int np, int m, bool masked, const double2 *G, double2 *Y, double2 *full, bool sort, double tol) {
+        const size_t stat = 32 * sizeof(double) + LD * sizeof(int) + 256;
+        int nc = std::max(1, std::min(h->num_sms / np, m / 6));
+        while (nc < m && jacobi_smem<T>(m, (m + nc - 1) / nc) + stat > (size_t)h->smem_optin) ++nc;
+        // a thread per 2x2 block up to 512: a round of a small problem is a few
+        // latencies and two barriers, which more warps only lengthen (m = 10:
+        // 50 us with 512 threads, 32 with 128)
+        const int npair = (m + 1) / 2, blocks = npair * (npair + 1) / 2;
+        const int nt = blocks <= 128 ? 128 : blocks <= 256 ? 256 : kJacobiThreads;
+        cuda(smem_limit_once((const void *)jacobi_kernel<T>, h->device, h->smem_optin));
+        MB_LAUNCH_E(KN_JACOBI, (jacobi_kernel<T><<<dim3(nc, np), nt, jacobi_smem<T>(m, (m + nc - 1) / nc), s>>>(
+                                   G, m, masked ? d_mask : nullptr, LD, 0, d_evals, Y, full, sort ? 1 : 0, 30, tol)));
     }
     // bulk cycles of the mixed solver (before the FP64 finish phase)
     bool lowp() const { return gs32 && !fp64_roots; }
@@ -2591,7 +2551,8 @@ int eigsolve(mb_handle *h, int nbands, double tol, int prec, double *evals, void
     S.d_U = S.alloc<double2>((size_t)S.nk * LD * LD);
     S.d_G2 = S.alloc<double2>((size_t)S.nk * LD * LD);
     S.d_T = S.alloc<double2>((size_t)S.nk * LD * LD);
-    S.part_cap = (size_t)std::max(2 * h->num_sms, nprob) * JMAX * JMAX;
+    // Gram partials; the four matrices of the FP64 refinement
+    S.part_cap = std::max((size_t)std::max(2 * h->num_sms, nprob) * JMAX * JMAX, (size_t)4 * nprob * LD * LD);
     S.d_part = S.alloc<double2>(S.part_cap);
     S.d_evals = S.alloc<double>((size_t)nprob * LD);
     S.d_eps = S.alloc<double>((size_t)S.nk * S.M);

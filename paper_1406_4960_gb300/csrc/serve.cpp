@@ -82,7 +82,7 @@ size_t footprint_of(const mb_handle &h, int nbands, int prec) {
         work += (size_t)(3 * M + nc * (1 + 3 * kd) + 2 * std::max(M, nblk * b)) * vec_bytes / 2;
     const size_t LD = 128;
     work += (size_t)h.kp.size() * nc * LD * LD * (prec != MB_FP64 ? 6 * 16 + 8 : 3 * 16) + (size_t)h.kp.size() * LD * LD * 16 * 3;
-    work += (size_t)std::max<size_t>(304, h.kp.size() * nc) * 112 * 112 * 16;
+    work += std::max((size_t)std::max<size_t>(304, h.kp.size() * nc) * 112 * 112, (size_t)4 * h.kp.size() * nc * LD * LD) * 16;
     // apply scratch: boundary rows + projector overlaps (generous bound)
     size_t scratch = (size_t)h.kp.size() *
                      ((size_t)M * 40 * 2 * (h.order - 1) * maxldg * 16 +

@@ -1,7 +1,7 @@
 """The eigensolver's tiled vector kernels at the edges of their tiles: the FP32
 and float-float rotations (48 and 96 columns per tile, one or two tiles), the
-S-Gram inverse and the small Rayleigh-Ritz problem at odd and large numbers of
-roots, and the float-float kernel's element and column remainders.
+S-Gram inverse and the small Rayleigh-Ritz problem (FP32 sweeps, and FP64 ones
+from a refined FP32 result) at odd and large numbers of roots, and the float-float kernel's element and column remainders.
 
 Tolerances: eigenvalues 1e-6 Ha of the dense FP64 ones as in
 test_gpu_eigsolve.py (residual 1e-6 and an error of its square over the gap);
@@ -37,11 +37,12 @@ def dense():
     return E.generalized_lowest(mod.dense_H(), mod.dense_S(), 95)
 
 
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
 @pytest.mark.parametrize("nroots", [9, 43, 85, 86, 95])
-def test_roots_at_the_tile_edges(mbmod, dense, nroots):
+def test_roots_at_the_tile_edges(mbmod, dense, nroots, prec):
     w = dataclasses.replace(W.tiny(), nbands=nroots, name=f"tiny-{nroots}")
     h = mbmod.Handle.from_workload(w)
-    ev, info = h.eigsolve(nroots, 1e-6, "fp32")
+    ev, info = h.eigsolve(nroots, 1e-6, prec)
     assert info.max_residual < 1e-6
     assert np.abs(ev[0] - dense[:nroots]).max() < 1e-6
     h.close()
