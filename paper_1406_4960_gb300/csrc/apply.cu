@@ -24,6 +24,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <numeric>
 #include <mutex>
 
 #include "apply_common.cuh"
@@ -694,6 +695,9 @@ static int upload_rs_tables(mb_handle *h) {
         h->rs_npos[ik] = (int)(pos.size() / per) - h->rs_pofs[ik];
     }
     if (pos.empty()) pos.push_back(0);
+    RsShape sh;
+    if (rs_shapes<float>(h->n1, h->n2, h->order, &sh, 1)) h->rs_slots[0] = rs_resident<float>(sh, h->num_sms);
+    if (rs_shapes<double>(h->n1, h->n2, h->order, &sh, 1)) h->rs_slots[1] = rs_resident<double>(sh, h->num_sms);
     int rc;
     if ((rc = dev_upload(h, &h->d_rspos, pos.data(), pos.size() * sizeof(int)))) return rc;
     if ((rc = dev_upload(h, (void **)&h->d_rsgpos, gpos.data(), gpos.size() * sizeof(int)))) return rc;
@@ -820,7 +824,9 @@ struct PlanePlan {
     bool rs = false;       // row-space kernel (else the radix-2 plane kernel)
     RsShape sh;            // its instance
     int np = 1;            // radix-2 kernel: planes in flight
-    int nchunks = 1;       // runs of rows (row-space) or knot intervals (radix-2)
+    int nchunks = 1;       // radix-2 kernel: runs of knot intervals
+    int workers = 1;       // row-space kernel: equal runs of all bands' rows,
+    int snap = 0;          // their ends moved to a band boundary this near
     size_t smem = 0;
 };
 
@@ -828,7 +834,7 @@ struct PlanePlan {
 // times the rounds that the items take on `slots` resident CTAs.  waves > 0:
 // an explicit target of about that many items per slot.
 template <typename Cost>
-static int wave_model_chunks(int pairs, int slots, int nmax_chunks, int waves, Cost cost) {
+static int wave_model_chunks(int pairs, int slots, int nmax_chunks, int waves, Cost cost, double *best_cost = nullptr) {
     if (waves > 0) {
         const int target = std::max(1, (waves * slots + pairs - 1) / pairs);
         return std::min(nmax_chunks, target);
@@ -841,6 +847,7 @@ static int wave_model_chunks(int pairs, int slots, int nmax_chunks, int waves, C
         const double c = (double)rounds * cost(n);
         if (c < best - 1e-9) { best = c; nch = n; }
     }
+    if (best_cost) *best_cost = best;
     return nch;
 }
 
@@ -867,13 +874,54 @@ static PlanePlan plan_plane(const mb_handle *h, int nsel, const int *iks, int nb
         // are about a third of a row's work, and a step of the row loop costs
         // about two rows' latency.  FP64 CTAs of one SM share its FP64 pipe,
         // which one of them fills: they count as one slot.
-        const int S = p.sh.s1 * p.sh.s2;
-        p.nchunks = wave_model_chunks(nsel * nbands, h->num_sms * (c2 == 16 ? 1 : p.sh.ctas_per_sm) / S, std::min(kMaxChunks, h->nb), waves, [&](int n) {
+        const int S = p.sh.s1 * p.sh.s2, pairs = nsel * nbands;
+        const int slots = c2 == 16 && S == 1 ? h->num_sms : h->rs_slots[c2 == 16];
+        double best = 0.0;
+        const int nchunks = wave_model_chunks(pairs, slots, std::min(kMaxChunks, h->nb), waves, [&](int n) {
             const int L = (h->nb + n - 1) / n;
             const int in = std::min(h->nb, L + (n == 1 ? 0 : n == 2 ? kRsHalo : 2 * kRsHalo));
             const int steps = (std::min(h->nb, L + (n > 2 ? kRsHalo : 0)) + kRsHalo + p.sh.rows - 1) / p.sh.rows;
             return 0.35 * in + 0.65 * L + 2.0 * steps;
-        });
+        }, &best);
+        p.workers = pairs * nchunks;
+        // Runs that do not end with a band, one for every slot: no last round
+        // that is nearly empty, for two halos and about two steps more a
+        // worker.  FP32: a plan costs between its longest slot and its mean
+        // slot, since the CTAs share L2's bandwidth for the potential (80
+        // folded bands on 36 clusters 327 -> 268 us, 1536 bands on 152 SMs
+        // 906 -> 812; but 256 half bands on 304 slots are 55 us and 304 runs
+        // 61).  FP64: the longest slot, with the projector overlaps (2 nz
+        // FMAs a coefficient, 59 operations a grid point) on what is left
+        // idle (320 CTAs in clusters of 4 5.45 -> 4.64 ms; but 128 bands on
+        // 152 SMs leave 24 SMs to the overlaps: 1.30 ms for the whole apply,
+        // 1.39 without).
+        const long long rows = (long long)pairs * h->nb;
+        if (waves == 0 && rows >= slots) {
+            const int L = (int)((rows + slots - 1) / slots), whole = L / h->nb, rest = L % h->nb, RR = p.sh.rows;
+            const int full = (h->nb + kRsHalo + RR - 1) / RR;            // steps of a whole band
+            const int steps = whole * full + (rest + 3 * kRsHalo + RR - 1) / RR + 1;
+            const long long rounds = ((long long)pairs * nchunks + slots - 1) / slots;
+            bool better;
+            if (c2 == 8) {
+                const int Lc = (h->nb + nchunks - 1) / nchunks;
+                const int in = std::min(h->nb, Lc + (nchunks == 1 ? 0 : nchunks == 2 ? kRsHalo : 2 * kRsHalo));
+                const int sc = (std::min(h->nb, Lc + (nchunks > 2 ? kRsHalo : 0)) + kRsHalo + RR - 1) / RR;
+                const double item = 0.35 * in + 0.65 * Lc + 1.5 * sc + 3.0;
+                const double runs = 0.5 * item * ((double)rounds + (double)pairs * nchunks / slots);
+                better = L + 0.7 * kRsHalo + 1.5 * steps + 3.0 * (whole + 2) < 0.98 * runs;
+            } else {
+                long long ldg = 0;
+                for (int i = 0; i < nsel; ++i) ldg += h->kp[iks[i]].ldg;
+                const double nl = (h->nterm > 0 ? 2.0 * h->nzf * ldg / nsel : 0.0) / (59.0 * NN) * rows;
+                const double cost = L + 0.7 * kRsHalo + 2.0 * steps;
+                auto with_nl = [&](double c, double busy) { return std::max(c, (busy + nl) / slots); };
+                better = with_nl(cost, cost * slots) < 0.98 * with_nl(best, best / rounds * pairs * nchunks);
+            }
+            if (better) {
+                p.workers = slots;
+                p.snap = std::min(2, L / 8);
+            }
+        }
         return p;
     }
     int maxldg = 0;
@@ -1163,7 +1211,11 @@ static int apply_H_launch(mb_handle *h, int nsel, const int *iks, const void *co
         ra.phase_stride = (size_t)h->total_ldg;
         ra.nbands = nbands;
         ra.nb = h->nb;
-        ra.nchunks = plan.nchunks;
+        ra.workers = plan.workers;
+        const long long rows = (long long)nsel * nbands * h->nb, div = std::gcd(rows, (long long)plan.workers);
+        ra.num = (int)(rows / div);
+        ra.den = (int)(plan.workers / div);
+        ra.snap = plan.snap;
         ra.s1 = plan.sh.s1;
         ra.s2 = plan.sh.s2;
         ra.pruned = h->rs_pruned;
@@ -1179,7 +1231,7 @@ static int apply_H_launch(mb_handle *h, int nsel, const int *iks, const void *co
             d.gofs = h->kofs[ik];
         }
         cudaError_t e = cudaSuccess;
-        MB_LAUNCH(h, s, KN_PLANE, e = rs_launch<R>(ra, plan.sh, (unsigned)(nsel * nbands * plan.nchunks), s));
+        MB_LAUNCH(h, s, KN_PLANE, e = rs_launch<R>(ra, plan.sh, s));
         MB_CUDA(e);
     } else {
         PlaneArgs<R> pa;

@@ -127,6 +127,7 @@ struct mb_handle {
     void *d_rspos = nullptr;
     std::vector<int> rs_pofs, rs_npos;
     bool rs_pruned = false;
+    int rs_slots[2] = {1, 1};         // CTAs or clusters of the kernel that fit on the device (FP32, FP64)
     void *d_projB = nullptr;         // BF16 projector tables for the tensor-core contractions
     void *d_tcerr = nullptr;         // status word of the tensor-core kernels' bounded waits
     std::vector<int> pb0_ofs, pb1_ofs, pb0_ld, pb1_ld;

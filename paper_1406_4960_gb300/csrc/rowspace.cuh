@@ -10,8 +10,9 @@
 // B-spline row replace one pair per Gauss plane (nquad per knot interval,
 // about six times as many).
 //
-// A CTA takes one (k-point, band, run of rows) item and walks the rows in
-// steps of RR, on RR planes in shared memory and five more for the history:
+// A CTA takes a run of the rows of all k-points and bands (a piece of a band,
+// or the end of one, whole ones and the beginning of another, so that every
+// CTA of one round has the same work) and walks each band's rows in steps of RR, on RR planes in shared memory and five more for the history:
 //   A  the step's coefficient rows onto compact planes (the disc's occupied
 //      rows and columns only: a cyclic shift of the frequency index along an
 //      axis is a phase in real space, which commutes with the real U);
@@ -42,9 +43,9 @@
 // latency at 16 warps per SM, which 128 registers a thread leave.  Against
 // one transform pair per Gauss plane (the compact-plane and register-FFT
 // kernels that this one replaced), per launch:
-//   slab, 4 k x 32 bands     FP32 0.155 -> 0.058 ms   FP64 4.38 -> 1.11 ms
-//   graphene, 80 bands       FP32 0.868 -> 0.33 ms    FP64 42 -> 5.5 ms
-//   64 k x 24 bands          FP32 3.48 -> 0.94 ms
+//   slab, 4 k x 32 bands     FP32 0.155 -> 0.055 ms   FP64 4.38 -> 1.00 ms
+//   graphene, 80 bands       FP32 0.868 -> 0.27 ms    FP64 42 -> 4.64 ms
+//   64 k x 24 bands          FP32 3.48 -> 0.81 ms
 // A line in one thread's registers sets the 32-point limit (64 FP32
 // registers); RR = 16 rows a step make one line per thread and keep the
 // 5-row halo small; 64-bit accesses to rows padded by one entry are free of
@@ -52,6 +53,7 @@
 // loads of U) and 8-row steps with twice the CTAs measured the same or slower.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <cstdio>
 
@@ -144,12 +146,17 @@ __global__ void __launch_bounds__(T, CTAS) rowspace_kernel(const __grid_constant
     const int tid = threadIdx.x;
     const int S = FOLD ? a.s1 * a.s2 : 1;
     const int rank = FOLD ? (int)(blockIdx.x % (unsigned)S) : 0;
-    const int item = FOLD ? (int)(blockIdx.x / (unsigned)S) : (int)blockIdx.x;
-    const int c = item % a.nchunks, kb = item / a.nchunks, b = kb % a.nbands;
+    const int w = FOLD ? (int)(blockIdx.x / (unsigned)S) : (int)blockIdx.x, nb = a.nb;
+    const int rbeg = rs_cut(w, a.num, a.den, nb, a.snap), rend = rs_cut(w + 1, a.num, a.den, nb, a.snap);
+    for (int r = rbeg; r < rend;) {
+    const bool first = r == rbeg;
+    const int kb = r / nb, b = kb % a.nbands;
     const RsK &d = a.d[kb / a.nbands];
-    const int nb = a.nb, ldg = d.ldg;
-    const int j0 = chunk_begin(c, nb, a.nchunks), j1 = chunk_begin(c + 1, nb, a.nchunks);   // output rows
-    const int ji = max(0, j0 - H), je = min(nb, j1 + H);                                    // rows transformed
+    const int ldg = d.ldg;
+    const int j0 = r - kb * nb, j1 = min(nb, j0 + rend - r);      // output rows
+    const int ji = max(0, j0 - H), je = min(nb, j1 + H);          // rows transformed
+    r += j1 - j0;
+    if (!FOLD && !first) __syncthreads();                         // the last band's planes are read
     const C *X = reinterpret_cast<const C *>(d.X) + (size_t)b * nb * ldg;
     C *Y = reinterpret_cast<C *>(d.Y) + (size_t)b * nb * ldg;
     const unsigned xrow = (unsigned)(ldg * sizeof(C));               // bytes per coefficient row
@@ -219,7 +226,7 @@ __global__ void __launch_bounds__(T, CTAS) rowspace_kernel(const __grid_constant
                             if (i < nin) cfma(v[i], ph, rs_at<C>(Xa, off));
                     }
                 }
-                if (u == 0 && a0 > ji) rs_cluster_wait();            // the other residues have read this CTA's planes
+                if (u == 0 && !(first && a0 == ji)) rs_cluster_wait();            // the other residues have read this CTA's planes
 #pragma unroll
                 for (int i = 0; i < RR; ++i) dst[i * G::PS] = v[i];
             }
@@ -371,24 +378,21 @@ __global__ void __launch_bounds__(T, CTAS) rowspace_kernel(const __grid_constant
             rs_cluster_arrive();      // waited for before the planes are written again
         }
     }
-    if constexpr (FOLD) rs_cluster_wait();
+    }
+    if (FOLD && rbeg < rend) rs_cluster_wait();
 }
 
 template <typename R, int M1, int M2, int T, int RR, int GR, int CTAS, bool PR, bool FOLD>
-static cudaError_t rs_launch_one(const RsArgs<R> &a, unsigned items, cudaStream_t s) {
-    const void *fn = (const void *)rowspace_kernel<R, M1, M2, T, RR, GR, CTAS, PR, FOLD>;
+static cudaError_t rs_config(unsigned S, unsigned workers, cudaStream_t s, cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at) {
     constexpr size_t smem = RsGeom<R, M1, M2, RR, PR>::smem;
     int dev = 0;
     cudaGetDevice(&dev);
-    cudaError_t e = smem_limit_once(fn, dev, (int)smem);
+    cudaError_t e = smem_limit_once((const void *)rowspace_kernel<R, M1, M2, T, RR, GR, CTAS, PR, FOLD>, dev, (int)smem);
     if (e != cudaSuccess) return e;
-    const unsigned S = (unsigned)(a.s1 * a.s2);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(items * S);
+    cfg.gridDim = dim3(workers * S);
     cfg.blockDim = dim3(T);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at = {};
     if (S > 1) {
         at.id = cudaLaunchAttributeClusterDimension;
         at.val.clusterDim.x = S;
@@ -396,17 +400,42 @@ static cudaError_t rs_launch_one(const RsArgs<R> &a, unsigned items, cudaStream_
         cfg.attrs = &at;
         cfg.numAttrs = 1;
     }
+    return cudaSuccess;
+}
+
+template <typename R, int M1, int M2, int T, int RR, int GR, int CTAS, bool PR, bool FOLD>
+static cudaError_t rs_launch_one(const RsArgs<R> &a, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = {};
+    const cudaError_t e = rs_config<R, M1, M2, T, RR, GR, CTAS, PR, FOLD>((unsigned)(a.s1 * a.s2), (unsigned)a.workers, s, cfg, at);
+    if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, rowspace_kernel<R, M1, M2, T, RR, GR, CTAS, PR, FOLD>, a);
 }
 
 template <typename R, int M1, int M2, int T, int RR, int GR, int CTAS>
-static cudaError_t rs_launch_shape(const RsArgs<R> &a, unsigned items, cudaStream_t s) {
+static cudaError_t rs_launch_shape(const RsArgs<R> &a, cudaStream_t s) {
     if (a.s1 * a.s2 > 1) {
-        if constexpr (M1 * M2 > 256) return rs_launch_one<R, M1, M2, T, RR, GR, CTAS, false, true>(a, items, s);
+        if constexpr (M1 * M2 > 256) return rs_launch_one<R, M1, M2, T, RR, GR, CTAS, false, true>(a, s);
         else return cudaErrorInvalidValue;
     }
-    return a.pruned ? rs_launch_one<R, M1, M2, T, RR, GR, CTAS, true, false>(a, items, s)
-                    : rs_launch_one<R, M1, M2, T, RR, GR, CTAS, false, false>(a, items, s);
+    return a.pruned ? rs_launch_one<R, M1, M2, T, RR, GR, CTAS, true, false>(a, s)
+                    : rs_launch_one<R, M1, M2, T, RR, GR, CTAS, false, false>(a, s);
+}
+
+// (a cluster's CTAs share a GPC, whose SMs need not be a multiple of it)
+template <typename R, int M1, int M2, int T, int RR, int GR, int CTAS>
+static int rs_resident_shape(const RsShape &sh, int num_sms) {
+    const int S = sh.s1 * sh.s2;
+    if constexpr (M1 * M2 > 256) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at = {};
+        int n = 0;
+        if (S > 1 && rs_config<R, M1, M2, T, RR, GR, CTAS, false, true>((unsigned)S, 1, nullptr, cfg, at) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&n, rowspace_kernel<R, M1, M2, T, RR, GR, CTAS, false, true>, &cfg) == cudaSuccess && n > 0)
+            return n;
+        if (S > 1) cudaGetLastError();
+    }
+    return std::max(1, num_sms * CTAS / S);
 }
 
 }  // namespace mb

@@ -23,7 +23,9 @@ template <typename R> struct RsArgs {
     const int4 *src;                  // folded: the up to four G of each plane position (-1: none)
     const typename V2<R>::T *phase;   // folded: [residue][G] exp(2 pi i (c1 n1 / N1 + c2 n2 / N2))
     size_t phase_stride;              // elements from one residue's phases to the next
-    int nbands, nb, nchunks;
+    int nbands, nb;
+    int workers;                      // equal runs of the k-points x bands x nb rows (rs_cut):
+    int num, den, snap;               // num / den rows each, in lowest terms
     int s1, s2;                       // folds of the two grid sides
     int pruned;                       // the tables are those of the 3/4 x 3/4 compact plane
     RsK d[kMaxK];
@@ -40,6 +42,16 @@ struct RsShape {
 };
 constexpr int kMaxRsShapes = 4;
 template <typename R> int rs_shapes(int n1, int n2, int order, RsShape *out, int max);
-template <typename R> cudaError_t rs_launch(const RsArgs<R> &a, const RsShape &sh, unsigned items, cudaStream_t s);
+template <typename R> cudaError_t rs_launch(const RsArgs<R> &a, const RsShape &sh, cudaStream_t s);
+// CTAs (clusters where the grid is folded) of a shape that the device holds at once
+template <typename R> int rs_resident(const RsShape &sh, int num_sms);
+
+// First row of worker w: equal shares of all rows, a share's end moved to the
+// next band boundary where that is at most snap rows away.
+__device__ __forceinline__ int rs_cut(int w, int num, int den, int nb, int snap) {
+    const unsigned long long x = (unsigned long long)w * (unsigned)num;
+    const int r = x >> 32 ? (int)(x / (unsigned)den) : (int)((unsigned)x / (unsigned)den), off = r % nb;
+    return off <= snap ? r - off : nb - off <= snap ? r + nb - off : r;
+}
 
 }  // namespace mb

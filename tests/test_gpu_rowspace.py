@@ -95,6 +95,36 @@ def test_run_lengths_around_a_step(mbmod, n_int, prec):
     _check(mbmod, _workload((16, 16), (4.7, 4.7), 5.0, n_int, 100), prec)
 
 
+@pytest.mark.parametrize("prec,case,nk,nbands", [
+    ("fp32", "16x16-full", 8, 100), ("fp32", "16x32", 4, 100), ("fp32", "32x32-full", 2, 100), ("fp32", "64x16-fold", 2, 100),
+    ("fp32", "64x64-fold", 2, 24), ("fp64", "16x16-full", 2, 100), ("fp64", "32x16-full", 2, 100), ("fp64", "64x32-fold", 2, 50)])
+def test_runs_across_bands(mbmod, prec, case, nk, nbands):
+    """A third more bands than the device holds at once: equal runs that begin
+    and end inside a band, of k-points with different discs.  A row's
+    operations do not depend on the run it is in, so the result is bitwise that
+    of whole bands per run (an explicit target of one run a slot)."""
+    w = _workload(*GRIDS[case], n_int=40, nbands=nbands)
+    w = dataclasses.replace(w, kpts=np.array([[0.03 * i, -0.02 * i * i / nk] for i in range(nk)]))
+    h = mbmod.Handle.from_workload(w)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    Xs = []
+    for ik in range(w.nk):
+        ng, nb, ldg = h.sizes(ik)
+        x = torch.randn(nbands, nb, ldg, dtype=torch.complex128 if prec == "fp64" else torch.complex64, device="cuda", generator=g)
+        x[:, :, ng:] = 0
+        Xs.append(x)
+    out = []
+    for waves in (0, 1):
+        h.plane_kernel_select(w.nk, nbands, prec, -1, waves)
+        Ys = [torch.full_like(x, complex(np.nan, np.nan)) for x in Xs]
+        h.apply_H_batch(list(range(w.nk)), Xs, Ys, prec)
+        out.append(Ys)
+    torch.cuda.synchronize()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+    h.close()
+
+
 @pytest.mark.parametrize("case,n_int,nbands", [(c, 9, 3) for c in GRIDS] + [("16x32", 24, 40), ("64x16-fold", 14, 20)])
 def test_density(mbmod, case, n_int, nbands):
     """The density of random bands on every grid shape, with some bands empty
