@@ -15,13 +15,14 @@
 // tile's nb rows of X arrive in shared memory by TMA bulk copies (one row of
 // CW columns per copy, issued by the lanes of one warp and counted on one
 // mbarrier), so the whole tile is in flight from HBM together.  Each thread
-// then runs the forward and backward banded triangular solves of its column
-// out of shared memory and writes Y directly (consecutive threads,
+// then runs the forward and backward banded triangular solves of one real
+// component of a column out of shared memory and writes Y directly (consecutive threads,
 // consecutive columns: coalesced stores).
 //
 // Every k-point and band of a batch is one launch.
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "apply_common.cuh"
 #include "mb_internal.h"
@@ -59,12 +60,16 @@ template <typename R, int WP> __device__ __forceinline__ void band_row(const R *
     }
 }
 
-// S X for one (k-point, band, 32-column, RT-row) tile, NS threads per column.
+// S X for one (k-point, band, 32-column, RT-row) tile, NS threads per element
+// of a row: a complex column, or in FP64 one real component (an FP64 warp
+// instruction holds its pipe for 64 clocks, so a small problem's tile takes as
+// long as its rows per thread: 16.4 -> 11.1 us for 10 columns of 1.5 k).
 template <typename R, int KK, int NS, int RT>
-__global__ void __launch_bounds__(32 * NS, sizeof(R) == 4 ? 16 : 8)
+__global__ void __launch_bounds__(32 * NS * (sizeof(R) / 4), sizeof(R) == 4 ? 16 : 6)
     band_S_kernel(const __grid_constant__ BandArgs<R> a) {
     typedef typename V2<R>::T R2;
-    constexpr int H = KK - 1, W = 2 * KK - 1, WP = band_pad(KK), RS = RT / NS;
+    constexpr int H = KK - 1, W = 2 * KK - 1, WP = band_pad(KK), RS = RT / NS, CP = sizeof(R) / 4, LN = 32 * CP;
+    typedef typename std::conditional<CP == 1, R2, R>::type E;   // CP elements per column, LN per row of the tile
     static_assert(RT % NS == 0, "whole row runs per thread");
     extern __shared__ __align__(128) unsigned char bsm[];
     __shared__ uint64_t bar;
@@ -103,25 +108,26 @@ __global__ void __launch_bounds__(32 * NS, sizeof(R) == 4 ? 16 : 8)
         const float4 *src = reinterpret_cast<const float4 *>(a.coef + (size_t)r0 * WP);
         float4 *dst = reinterpret_cast<float4 *>(cf);
         const int n16 = (int)((size_t)(r1 - r0) * WP * sizeof(R) / 16);
-        for (int e = threadIdx.x; e < n16; e += 32 * NS) dst[e] = __ldg(src + e);
+        for (int e = threadIdx.x; e < n16; e += LN * NS) dst[e] = __ldg(src + e);
     }
     __syncthreads();
     if (!tc::mbar_wait(&bar, 0, 1ll << 24)) {    // every row of the tile is in shared memory
         if (threadIdx.x == 0) atomicExch(a.err, 1);
         return;
     }
-    const int c = threadIdx.x % 32, seg = threadIdx.x / 32;
+    const int c = threadIdx.x % LN, seg = threadIdx.x / LN;
     const int ja = r0 + seg * RS;                // this thread's rows: ja .. ja + RS - 1 (those < r1)
-    R2 *y = reinterpret_cast<R2 *>(d.Y) + (size_t)b * nb * ldg + g0 + c;
-    if (g0 + c >= d.ng) {                        // padding columns are written as zero
+    const size_t yrow = (size_t)CP * ldg;
+    E *y = reinterpret_cast<E *>(reinterpret_cast<R2 *>(d.Y) + (size_t)b * nb * ldg + g0) + c;
+    if (g0 + c / CP >= d.ng) {                   // padding columns are written as zero
 #pragma unroll
         for (int r = 0; r < RS; ++r)
-            if (ja + r < r1) y[(size_t)(ja + r) * ldg] = czero<R2>();
+            if (ja + r < r1) y[(ja + r) * yrow] = E{};
         return;
     }
-    const R2 *x = buf + c - (size_t)x0 * 32;     // x[row * 32]: rows x0 .. x1 - 1 of the column
-    auto xrow = [&](int row) { return (row >= x0 && row < x1) ? x[(size_t)row * 32] : czero<R2>(); };
-    R2 win[W];                                   // win[i] = X[j - H + i]
+    const E *x = reinterpret_cast<const E *>(buf) + c - (size_t)x0 * LN;     // x[row * LN]: rows x0 .. x1 - 1
+    auto xrow = [&](int row) { return (row >= x0 && row < x1) ? x[(size_t)row * LN] : E{}; };
+    E win[W];                                    // win[i] = X[j - H + i]
 #pragma unroll
     for (int i = 0; i + 1 < W; ++i) win[i + 1] = xrow(ja - H + i);
 #pragma unroll
@@ -133,19 +139,23 @@ __global__ void __launch_bounds__(32 * NS, sizeof(R) == 4 ? 16 : 8)
         if (j < r1) {
             R cj[WP];
             band_row<R, WP>(cf + (size_t)(j - r0) * WP, cj);
-            R2 v = czero<R2>();
+            E v{};
 #pragma unroll
             for (int i = 0; i < W; ++i) rfma(v, cj[i], win[i]);
-            y[(size_t)j * ldg] = v;
+            y[j * yrow] = v;
         }
     }
 }
 
 // S^-1 X for one (k-point, band, CW-column) tile: L y = x (forward), then
 // L^T z = y (backward), L[j][j-dd] at coef[j K + dd] with 1 / L[j][j] at
-// dd = 0; the whole column in shared memory, y overwriting x there.
+// dd = 0; the whole column in shared memory, y overwriting x there.  A thread
+// takes one real component of a column (L is real): shared memory holds three
+// FP64 tiles an SM, and one warp each with both components of 32 columns left
+// an FP64 pipe idle and waited out every row's chain on the others: 128 bands
+// of the slab 221 -> 154 us in FP64 (113 at the pipe's rate).
 template <typename R, int KK, int CW>
-__global__ void __launch_bounds__(CW) band_Sinv_kernel(const __grid_constant__ BandArgs<R> a) {
+__global__ void __launch_bounds__(2 * CW) band_Sinv_kernel(const __grid_constant__ BandArgs<R> a) {
     typedef typename V2<R>::T R2;
     extern __shared__ __align__(128) unsigned char bsm[];
     __shared__ uint64_t bar;
@@ -179,45 +189,45 @@ __global__ void __launch_bounds__(CW) band_Sinv_kernel(const __grid_constant__ B
                 : "memory");
     }
     // the factor's coefficients while the rows are in flight
-    for (int e = threadIdx.x; e < nb * KK; e += CW) cf[e] = a.coef[e];
+    for (int e = threadIdx.x; e < nb * KK; e += 2 * CW) cf[e] = a.coef[e];
     __syncthreads();
     if (!tc::mbar_wait(&bar, 0, 1ll << 24)) {    // every row of the tile is in shared memory
         if (threadIdx.x == 0) atomicExch(a.err, 1);
         return;
     }
-    const int c = threadIdx.x;
-    if (c >= ncol) return;
-    const int g = g0 + c;
-    R2 *y = Y + c;
-    if (g >= d.ng) {                             // padding columns are written as zero
-        for (int j = 0; j < nb; ++j) y[(size_t)j * ldg] = czero<R2>();
+    const int c = threadIdx.x;                   // component c % 2 of column c / 2
+    if (c >= 2 * ncol) return;
+    R *y = reinterpret_cast<R *>(Y) + c;
+    const size_t yrow = 2 * (size_t)ldg;
+    if (g0 + c / 2 >= d.ng) {                    // padding columns are written as zero
+        for (int j = 0; j < nb; ++j) y[j * yrow] = R(0);
         return;
     }
-    R2 *xw = buf + c;
-    R2 w[KK - 1];                                // w[dd-1] = y[j - dd]
+    R *xw = reinterpret_cast<R *>(buf) + c;
+    R w[KK - 1];                                 // w[dd-1] = y[j - dd]
 #pragma unroll
-    for (int i = 0; i < KK - 1; ++i) w[i] = czero<R2>();
+    for (int i = 0; i < KK - 1; ++i) w[i] = R(0);
     for (int j = 0; j < nb; ++j) {
         const R *lj = cf + (size_t)j * KK;
-        R2 s = xw[(size_t)j * CW];
+        R s = xw[(size_t)j * 2 * CW];
         // oldest term first: only the last FMA waits on y[j-1]
 #pragma unroll
         for (int dd = KK - 1; dd >= 1; --dd) rfma(s, -lj[dd], w[dd - 1]);   // w = 0 before row 0
-        const R2 yj = rscale(lj[0], s);
-        xw[(size_t)j * CW] = yj;
+        const R yj = rscale(lj[0], s);
+        xw[(size_t)j * 2 * CW] = yj;
 #pragma unroll
         for (int i = KK - 2; i > 0; --i) w[i] = w[i - 1];
         w[0] = yj;
     }
 #pragma unroll
-    for (int i = 0; i < KK - 1; ++i) w[i] = czero<R2>();
+    for (int i = 0; i < KK - 1; ++i) w[i] = R(0);
     for (int j = nb - 1; j >= 0; --j) {
-        R2 s = xw[(size_t)j * CW];
+        R s = xw[(size_t)j * 2 * CW];
 #pragma unroll
         for (int dd = KK - 1; dd >= 1; --dd)
             if (j + dd < nb) rfma(s, -cf[(size_t)(j + dd) * KK + dd], w[dd - 1]);
-        const R2 zj = rscale(cf[(size_t)j * KK], s);
-        y[(size_t)j * ldg] = zj;
+        const R zj = rscale(cf[(size_t)j * KK], s);
+        y[j * yrow] = zj;
 #pragma unroll
         for (int i = KK - 2; i > 0; --i) w[i] = w[i - 1];
         w[0] = zj;
@@ -273,7 +283,7 @@ static int launch_S(mb_handle *h, int nsel, const int *iks, const void *const *X
     prof_begin(h, s, KN_BANDED, &ev);
     switch (K) {
 #define MB_BAND_S(KK) \
-    case KK: band_S_kernel<R, KK, kBandNS, kBandRT><<<grid, 32 * kBandNS, smem, s>>>(a); break;
+    case KK: band_S_kernel<R, KK, kBandNS, kBandRT><<<grid, 32 * kBandNS * (sizeof(R) / 4), smem, s>>>(a); break;
         MB_BAND_S(3) MB_BAND_S(4) MB_BAND_S(5) MB_BAND_S(6) MB_BAND_S(7) MB_BAND_S(8)
 #undef MB_BAND_S
     }
@@ -295,7 +305,7 @@ static int launch_Sinv(mb_handle *h, int nsel, const int *iks, const void *const
     const dim3 grid((maxldg + kBandCW - 1) / kBandCW, nbands, nsel);
     cudaEvent_t ev;
     prof_begin(h, s, KN_BANDED, &ev);
-    band_Sinv_kernel<R, 6, kBandCW><<<grid, kBandCW, smem, s>>>(a);
+    band_Sinv_kernel<R, 6, kBandCW><<<grid, 2 * kBandCW, smem, s>>>(a);
     prof_end(h, s, KN_BANDED, ev);
     e = cudaGetLastError();
     return e == cudaSuccess ? MB_OK : cuda_fail(h, e);

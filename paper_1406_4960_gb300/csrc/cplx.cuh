@@ -64,5 +64,10 @@ __device__ __forceinline__ void rfma(double2 &acc, double r, double2 a) {
 }
 __device__ __forceinline__ float2 rscale(float r, float2 a) { return make_float2(r * a.x, r * a.y); }
 __device__ __forceinline__ double2 rscale(double r, double2 a) { return make_double2(r * a.x, r * a.y); }
+// the same on one real component (kernels that give each its own thread)
+__device__ __forceinline__ void rfma(float &acc, float r, float a) { acc = fmaf(r, a, acc); }
+__device__ __forceinline__ void rfma(double &acc, double r, double a) { acc = fma(r, a, acc); }
+__device__ __forceinline__ float rscale(float r, float a) { return r * a; }
+__device__ __forceinline__ double rscale(double r, double a) { return r * a; }
 
 }  // namespace mb

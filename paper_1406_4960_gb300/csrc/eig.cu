@@ -724,7 +724,9 @@ __global__ void take_evals_kernel(const double *evals, int M, int nk, double *ep
 }
 
 // Banded solves on vector ranges of every k-point: L L^T y = x, one thread per
-// G column and NV vectors; the last K-1 solution values ride in registers.
+// G column (FP64: per real component of one, since the factors are real and an
+// FP64 warp instruction holds its pipe for 64 clocks: 45 -> 28 us for small
+// problems) and NV vectors; the last K-1 solution values ride in registers.
 // per_g: the k-point's factors L_G[j][d] stored as pfac[(j*K + d)*ldg + G]
 // (coalesced over G); else the G-independent L_z.  F32: on the FP32
 // Gram-Schmidt copies with FP32 factors (a preconditioner solve, whose
@@ -736,29 +738,31 @@ __global__ void take_evals_kernel(const double *evals, int M, int nk, double *ep
 template <int K, bool F32, int NV>
 __global__ void __launch_bounds__(64) eig_banded_solve_kernel(const EigK *ks, const void *Lbv, int per_g, int nb, int src,
                                                               int dst, int nv) {
-    typedef typename std::conditional<F32, float2, double2>::type T2;
     typedef typename std::conditional<F32, float, double>::type T;
+    typedef typename std::conditional<F32, float2, double>::type T2;      // a thread's element: a column, or one component
+    constexpr int CP = F32 ? 1 : 2;                                        // elements per column
     const int nvt = (nv + NV - 1) / NV;
     const int k = blockIdx.z / nvt, v0 = blockIdx.z % nvt * NV, nvl = min(NV, nv - v0);
     const EigK d = ks[k];
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, g = t / CP;
     if (g >= d.ldg) return;
     T2 *vb = F32 ? reinterpret_cast<T2 *>(d.v32) : reinterpret_cast<T2 *>(d.base);
     const T *Lb = reinterpret_cast<const T *>(Lbv);
     const T *pf = F32 ? reinterpret_cast<const T *>(d.pfac32) : reinterpret_cast<const T *>(d.pfac);
-    const int ldg = d.ldg;
+    const int ldg = d.ldg, row = CP * ldg;
+    const long long nvec = CP * d.nvec;
     // vector v of the thread (past the last one: the last one again, not written)
     const T2 *xv[NV];
     T2 *yv[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-        xv[v] = vb + (long long)(src + v0 + min(v, nvl - 1)) * d.nvec + g;
-        yv[v] = vb + (long long)(dst + v0 + min(v, nvl - 1)) * d.nvec + g;
+        xv[v] = vb + (src + v0 + min(v, nvl - 1)) * nvec + t;
+        yv[v] = vb + (dst + v0 + min(v, nvl - 1)) * nvec + t;
     }
     if (g >= d.ng) {
 #pragma unroll
         for (int v = 0; v < NV; ++v)
-            for (int j = 0; j < nb; ++j) yv[v][j * ldg] = czero<T2>();
+            for (int j = 0; j < nb; ++j) yv[v][j * row] = T2{};
         return;
     }
     // factors hold L[j][j-d] for d >= 1 (0 where j < d) and 1 / L[j][j] at
@@ -775,7 +779,7 @@ __global__ void __launch_bounds__(64) eig_banded_solve_kernel(const EigK *ks, co
 #pragma unroll
         for (int v = 0; v < NV; ++v)
 #pragma unroll
-            for (int i = 0; i < K; ++i) win[v][i] = czero<T2>();
+            for (int i = 0; i < K; ++i) win[v][i] = T2{};
     };
     // one row: s - sum_d f_d win_d, the newest solution last (only its FMA waits for the previous row)
     auto solve = [&](int v, T2 s, const T(&f)[K]) {
@@ -794,7 +798,7 @@ __global__ void __launch_bounds__(64) eig_banded_solve_kernel(const EigK *ks, co
 #pragma unroll
             for (int dd = 0; dd < K; ++dd) t.f[u][dd] = fp[o + dd * fd];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) t.x[v][u] = xv[v][j * ldg];
+            for (int v = 0; v < NV; ++v) t.x[v][u] = xv[v][j * row];
         }
     };
     auto load_b = [&](Tile &t, int j1) {
@@ -805,7 +809,7 @@ __global__ void __launch_bounds__(64) eig_banded_solve_kernel(const EigK *ks, co
 #pragma unroll
             for (int dd = 0; dd < K; ++dd) t.f[u][dd] = fp[j + dd < nb ? o + dd * (fr + fd) : o];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) t.x[v][u] = yv[v][j * ldg];
+            for (int v = 0; v < NV; ++v) t.x[v][u] = yv[v][j * row];
         }
     };
     auto run_f = [&](const Tile &t, int j0) {
@@ -815,7 +819,7 @@ __global__ void __launch_bounds__(64) eig_banded_solve_kernel(const EigK *ks, co
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
                 const T2 r = solve(v, t.x[v][u], t.f[u]);
-                if (NV == 1 || v < nvl) yv[v][(j0 + u) * ldg] = r;
+                if (NV == 1 || v < nvl) yv[v][(j0 + u) * row] = r;
             }
         }
     };
@@ -826,7 +830,7 @@ __global__ void __launch_bounds__(64) eig_banded_solve_kernel(const EigK *ks, co
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
                 const T2 r = solve(v, t.x[v][u], t.f[u]);
-                if (NV == 1 || v < nvl) yv[v][(j1 - u) * ldg] = r;
+                if (NV == 1 || v < nvl) yv[v][(j1 - u) * row] = r;
             }
         }
     };
@@ -2092,7 +2096,7 @@ struct Solver {
         // four (two) vectors per thread where that leaves at least 96 threads an SM
         const long long cols = (long long)nk * nv * maxldg;
         const int nvt = !f32 ? 1 : cols >= 4ll * 96 * h->num_sms ? 4 : cols >= 2ll * 96 * h->num_sms ? 2 : 1;
-        const dim3 grid((maxldg + 63) / 64, 1, nk * ((nv + nvt - 1) / nvt));
+        const dim3 grid(((f32 ? 1 : 2) * maxldg + 63) / 64, 1, nk * ((nv + nvt - 1) / nvt));
         switch (h->order) {
 #define MB_BLV(KK, F, NVV)                                                                              \
     MB_LAUNCH_E(KN_BANDED, (eig_banded_solve_kernel<KK, F, NVV><<<grid, 64, 0, s>>>(d_k, Lb, per_g, h->nb, src, dst, nv)))
