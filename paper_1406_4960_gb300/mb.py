@@ -168,6 +168,25 @@ def _stream_ptr(stream):
     return ctypes.c_void_p(int(stream.cuda_stream))
 
 
+def _block_dtype(prec):
+    import torch
+    return torch.complex128 if prec == MB_FP64 else torch.complex64
+
+
+_C_ARRAYS = {}
+
+
+def _c_arrays(n):
+    """The ctypes array types of n ints and n pointers (making a type takes
+    longer than a call)."""
+    t = _C_ARRAYS.get(n)
+    if t is None:
+        t = (ctypes.c_int * n, ctypes.c_void_p * n)
+        if n <= 256:
+            _C_ARRAYS[n] = t
+    return t
+
+
 def _atoms_array(atoms):
     arr = (_Atom * max(1, len(atoms)))()
     for i, at in enumerate(atoms):
@@ -268,6 +287,7 @@ class Handle:
         if rc:
             raise MBError(rc, "mb_setup")
         self._h = h
+        self._block_sizes = {}      # ik -> (nb, ldg): fixed when the handle is created
         self.nk = kp.shape[0]
         self.device = device
         self.grid = (int(grid[0]), int(grid[1]))
@@ -280,6 +300,7 @@ class Handle:
         if getattr(self, "_h", None):
             self._lib.mb_destroy(self._h)
             self._h = None
+            self._block_sizes = {}
 
     def __del__(self):
         try:
@@ -387,16 +408,39 @@ class Handle:
     def _check_block(self, ik, T, prec):
         """Reject tensors whose size, dtype or placement would make the kernels
         read or write outside them."""
-        import torch
-        ng, nb, ldg = self.sizes(ik)
-        want = torch.complex128 if self._prec(prec) == MB_FP64 else torch.complex64
+        return self._block_bands(ik, T, _block_dtype(self._prec(prec)))
+
+    def _block_bands(self, ik, T, want):
+        size = self._block_sizes.get(ik)
+        if size is None:
+            size = self._block_sizes[ik] = self.sizes(ik)[1:]
+        shape = T.shape
+        if (T.dtype is not want or len(shape) != 3 or shape[1] != size[0] or shape[2] != size[1] or not T.is_cuda
+                or T.get_device() != self.device or not T.is_contiguous()):
+            self._reject_block(T, want, *size)
+        return shape[0]
+
+    def _reject_block(self, T, want, nb, ldg):
         if T.dtype != want or not T.is_cuda or not T.is_contiguous():
             raise MBError(1, "block must be a contiguous CUDA %s tensor" % want)
         if T.dim() != 3 or T.shape[1] != nb or T.shape[2] != ldg:
             raise MBError(1, "block shape must be (nbands, %d, %d), got %s" % (nb, ldg, tuple(T.shape)))
-        if T.device.index != self.device:
-            raise MBError(1, "block is on cuda:%s, handle on cuda:%d" % (T.device.index, self.device))
-        return T.shape[0]
+        raise MBError(1, "block is on cuda:%s, handle on cuda:%d" % (T.device.index, self.device))
+
+    def _batch_args(self, iks, Xs, Ys, prec):
+        """The checked arguments of a batched apply: k-points and pointers as C
+        arrays, bands, precision."""
+        n = len(iks)
+        if len(Xs) != n or len(Ys) != n:
+            raise MBError(1, "one X and one Y per k-point")
+        prec = self._prec(prec)
+        want, bands = _block_dtype(prec), self._block_bands
+        for ik, X, Y in zip(iks, Xs, Ys):
+            if bands(ik, X, want) != Xs[0].shape[0] or bands(ik, Y, want) != Xs[0].shape[0]:
+                raise MBError(1, "all blocks need the same band count")
+        int_n, ptr_n = _c_arrays(n)
+        return (n, int_n(*iks), ptr_n(*[x.data_ptr() for x in Xs]), ptr_n(*[y.data_ptr() for y in Ys]),
+                Xs[0].shape[0], prec)
 
     def apply_H(self, ik, X, Y, prec="fp64", stream=None):
         nb = self._check_block(ik, X, prec)
@@ -407,17 +451,8 @@ class Handle:
                                          _stream_ptr(stream)), "mb_apply_H")
 
     def apply_H_batch(self, iks: Sequence[int], Xs, Ys, prec="fp64", stream=None):
-        n = len(iks)
-        if len(Xs) != n or len(Ys) != n:
-            raise MBError(1, "one X and one Y per k-point")
-        for ik, X, Y in zip(iks, Xs, Ys):
-            if self._check_block(ik, X, prec) != Xs[0].shape[0] or self._check_block(ik, Y, prec) != Xs[0].shape[0]:
-                raise MBError(1, "all blocks need the same band count")
-        ik_arr = (ctypes.c_int * n)(*iks)
-        xp = (ctypes.c_void_p * n)(*[x.data_ptr() for x in Xs])
-        yp = (ctypes.c_void_p * n)(*[y.data_ptr() for y in Ys])
-        self._check(self._lib.mb_apply_H_batch(self._h, n, ik_arr, xp, yp, Xs[0].shape[0],
-                                               self._prec(prec), _stream_ptr(stream)), "mb_apply_H_batch")
+        self._check(self._lib.mb_apply_H_batch(self._h, *self._batch_args(iks, Xs, Ys, prec), _stream_ptr(stream)),
+                    "mb_apply_H_batch")
 
     def apply_S(self, ik, X, Y, prec="fp64", stream=None):
         if self._check_block(ik, X, prec) != self._check_block(ik, Y, prec):
@@ -434,16 +469,7 @@ class Handle:
                                             self._prec(prec), _stream_ptr(stream)), "mb_apply_Sinv")
 
     def _banded_batch(self, fn, name, iks, Xs, Ys, prec, stream):
-        n = len(iks)
-        if len(Xs) != n or len(Ys) != n:
-            raise MBError(1, "one X and one Y per k-point")
-        for ik, X, Y in zip(iks, Xs, Ys):
-            if self._check_block(ik, X, prec) != Xs[0].shape[0] or self._check_block(ik, Y, prec) != Xs[0].shape[0]:
-                raise MBError(1, "all blocks need the same band count")
-        ik_arr = (ctypes.c_int * n)(*iks)
-        xp = (ctypes.c_void_p * n)(*[x.data_ptr() for x in Xs])
-        yp = (ctypes.c_void_p * n)(*[y.data_ptr() for y in Ys])
-        self._check(fn(self._h, n, ik_arr, xp, yp, Xs[0].shape[0], self._prec(prec), _stream_ptr(stream)), name)
+        self._check(fn(self._h, *self._batch_args(iks, Xs, Ys, prec), _stream_ptr(stream)), name)
 
     def apply_S_batch(self, iks, Xs, Ys, prec="fp64", stream=None):
         self._banded_batch(self._lib.mb_apply_S_batch, "mb_apply_S_batch", iks, Xs, Ys, prec, stream)
