@@ -910,6 +910,67 @@ __global__ void __launch_bounds__(256) gram_rows_kernel(const EigK *ks, int nch,
     }
 }
 
+// A^H b for one vector b and up to eight rows on the FP32 copies (the
+// Gram-Schmidt products within many chains): every thread of a CTA takes 16
+// bytes of b and of every row at a time, and the sums meet once at the end of
+// the CTA's chunk.  Bound by the read of the vectors.  (gram_rows_kernel's
+// warp per row leaves most warps without one in the first chain steps: 90
+// chains of 115 k elements 136 -> 87 us, 144 of 23 k 45 -> 34 us; for few
+// problems or more rows its smaller chunks are faster, 26 us against 31 for 90
+// rows.)
+constexpr int kGram1Rows = 8;
+__global__ void __launch_bounds__(256) gram1_kernel(const EigK *ks, int nch, VSet A, VSet B, int nsplit, double2 *part) {
+    constexpr int VE = 2, NR = kGram1Rows;                // elements per load (nvec is a multiple of 32)
+    struct __align__(16) Pack { float2 v[VE]; };
+    const int split = blockIdx.x, prob = blockIdx.y;
+    const int k = prob / nch, ch = prob % nch;
+    const EigK d = ks[k];
+    const int ma = A.count();
+    const long long np = d.nvec / VE;
+    const long long t0 = split * np / nsplit, t1 = (split + 1) * np / nsplit;
+    const Pack *b = reinterpret_cast<const Pack *>(d.v32 + (long long)B.at(0, ch) * d.nvec);
+    const Pack *a[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) a[r] = reinterpret_cast<const Pack *>(d.v32 + (long long)A.at(min(r, ma - 1), ch) * d.nvec);
+    float sx[NR], sy[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) sx[r] = sy[r] = 0.f;
+#pragma unroll 2
+    for (long long t = t0 + threadIdx.x; t < t1; t += 256) {
+        Pack av[NR];
+        const Pack bv = b[t];
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            if (r < ma) av[r] = a[r][t];
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            if (r < ma)
+#pragma unroll
+                for (int u = 0; u < VE; ++u) {
+                    sx[r] = fma(av[r].v[u].x, bv.v[u].x, fma(av[r].v[u].y, bv.v[u].y, sx[r]));
+                    sy[r] = fma(av[r].v[u].x, bv.v[u].y, fma(-av[r].v[u].y, bv.v[u].x, sy[r]));
+                }
+    }
+    __shared__ double2 red[8][NR];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        if (r >= ma) break;
+        float x = sx[r], y = sy[r];
+        for (int off = 16; off > 0; off >>= 1) {
+            x += __shfl_down_sync(0xffffffffu, x, off);
+            y += __shfl_down_sync(0xffffffffu, y, off);
+        }
+        if (lane == 0) red[warp][r] = make_double2(x, y);
+    }
+    __syncthreads();
+    if (threadIdx.x < ma) {
+        double2 s = red[0][threadIdx.x];
+        for (int w = 1; w < 8; ++w) s = s + red[w][threadIdx.x];
+        part[((size_t)prob * nsplit + split) * ma + threadIdx.x] = s;
+    }
+}
+
 // A^H B on the FP32 copies for products wider than the tensor-core kernel's
 // tile: a CTA takes one chunk of the vector length for a 96 x 96 tile of the
 // product, 6 x 6 complex outputs per thread (rows ti + 16 i, columns tj + 16 j:
@@ -1469,30 +1530,24 @@ __global__ void __launch_bounds__(kCombThreads) combine2_kernel(const EigK *ks, 
 }
 
 // The same for many columns of the FP32 copies, as a matrix product in tiles
-// of 128 elements x 16 RJ columns: 8 x RJ complex outputs per thread (elements
+// of 128 elements x 48 columns: 8 x 3 complex outputs per thread (elements
 // tx + 16 i, columns ty + 16 j), A staged KC vectors at a time by cp.async,
 // so that every element of A is read once for all its columns.  Yf: the
 // coefficients in FP32 (to_float_kernel; FP64 conversions run at the FP64
 // rate and would cost every CTA a quarter of its time).  Bound by the FMA
-// pipe: 90 x 90 over 115 k elements 341 -> 188 us, four problems of 36 x 36
-// over 23 k 54 -> 39 us against combine2_kernel's 12 columns per CTA.
-constexpr int CT_T = 128, CT_KC = 8;
-template <int RJ> constexpr size_t combine_tile_smem() {
-    return (size_t)2 * CT_KC * (CT_T + 16 * RJ) * sizeof(float2);
-}
-template <int RJ>
-__global__ void __launch_bounds__(256, RJ > 3 ? 1 : 2) combine_tile_kernel(const EigK *ks, int nch, VSet A, VSet C,
-                                                                          const float2 *Yf, float alpha, float beta) {
-    extern __shared__ __align__(16) unsigned char ctsm[];
-    typedef float2 StageA[CT_KC][CT_T];
-    typedef float2 StageY[CT_KC][16 * RJ];
-    StageA *As = reinterpret_cast<StageA *>(ctsm);                 // two buffers each
-    StageY *Ys = reinterpret_cast<StageY *>(As + 2);
+// pipe: 90 x 90 over 115 k elements 341 -> 173 us, four problems of 36 x 36
+// over 23 k 54 -> 39 us against combine2_kernel's 12 columns per CTA.  (96
+// columns and one CTA an SM: 188 us.)
+constexpr int CT_T = 128, CT_KC = 8, CT_RJ = 3, CT_C = 16 * CT_RJ;
+__global__ void __launch_bounds__(256, 2) combine_tile_kernel(const EigK *ks, int nch, VSet A, VSet C, const float2 *Yf,
+                                                              float alpha, float beta) {
+    constexpr int RJ = CT_RJ;
+    __shared__ __align__(16) float2 As[2][CT_KC][CT_T], Ys[2][CT_KC][CT_C];
     const int ma = A.count(), mc = C.count(), prob = blockIdx.y, tid = threadIdx.x;
     const int k = prob / nch, ch = prob % nch;
     const EigK d = ks[k];
-    const int j0 = tile_col(mc, 16 * RJ);
-    const long long t0 = tile_elem(mc, 16 * RJ, CT_T);
+    const int j0 = tile_col(mc, CT_C);
+    const long long t0 = tile_elem(mc, CT_C, CT_T);
     if (t0 >= d.nvec) return;                                      // the batch's longest vectors size the grid
     const int nt = (int)min((long long)CT_T, d.nvec - t0);         // a multiple of 32
     const float2 *y = Yf + (size_t)prob * LD * LD;
@@ -1508,8 +1563,8 @@ __global__ void __launch_bounds__(256, RJ > 3 ? 1 : 2) combine_tile_kernel(const
                          : "memory");
         }
 #pragma unroll
-        for (int e = tid; e < CT_KC * 16 * RJ; e += 256) {
-            const int q = e / (16 * RJ), j = e % (16 * RJ);
+        for (int e = tid; e < CT_KC * CT_C; e += 256) {
+            const int q = e / CT_C, j = e % CT_C;
             const bool in = i0 + q < ma && j0 + j < mc;
             asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(tc::smem_u32(&Ys[buf][q][j])),
                          "l"(y + (in ? (i0 + q) * LD + j0 + j : 0)), "r"(in ? 8 : 0)
@@ -1903,6 +1958,17 @@ struct Solver {
     // vectors in the same order), only j <= i is computed
     void gram(int nch, VSet A, VSet B, double2 *G, bool f32 = false, bool lower = false) {
         const int mbc = B.count();
+        if (f32 && mbc == 1 && A.count() <= kGram1Rows && nk * nch >= 32) {
+            // chunks of at least 512 loads, eight CTAs per SM over the grid
+            const int ma = A.count(), np = nk * nch;
+            int nsplit = std::max(1, std::min(512, (8 * h->num_sms + np - 1) / np));
+            nsplit = (int)std::min<long long>(nsplit, std::max<long long>(1, nmax / 1024));
+            while ((size_t)np * nsplit * ma > part_cap && nsplit > 1) --nsplit;
+            MB_LAUNCH_E(KN_GRAM32, gram1_kernel<<<dim3(nsplit, np), 256, 0, s>>>(d_k, nch, A, B, nsplit, d_part));
+            MB_LAUNCH_E(KN_GRAM32,
+                        gram_reduce_kernel<<<dim3((ma + 7) / 8, np), 256, 0, s>>>(d_part, nsplit, ma, 1, G, lower ? 1 : 0));
+            return;
+        }
         // narrowest column group that covers mbc in the fewest slots
         static const int widths[] = {1, 2, 3, 4, 5, 6, 7, 8, 12, 16};
         int gj = 16;
@@ -1992,20 +2058,10 @@ struct Solver {
             return;
         }
         if (F32 && mc > 8) {
-            // one column tile where 48 or 96 columns hold them all, else the
-            // width with less padding
-            const int np = nk * nch, w48 = (mc + 47) / 48 * 48, w96 = (mc + 95) / 96 * 96;
-            const float fa = (float)alpha, fb = (float)beta;
+            const int np = nk * nch;
             MB_LAUNCH_E(KN_COMBINE32, to_float_kernel<<<dim3((A.count() * mc + 127) / 128, np), 128, 0, s>>>(Y, d_Yf, A.count(), mc));
-            if (w48 < w96) {
-                cuda(smem_limit_once((const void *)combine_tile_kernel<3>, h->device, h->smem_optin));
-                MB_LAUNCH_E(KN_COMBINE32, (combine_tile_kernel<3><<<dim3(tile_grid(nmax, CT_T, mc, 48), np), 256, combine_tile_smem<3>(), s>>>(
-                                              d_k, nch, A, C, d_Yf, fa, fb)));
-            } else {
-                cuda(smem_limit_once((const void *)combine_tile_kernel<6>, h->device, h->smem_optin));
-                MB_LAUNCH_E(KN_COMBINE32, (combine_tile_kernel<6><<<dim3(tile_grid(nmax, CT_T, mc, 96), np), 256, combine_tile_smem<6>(), s>>>(
-                                              d_k, nch, A, C, d_Yf, fa, fb)));
-            }
+            MB_LAUNCH_E(KN_COMBINE32, combine_tile_kernel<<<dim3(tile_grid(nmax, CT_T, mc, CT_C), np), 256, 0, s>>>(
+                                          d_k, nch, A, C, d_Yf, (float)alpha, (float)beta));
             return;
         }
         // the widest column group (least re-reading of A) among those with the

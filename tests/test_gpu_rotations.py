@@ -1,5 +1,5 @@
 """The eigensolver's tiled vector kernels at the edges of their tiles: the FP32
-and float-float rotations (48 and 96 columns per tile, one or two tiles), the
+and float-float rotations (one, two and three tiles of 48 columns), the
 S-Gram inverse and the small Rayleigh-Ritz problem (FP32 sweeps, and FP64 ones
 from a refined FP32 result) at odd and large numbers of roots, and the float-float kernel's element and column remainders.
 
