@@ -827,6 +827,7 @@ struct PlanePlan {
     int nchunks = 1;       // radix-2 kernel: runs of knot intervals
     int workers = 1;       // row-space kernel: equal runs of all bands' rows,
     int snap = 0;          // their ends moved to a band boundary this near
+    bool small = false;    // or a cluster of CTAs per band
     size_t smem = 0;
 };
 
@@ -884,6 +885,10 @@ static PlanePlan plan_plane(const mb_handle *h, int nsel, const int *iks, int nb
             return 0.35 * in + 0.65 * L + 2.0 * steps;
         }, &best);
         p.workers = pairs * nchunks;
+        if (c2 == 16 && waves == 0 && rs_small_supported(p.sh, pairs, h->nb, h->num_sms)) {
+            p.small = true;
+            return p;
+        }
         // Runs that do not end with a band, one for every slot: no last round
         // that is nearly empty, for two halos and about two steps more a
         // worker.  FP32: a plan costs between its longest slot and its mean
@@ -1231,7 +1236,10 @@ static int apply_H_launch(mb_handle *h, int nsel, const int *iks, const void *co
             d.gofs = h->kofs[ik];
         }
         cudaError_t e = cudaSuccess;
-        MB_LAUNCH(h, s, KN_PLANE, e = rs_launch<R>(ra, plan.sh, s));
+        if constexpr (sizeof(R) == 8) {
+            if (plan.small) MB_LAUNCH(h, s, KN_PLANE, e = rs_launch_small(ra, (unsigned)(nsel * nbands), s));
+        }
+        if (!plan.small) MB_LAUNCH(h, s, KN_PLANE, e = rs_launch<R>(ra, plan.sh, s));
         MB_CUDA(e);
     } else {
         PlaneArgs<R> pa;
@@ -1268,9 +1276,12 @@ static int apply_H_launch(mb_handle *h, int nsel, const int *iks, const void *co
     ea.nchunks = nchunks;
     ea.nint = h->nint;
     ea.nz = h->nzf;
-    // rows per epilogue thread: at most 8 (FP32) / 4 (FP64), all loaded at once
+    // rows per epilogue thread, all loaded at once: 8 (FP32) or 4 (FP64), one
+    // where four would leave a quarter of the FP64 pipes without a warp (an
+    // FP64 warp instruction holds its pipe for 64 clocks: a row's 41 take 1.3 us)
     constexpr int ERM = sizeof(R) == 4 ? 8 : 4;
-    const int ejseg = (h->nb + ERM - 1) / ERM;
+    const bool short_runs = sizeof(R) == 8 && (cols / 32) * ((h->nb + ERM - 1) / ERM) < 3ll * h->num_sms;
+    const int erm = short_runs ? 1 : ERM, ejseg = (h->nb + erm - 1) / erm;
     ea.njseg = ejseg;
     // where each row's local part lives: run boundary bc (between runs bc and
     // bc+1) starts at interval t1 and owns rows [t1 - 1, t1 + K - 3]
@@ -1295,11 +1306,21 @@ static int apply_H_launch(mb_handle *h, int nsel, const int *iks, const void *co
         const int HWn = h->order <= 6 ? 5 : 7;
         const int nfp = ea.f1 - ea.f0;
         const int nzb = nfp <= 4 ? 4 : nfp <= 8 ? 8 : nfp <= 12 ? 12 : 16;
-        const size_t esm = ((size_t)2 * ERM * ((2 * HWn + 1 + 3) / 4 * 4) + (size_t)ERM * nzb) * sizeof(R);
-#define MB_EPI(NZ, HWV)                                                                                        \
-    do {                                                                                                       \
-        MB_CUDA(smem_limit_once((const void *)epilogue_kernel<R, NZ, HWV, ERM>, h->device, h->smem_optin));  \
-        MB_LAUNCH(h, s, KN_EPILOGUE, (epilogue_kernel<R, NZ, HWV, ERM><<<ge, 64, esm, s>>>(ea)));            \
+        const size_t esm = ((size_t)2 * erm * ((2 * HWn + 1 + 3) / 4 * 4) + (size_t)erm * nzb) * sizeof(R);
+        auto go = [&](auto kern) -> int {
+            MB_CUDA(smem_limit_once((const void *)kern, h->device, h->smem_optin));
+            MB_LAUNCH(h, s, KN_EPILOGUE, (kern<<<ge, 64, esm, s>>>(ea)));
+            return MB_OK;
+        };
+        int rc = MB_OK;
+#define MB_EPI(NZ, HWV)                                                             \
+    do {                                                                            \
+        if constexpr (sizeof(R) == 8)                                               \
+            if (short_runs) {                                                       \
+                rc = go(epilogue_kernel<R, NZ, HWV, 1>);                            \
+                break;                                                              \
+            }                                                                       \
+        rc = go(epilogue_kernel<R, NZ, HWV, ERM>);                                  \
     } while (0)
         if (HWn == 5) {
             if (nzb == 4) MB_EPI(4, 5);
@@ -1313,6 +1334,7 @@ static int apply_H_launch(mb_handle *h, int nsel, const int *iks, const void *co
             else MB_EPI(16, 7);
         }
 #undef MB_EPI
+        if (rc) return rc;
     }
     if (h->nterm > 0 && tensor) {
         cudaError_t e = cudaSuccess;

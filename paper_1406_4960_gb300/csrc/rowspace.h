@@ -46,6 +46,12 @@ template <typename R> cudaError_t rs_launch(const RsArgs<R> &a, const RsShape &s
 // CTAs (clusters where the grid is folded) of a shape that the device holds at once
 template <typename R> int rs_resident(const RsShape &sh, int num_sms);
 
+// Small FP64 problems: a cluster of kRsSmallCl CTAs per (k-point, band), at most
+// kRsSmallRows rows each (rowspace64.cu), where every one has an SM to itself.
+constexpr int kRsSmallCl = 8, kRsSmallRows = 8;
+bool rs_small_supported(const RsShape &sh, int pairs, int nb, int num_sms);
+cudaError_t rs_launch_small(const RsArgs<double> &a, unsigned pairs, cudaStream_t s);
+
 // First row of worker w: equal shares of all rows, a share's end moved to the
 // next band boundary where that is at most snap rows away.
 __device__ __forceinline__ int rs_cut(int w, int num, int den, int nb, int snap) {

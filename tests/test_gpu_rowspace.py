@@ -95,6 +95,15 @@ def test_run_lengths_around_a_step(mbmod, n_int, prec):
     _check(mbmod, _workload((16, 16), (4.7, 4.7), 5.0, n_int, 100), prec)
 
 
+@pytest.mark.parametrize("case", ["16x16", "16x16-full"])
+@pytest.mark.parametrize("n_int,nbands", [(6, 2), (7, 1), (13, 9), (38, 9), (60, 9), (61, 9), (62, 9), (38, 10)])
+def test_small_fp64_clusters(mbmod, case, n_int, nbands):
+    """One cluster of CTAs per band: one or two rows a CTA (9 splines) up to eight (64),
+    and the sizes just outside (65 splines, 20 bands of two k-points)."""
+    grid = {"16x16": ((16, 16), (4.7, 4.7), 12.0), "16x16-full": GRIDS["16x16-full"]}[case]
+    _check(mbmod, _workload(*grid, n_int=n_int, nbands=nbands), "fp64")
+
+
 @pytest.mark.parametrize("prec,case,nk,nbands", [
     ("fp32", "16x16-full", 8, 100), ("fp32", "16x32", 4, 100), ("fp32", "32x32-full", 2, 100), ("fp32", "64x16-fold", 2, 100),
     ("fp32", "64x64-fold", 2, 24), ("fp64", "16x16-full", 2, 100), ("fp64", "32x16-full", 2, 100), ("fp64", "64x32-fold", 2, 50)])
