@@ -15,9 +15,9 @@
 // tile's nb rows of X arrive in shared memory by TMA bulk copies (one row of
 // CW columns per copy, issued by the lanes of one warp and counted on one
 // mbarrier), so the whole tile is in flight from HBM together.  Each thread
-// then runs the forward and backward banded triangular solves of one real
-// component of a column out of shared memory and writes Y directly (consecutive threads,
-// consecutive columns: coalesced stores).
+// then runs the forward and backward banded triangular solves of its column
+// (FP64: of one real component of it) out of shared memory and writes Y
+// directly (consecutive threads, consecutive columns: coalesced stores).
 //
 // Every k-point and band of a batch is one launch.
 #include <algorithm>
@@ -149,14 +149,17 @@ __global__ void __launch_bounds__(32 * NS * (sizeof(R) / 4), sizeof(R) == 4 ? 16
 
 // S^-1 X for one (k-point, band, CW-column) tile: L y = x (forward), then
 // L^T z = y (backward), L[j][j-dd] at coef[j K + dd] with 1 / L[j][j] at
-// dd = 0; the whole column in shared memory, y overwriting x there.  A thread
-// takes one real component of a column (L is real): shared memory holds three
-// FP64 tiles an SM, and one warp each with both components of 32 columns left
+// dd = 0; the whole column in shared memory, y overwriting x there.  In FP64 a
+// thread takes one real component of a column (L is real): shared memory holds
+// three tiles an SM, and one warp each with both components of 32 columns left
 // an FP64 pipe idle and waited out every row's chain on the others: 128 bands
-// of the slab 221 -> 154 us in FP64 (113 at the pipe's rate).
+// of the slab 221 -> 154 us (113 at the pipe's rate).  In FP32, bound by
+// latency and the shared-memory accesses, that is slower (23.2 us for 21.8).
 template <typename R, int KK, int CW>
-__global__ void __launch_bounds__(2 * CW) band_Sinv_kernel(const __grid_constant__ BandArgs<R> a) {
+__global__ void __launch_bounds__(CW * (sizeof(R) / 4)) band_Sinv_kernel(const __grid_constant__ BandArgs<R> a) {
     typedef typename V2<R>::T R2;
+    constexpr int CP = sizeof(R) / 4, LN = CP * CW;
+    typedef typename std::conditional<CP == 1, R2, R>::type E;   // CP elements per column, LN per row of the tile
     extern __shared__ __align__(128) unsigned char bsm[];
     __shared__ uint64_t bar;
     const BandK &d = a.d[blockIdx.z];
@@ -189,44 +192,44 @@ __global__ void __launch_bounds__(2 * CW) band_Sinv_kernel(const __grid_constant
                 : "memory");
     }
     // the factor's coefficients while the rows are in flight
-    for (int e = threadIdx.x; e < nb * KK; e += 2 * CW) cf[e] = a.coef[e];
+    for (int e = threadIdx.x; e < nb * KK; e += LN) cf[e] = a.coef[e];
     __syncthreads();
     if (!tc::mbar_wait(&bar, 0, 1ll << 24)) {    // every row of the tile is in shared memory
         if (threadIdx.x == 0) atomicExch(a.err, 1);
         return;
     }
-    const int c = threadIdx.x;                   // component c % 2 of column c / 2
-    if (c >= 2 * ncol) return;
-    R *y = reinterpret_cast<R *>(Y) + c;
-    const size_t yrow = 2 * (size_t)ldg;
-    if (g0 + c / 2 >= d.ng) {                    // padding columns are written as zero
-        for (int j = 0; j < nb; ++j) y[j * yrow] = R(0);
+    const int c = threadIdx.x;                   // element c % CP of column c / CP
+    if (c >= CP * ncol) return;
+    E *y = reinterpret_cast<E *>(Y) + c;
+    const size_t yrow = CP * (size_t)ldg;
+    if (g0 + c / CP >= d.ng) {                   // padding columns are written as zero
+        for (int j = 0; j < nb; ++j) y[j * yrow] = E{};
         return;
     }
-    R *xw = reinterpret_cast<R *>(buf) + c;
-    R w[KK - 1];                                 // w[dd-1] = y[j - dd]
+    E *xw = reinterpret_cast<E *>(buf) + c;
+    E w[KK - 1];                                 // w[dd-1] = y[j - dd]
 #pragma unroll
-    for (int i = 0; i < KK - 1; ++i) w[i] = R(0);
+    for (int i = 0; i < KK - 1; ++i) w[i] = E{};
     for (int j = 0; j < nb; ++j) {
         const R *lj = cf + (size_t)j * KK;
-        R s = xw[(size_t)j * 2 * CW];
+        E s = xw[(size_t)j * LN];
         // oldest term first: only the last FMA waits on y[j-1]
 #pragma unroll
         for (int dd = KK - 1; dd >= 1; --dd) rfma(s, -lj[dd], w[dd - 1]);   // w = 0 before row 0
-        const R yj = rscale(lj[0], s);
-        xw[(size_t)j * 2 * CW] = yj;
+        const E yj = rscale(lj[0], s);
+        xw[(size_t)j * LN] = yj;
 #pragma unroll
         for (int i = KK - 2; i > 0; --i) w[i] = w[i - 1];
         w[0] = yj;
     }
 #pragma unroll
-    for (int i = 0; i < KK - 1; ++i) w[i] = R(0);
+    for (int i = 0; i < KK - 1; ++i) w[i] = E{};
     for (int j = nb - 1; j >= 0; --j) {
-        R s = xw[(size_t)j * 2 * CW];
+        E s = xw[(size_t)j * LN];
 #pragma unroll
         for (int dd = KK - 1; dd >= 1; --dd)
             if (j + dd < nb) rfma(s, -cf[(size_t)(j + dd) * KK + dd], w[dd - 1]);
-        const R zj = rscale(cf[(size_t)j * KK], s);
+        const E zj = rscale(cf[(size_t)j * KK], s);
         y[j * yrow] = zj;
 #pragma unroll
         for (int i = KK - 2; i > 0; --i) w[i] = w[i - 1];
@@ -305,7 +308,7 @@ static int launch_Sinv(mb_handle *h, int nsel, const int *iks, const void *const
     const dim3 grid((maxldg + kBandCW - 1) / kBandCW, nbands, nsel);
     cudaEvent_t ev;
     prof_begin(h, s, KN_BANDED, &ev);
-    band_Sinv_kernel<R, 6, kBandCW><<<grid, 2 * kBandCW, smem, s>>>(a);
+    band_Sinv_kernel<R, 6, kBandCW><<<grid, kBandCW * (sizeof(R) / 4), smem, s>>>(a);
     prof_end(h, s, KN_BANDED, ev);
     e = cudaGetLastError();
     return e == cudaSuccess ? MB_OK : cuda_fail(h, e);
