@@ -370,16 +370,16 @@ def scf_workload(W):
     return W.with_core(W.slab(), SCF_Z, SCF_RCORE, name="slab-scf")
 
 
-def density_flops(h, w, nbands):
-    """Algorithmic flops of one density: per (k, band, plane) the B-spline
-    evaluation (4 kappa ng), one inverse FFT (5 N log2 N) and f |psi|^2 (4 N)."""
-    N = w.grid[0] * w.grid[1]
+def density_flops(h, w, nocc):
+    """FP64 flops of one density call through row space: per occupied band and
+    B-spline row an inverse 2D FFT (5 N log2 N) and, per grid point, the six
+    products f Re(conj x_i x_j) with the rows within the band's width (28), then
+    per Gauss plane the 21 products of B values (42)."""
+    n1, n2 = w.grid
+    N = n1 * n2
     zq, _ = h.zplanes()
-    tot = 0.0
-    for ik in range(w.nk):
-        ng = h.sizes(ik)[0]
-        tot += nbands * len(zq) * (4 * w.order * ng + 5 * N * math.log2(N) + 4 * N)
-    return tot
+    rows = sum(h.sizes(ik)[1] for ik in range(w.nk)) * nocc
+    return rows * (5 * N * math.log2(N) + 28 * N) + len(zq) * N * 42
 
 
 def scf_steps(mb, h, w, local):
@@ -414,7 +414,7 @@ def scf_steps(mb, h, w, local):
         e1.record(st)
         torch.cuda.synchronize(local)
         ms[name] = e0.elapsed_time(e1) / reps
-    fl = density_flops(h, w, w.nbands)
+    fl = density_flops(h, w, int((occ[0] != 0).sum()))
     peak64 = probe_fp64_peak(mb.load(), local)
     ach = fl / (ms["density"] * 1e-3) / 1e12
     roof = {"bound": "alu", "achieved": ach, "peak": peak64, "unit": "TFLOP/s",
