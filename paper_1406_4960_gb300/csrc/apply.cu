@@ -1703,7 +1703,7 @@ int plane_kernel_name(const mb_handle *h, int nk, int nbands, int prec, char *bu
     const size_t c2 = prec == MB_FP64 ? 16 : 8;
     const PlanePlan p = plan_plane(h, nk, iks.data(), nbands, c2);
     char tmp[128];
-    if (p.rs) std::snprintf(tmp, sizeof(tmp), "%s", p.sh.name);
+    if (p.rs) std::snprintf(tmp, sizeof(tmp), "%s", p.small ? "rowspace_small_kernel" : p.sh.name);
     else std::snprintf(tmp, sizeof(tmp), "plane_kernel<%s>", c2 == 8 ? "float" : "double");
     std::snprintf(buf, (size_t)len, "%s", tmp);
     return MB_OK;

@@ -55,7 +55,7 @@ def _workload(grid, sides, ecut, n_int, nbands):
                                breaks=W.uniform_breaks(-4.0, 4.0, n_int), nbands=nbands, name="rowspace")
 
 
-def _check(mbmod, w, prec, waves=(0,)):
+def _check(mbmod, w, prec, waves=(0,), kernel="rowspace_"):
     h = mbmod.Handle.from_workload(w)
     cdt = np.complex128 if prec == "fp64" else np.complex64
     Xs, perms, refs = [], [], []
@@ -68,7 +68,7 @@ def _check(mbmod, w, prec, waves=(0,)):
         Xs.append(torch.from_numpy(lib_block(X, perms[ik], ldg, cdt)).cuda())
     for wv in waves:
         h.plane_kernel_select(w.nk, w.nbands, prec, -1, wv)
-        assert h.plane_kernel_name(w.nk, w.nbands, prec).startswith("rowspace_kernel")
+        assert h.plane_kernel_name(w.nk, w.nbands, prec).startswith(kernel)
         Ys = [torch.full_like(x, complex(np.nan, np.nan)) for x in Xs]
         h.apply_H_batch(list(range(w.nk)), Xs, Ys, prec)
         torch.cuda.synchronize()
@@ -101,7 +101,9 @@ def test_small_fp64_clusters(mbmod, case, n_int, nbands):
     """One cluster of CTAs per band: one or two rows a CTA (9 splines) up to eight (64),
     and the sizes just outside (65 splines, 20 bands of two k-points)."""
     grid = {"16x16": ((16, 16), (4.7, 4.7), 12.0), "16x16-full": GRIDS["16x16-full"]}[case]
-    _check(mbmod, _workload(*grid, n_int=n_int, nbands=nbands), "fp64")
+    small = n_int + 3 <= 64 and 2 * nbands * 8 <= 152
+    _check(mbmod, _workload(*grid, n_int=n_int, nbands=nbands), "fp64",
+           kernel="rowspace_small_kernel" if small else "rowspace_kernel")
 
 
 @pytest.mark.parametrize("prec,case,nk,nbands", [
