@@ -158,7 +158,8 @@ __global__ void __launch_bounds__(T, CTAS) density_rows_kernel(const __grid_cons
 // rho of one knot interval's planes at one grid point: the band of P that the
 // interval's kappa splines touch, summed over the parts in order, then the
 // quadratic form at every Gauss point.  clamp: occupations are >= 0, and so
-// is rho (rounding may leave -1e-17 of the largest product where it vanishes).
+// is rho (rounding may leave -1e-17 of the largest product where it vanishes);
+// NaN and infinite sums stay what they are.
 __global__ void __launch_bounds__(128) density_planes_kernel(const double *part, int nparts, int nb, int nint, int nquad,
                                                              int N1, int N2, int s1, int s2, const double *Bq,
                                                              double scale, int clamp, double *rho) {
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(128) density_planes_kernel(const double *part,
             s = fma(B[u], w, s);
         }
         s *= scale;
-        rho[(size_t)q * NN + r] = clamp ? fmax(s, 0.0) : s;
+        rho[(size_t)q * NN + r] = clamp && s < 0.0 && !isinf(s) ? 0.0 : s;
     }
 }
 
