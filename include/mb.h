@@ -253,7 +253,8 @@ typedef struct {
 } mb_solve_opts;
 
 /* Lowest `nbands` roots of H c = eps S c at every k-point (§II.C).
- *   prec   MB_FP64: every step in double ("plain").  MB_FP32 / MB_BF16:
+ *   prec   MB_FP64: every step in double ("plain"; the small dense problems
+ *          start from FP32 sweeps and are refined to double).  MB_FP32 / MB_BF16:
  *          bulk cycles with every vector step in FP32 (applies in that
  *          precision, Gram products on the tensor cores, small dense
  *          problems in FP32 or FP64), then finish cycles with FP64 roots

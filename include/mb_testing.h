@@ -3,6 +3,7 @@
  * building block of the library on its own. */
 #ifndef MB_TESTING_H
 #define MB_TESTING_H
+#include "mb.h"
 #ifdef __cplusplus
 extern "C" {
 #endif
@@ -31,6 +32,15 @@ int mb_debug_gram_tc32(const void *V, long long n, int ma, int mb, int nsplit, d
  * mc vectors of n elements, overwritten.  1 <= ma <= 112, 1 <= mc <= 128.
  * Allocates and frees its own device buffers; MB_EINVAL for bad sizes. */
 int mb_debug_combine_ff(const void *A, const double *Y, long long n, int ma, int mc, void *C, void *stream);
+
+/* The eigensolver's Rayleigh-Ritz problems: eigenpairs of nprob Hermitian
+ * m x m matrices A (host, row-major interleaved doubles, one after another;
+ * the lower triangles are read) on the handle's device.  refined: as a solve
+ * treats its FP64 problems; 0: Jacobi sweeps in FP64 alone.  evals: host,
+ * nprob x m, ascending; Y: host, nprob x m x m complex, column i of a problem
+ * the vector of its value i.  1 <= m <= 112, 1 <= nprob <= 4096.  Allocates
+ * and frees its own device buffers; MB_EINVAL for bad sizes. */
+int mb_debug_rayleigh_ritz(mb_handle *h, const double *A, int m, int nprob, int refined, double *evals, double *Y);
 
 /* FP32 fused multiply-add throughput of `device` in TFLOP/s (2 flops per
  * FFMA): eight independent FFMA chains per thread, 2048 threads on every SM,

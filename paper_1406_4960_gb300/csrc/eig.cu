@@ -547,16 +547,20 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double2 *G
     }
 }
 
-// FP64 result from FP32 sweeps: X0 of the FP32 sweeps is refined by two steps
+// FP64 result from FP32 sweeps: X0 of the FP32 sweeps is refined by steps
 // of the Ogita-Aishima iteration (Iterative refinement for symmetric
 // eigenvalue decomposition, Japan J. Indust. Appl. Math. 35, 2018): with
 // S = X^H A X, P = X^H X, R = I - P and l_i = S_ii / P_ii,
 //   X <- X + X E,  E_ij = (S_ij + l_j R_ij) / (l_j - l_i),  E_ii = R_ii / 2,
 // which squares the error of the vectors and of their orthogonality.  Where
 // that E_ij is above lim (neighbours that FP32 does not separate), R_ij / 2
-// only makes the two orthogonal and the FP64 sweeps on X^H A X rotate them.
-// lim^2 is the loss of orthogonality the next step (or FP64) must absorb:
-// 1e-4 in the first step, 1e-8 in the second.
+// only makes the two orthogonal and the FP64 sweeps on X^H A X rotate them.  A
+// step leaves I - P = E^H E + O(R^2), at most (m lim)^2 where all corrections
+// are at lim and in phase: 1.3e-4 after the first step with lim = 1e-4, 1e-8
+// after the second with 1e-8, and 1e-16 after a third that only
+// orthonormalizes, E = R / 2 (without it, a cluster coupled at 1e-4 of its gaps
+// lost 2e-11 of 95 vectors' orthonormality, which the FP64 sweeps, unitary
+// themselves, do not restore).
 __global__ void refine_kernel(const double2 *S, const double2 *P, double2 *E, int m, double lim) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= m * m) return;
@@ -1710,15 +1714,17 @@ __global__ void mask_sgram_kernel(double2 *G, const int *mask, int m) {
     if (di || dj) g[i * LD + j] = make_double2(i == j ? 1.0 : 0.0, 0.0);
 }
 
-// C = op(A) B (+ D) for small m x m matrices (leading dimension LD), op =
-// conjugate transpose when conjA; a second product op(A) B2 into C2 where given.
+// C = op(A) B, or alpha op(A) B + delta D where D is given, for small m x m
+// matrices (leading dimension LD), op = conjugate transpose when conjA; a
+// second product op(A) B2 into C2 where B2 is given.
 // Bound by the FP64 pipe and the latency of the operands: 8 x 8 outputs per
 // CTA, so that 90 x 90 reaches every SM, the sum split over the warps of all
 // four FP64 pipes, all of A's and B's share in shared memory behind one
 // barrier.  (One thread per output on 128-thread CTAs reading both operands
 // through L2: 30 us for m = 95, now 12.)
 __global__ void __launch_bounds__(256) small_zgemm_kernel(const double2 *A, const double2 *B, double2 *C, int m, int conjA,
-                                                          const double2 *D, const double2 *B2, double2 *C2) {
+                                                          const double2 *D, double alpha, double delta, const double2 *B2,
+                                                          double2 *C2) {
     __shared__ double2 As[JMAX][9], Bs[JMAX][8], sum[3][64];
     const size_t o = (size_t)blockIdx.z * LD * LD;
     const int i0 = blockIdx.y * 8, j0 = blockIdx.x * 8, tid = threadIdx.x, part = tid / 64, t = tid % 64, ti = t / 8, tj = t % 8;
@@ -1743,7 +1749,7 @@ __global__ void __launch_bounds__(256) small_zgemm_kernel(const double2 *A, cons
         __syncthreads();
         if (in) {
             s = (s + sum[0][t]) + (sum[1][t] + sum[2][t]);
-            if (D) s = s + D[o + i * LD + j];
+            if (D) s = rscale(alpha, s) + rscale(delta, D[o + i * LD + j]);
             (pass ? C2 : C)[o + i * LD + j] = s;
         }
         __syncthreads();
@@ -2091,9 +2097,9 @@ struct Solver {
         }
     }
     void small_gemm(const double2 *A, const double2 *B, double2 *C, int m, int conjA, int np = 0, const double2 *D = nullptr,
-                    const double2 *B2 = nullptr, double2 *C2 = nullptr) {
+                    const double2 *B2 = nullptr, double2 *C2 = nullptr, double alpha = 1.0, double delta = 1.0) {
         const unsigned t = (unsigned)(m + 7) / 8;
-        MB_LAUNCH_E(KN_SMALL, small_zgemm_kernel<<<dim3(t, t, np > 0 ? np : nk), 256, 0, s>>>(A, B, C, m, conjA, D, B2, C2));
+        MB_LAUNCH_E(KN_SMALL, small_zgemm_kernel<<<dim3(t, t, np > 0 ? np : nk), 256, 0, s>>>(A, B, C, m, conjA, D, alpha, delta, B2, C2));
     }
     void copy(int nch, VSet S, VSet D, int mode) {
         const unsigned bx = (unsigned)std::min<long long>(64, (nmax + 255) / 256);
@@ -2306,7 +2312,8 @@ struct Solver {
             jacobi_t<float>(np, m, masked, d_G, d_Y, nullptr, true, 1e-6);
             return;
         }
-        // FP32 sweeps, two refinement steps, FP64 sweeps on what they leave
+        // FP32 sweeps, two refinement steps and an orthonormalization, FP64
+        // sweeps on what they leave
         // (m = 95: 0.15 to 1.5 ms in all, 6.8 ms with FP64 sweeps throughout,
         // which the FP64 pipe of one SM bounds at 3 ms a sweep)
         const size_t one = (size_t)np * LD * LD;
@@ -2321,10 +2328,12 @@ struct Solver {
         small_gemm(b1, b0, b2, m, 1, np, nullptr, b1, d_Y);
         MB_LAUNCH_E(KN_JACOBI, refine_kernel<<<ge, 128, 0, s>>>(b2, d_Y, b0, m, 1e-8));
         small_gemm(b1, b0, b2, m, 0, np, b1);                      // X2
-        small_gemm(A, b2, b0, m, 0, np);
-        small_gemm(b2, b0, d_G, m, 1, np);                         // X2^H A X2
+        small_gemm(b2, b2, b0, m, 1, np);
+        small_gemm(b2, b0, b1, m, 0, np, b2, nullptr, nullptr, -0.5, 1.5);   // X3 = X2 + X2 (I - P) / 2
+        small_gemm(A, b1, b0, m, 0, np);
+        small_gemm(b1, b0, d_G, m, 1, np);                         // X3^H A X3
         jacobi_t<double>(np, m, masked, d_G, b0, nullptr, true, 1e-13);
-        small_gemm(b2, b0, d_Y, m, 0, np);
+        small_gemm(b1, b0, d_Y, m, 0, np);
     }
     // CTAs per problem: as many as give each 6 rows of eigenvectors (fewer
     // would not shorten a round) and fit on the SMs, and enough for the
@@ -2934,4 +2943,54 @@ extern "C" int mb_debug_combine_ff(const void *A, const double *Y, long long n, 
     cudaFree(Yd);
     cudaFree(dk);
     return e == cudaSuccess ? MB_OK : MB_ECUDA;
+}
+
+// Self-test hook for the Rayleigh-Ritz problems: eigenpairs of nprob Hermitian
+// m x m matrices A (host, row-major interleaved doubles, one after another).
+// refined: as the solver treats its FP64 problems; 0: FP64 sweeps alone.
+// evals: nprob x m ascending; Y: nprob x m x m, column i the vector of value i.
+extern "C" int mb_debug_rayleigh_ritz(mb_handle *h, const double *A, int m, int nprob, int refined, double *evals,
+                                      double *Y) {
+    using namespace mb;
+    if (!h || !A || !evals || !Y || m < 1 || m > JMAX || nprob < 1 || nprob > 4096) return MB_EINVAL;
+    if (cudaSetDevice(h->device) != cudaSuccess) return MB_ECUDA;
+    SolveStream stream(nullptr);
+    if (stream.err != cudaSuccess) return cuda_fail(h, stream.err);
+    Solver S;
+    S.h = h;
+    S.s = stream.s;
+    S.nk = nprob;
+    const size_t one = (size_t)LD * LD;
+    S.part_cap = std::max((size_t)std::max(2 * h->num_sms, nprob) * JMAX * JMAX, (size_t)4 * nprob * LD * LD);
+    S.d_G = S.alloc<double2>(nprob * one);
+    S.d_Y = S.alloc<double2>(nprob * one);
+    S.d_part = S.alloc<double2>(S.part_cap);
+    S.d_evals = S.alloc<double>((size_t)nprob * LD);
+    std::vector<double2> g(nprob * one, make_double2(0.0, 0.0));
+    std::vector<double> ev((size_t)nprob * LD);
+    for (int p = 0; p < nprob; ++p)
+        for (int i = 0; i < m; ++i)
+            for (int j = 0; j < m; ++j) {
+                const size_t e = 2 * (((size_t)p * m + i) * m + j);
+                g[p * one + (size_t)i * LD + j] = make_double2(A[e], A[e + 1]);
+            }
+    if (S.rc == MB_OK) S.cuda(cudaMemcpyAsync(S.d_G, g.data(), sizeof(double2) * g.size(), cudaMemcpyHostToDevice, S.s));
+    if (S.rc == MB_OK) {
+        if (refined) S.jacobi(1, m, false, 0);
+        else S.jacobi_t<double>(nprob, m, false, S.d_G, S.d_Y, nullptr, true, 1e-13);
+    }
+    if (S.rc == MB_OK) S.cuda(cudaMemcpyAsync(g.data(), S.d_Y, sizeof(double2) * g.size(), cudaMemcpyDeviceToHost, S.s));
+    if (S.rc == MB_OK) S.cuda(cudaMemcpyAsync(ev.data(), S.d_evals, sizeof(double) * ev.size(), cudaMemcpyDeviceToHost, S.s));
+    cudaStreamSynchronize(S.s);
+    if (S.rc) return S.rc;
+    for (int p = 0; p < nprob; ++p)
+        for (int i = 0; i < m; ++i) {
+            evals[(size_t)p * m + i] = ev[(size_t)p * LD + i];
+            for (int j = 0; j < m; ++j) {
+                const size_t e = 2 * (((size_t)p * m + i) * m + j);
+                Y[e] = g[p * one + (size_t)i * LD + j].x;
+                Y[e + 1] = g[p * one + (size_t)i * LD + j].y;
+            }
+        }
+    return MB_OK;
 }
