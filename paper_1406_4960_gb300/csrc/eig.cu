@@ -40,6 +40,14 @@ constexpr int LD = 128;       // leading dimension of subspace matrices
 constexpr int JMAX = 112;     // largest subspace the Jacobi kernel holds (matrix in shared memory)
 constexpr int JPAIRS = 56;    // rotation slots per Jacobi round (JMAX / 2)
 
+// the small matrices of consecutive problems: leading dimension ld, ld^2 apart
+struct Mat {
+    double2 *p;
+    int ld;
+    Mat(const double2 *q = nullptr, int l = LD) : p(const_cast<double2 *>(q)), ld(l) {}
+    __device__ double2 *of(int prob) const { return p + (size_t)prob * ld * ld; }
+};
+
 struct EigK {
     double2 *base;            // FP64 vectors of this k-point, stride nvec
     float2 *stage;            // FP32 staging for mixed-precision applies
@@ -345,8 +353,8 @@ template <typename T> constexpr size_t jacobi_smem(int m, int rows) {
 // K^H (H X), which uses the roots' HX rather than the Krylov vectors' HK,
 // which may come from a reduced-precision apply); dead slots become decoupled
 // with a huge diagonal.  full (or null): the completed matrix, of which this
-// CTA writes rows [r0, r1).  Returns the squared Frobenius norm of the live
-// part (all threads).
+// CTA writes rows [r0, r1) (leading dimension m).  Returns the squared
+// Frobenius norm of the live part (all threads).
 template <typename T2>
 __device__ double jacobi_load(const double2 *g, int m, const int *dead, int dead_ofs, T2 *A, double2 *full, int r0, int r1,
                               double *red) {
@@ -361,7 +369,7 @@ __device__ double jacobi_load(const double2 *g, int m, const int *dead, int dead
         if (di || dj) v = make_double2((i == j) ? 1e30 : 0.0, 0.0);
         else f += v.x * v.x + v.y * v.y;
         A[e] = mk((decltype(A[0].x))v.x, (decltype(A[0].x))v.y);
-        if (full && i >= r0 && i < r1) full[i * LD + j] = v;
+        if (full && i >= r0 && i < r1) full[e] = v;
     }
     for (int off = 16; off > 0; off >>= 1) f += __shfl_down_sync(0xffffffffu, f, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = f;
@@ -377,8 +385,8 @@ __device__ double jacobi_load(const double2 *g, int m, const int *dead, int dead
 // slots exactly there).  T = float: the rotations in FP32.
 template <typename T>
 __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double2 *G, int m, const int *dead, int dead_stride,
-                                                                int dead_ofs, double *evals, double2 *evecs, double2 *full,
-                                                                int sort, int max_sweeps, double rel_tol) {
+                                                                int dead_ofs, double *evals, Mat evecs, double2 *full, int sort,
+                                                                int max_sweeps, double rel_tol) {
     typedef typename std::conditional<std::is_same<T, float>::value, float2, double2>::type T2;
     extern __shared__ __align__(16) unsigned char sm[];
     const int prob = blockIdx.y, tid = threadIdx.x, nt = blockDim.x;
@@ -391,9 +399,8 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double2 *G
     int2 *pq = reinterpret_cast<int2 *>(diag + 2 * JPAIRS);
     __shared__ double red[32];
     __shared__ int perm[LD];
-    const size_t o = (size_t)prob * LD * LD;
-    const double fro2 = jacobi_load(G + o, m, dead ? dead + prob * dead_stride : nullptr, dead_ofs, A,
-                                    full ? full + o : nullptr, r0, r1, red);
+    const double fro2 = jacobi_load(G + (size_t)prob * LD * LD, m, dead ? dead + prob * dead_stride : nullptr, dead_ofs, A,
+                                    full ? full + (size_t)prob * m * m : nullptr, r0, r1, red);
     for (int e = tid; e < rows * m; e += nt) V[e] = mk(T(e % m == r0 + e / m ? 1 : 0), T(0));
     const int mp = (m + 1) & ~1;      // players, padded to even
     const int npair = mp / 2;
@@ -541,9 +548,10 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double2 *G
     }
     __syncthreads();
     if (blockIdx.x == 0 && tid < m) evals[(size_t)prob * LD + tid] = A[perm[tid] * m + perm[tid]].x;
+    double2 *out = evecs.of(prob);
     for (int e = tid; e < rows * m; e += nt) {
         const T2 v = V[e / m * m + perm[e % m]];
-        evecs[o + (size_t)(r0 + e / m) * LD + e % m] = make_double2(v.x, v.y);
+        out[(r0 + e / m) * evecs.ld + e % m] = make_double2(v.x, v.y);
     }
 }
 
@@ -561,26 +569,27 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double2 *G
 // orthonormalizes, E = R / 2 (without it, a cluster coupled at 1e-4 of its gaps
 // lost 2e-11 of 95 vectors' orthonormality, which the FP64 sweeps, unitary
 // themselves, do not restore).
-__global__ void refine_kernel(const double2 *S, const double2 *P, double2 *E, int m, double lim) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= m * m) return;
-    const size_t o = (size_t)blockIdx.y * LD * LD;
-    const int i = e / m, j = e % m;
+__global__ void refine_kernel(Mat Sm, Mat Pm, Mat Em, int m, double lim) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= m * m) return;
+    const int i = t / m, j = t % m;
     if (i < j) return;
-    const double2 p = P[o + i * LD + j];
+    const double2 *S = Sm.of(blockIdx.y), *P = Pm.of(blockIdx.y);
+    double2 *E = Em.of(blockIdx.y);
+    const double2 p = P[i * Pm.ld + j];
     if (i == j) {
-        E[o + i * LD + i] = make_double2(0.5 * (1.0 - p.x), 0.0);
+        E[i * Em.ld + i] = make_double2(0.5 * (1.0 - p.x), 0.0);
         return;
     }
     // the lower triangle, and E_ji = conj(R_ij - E_ij), so that E + E^H = R
     // holds to rounding however small the gap
-    const double li = S[o + i * LD + i].x / P[o + i * LD + i].x, lj = S[o + j * LD + j].x / P[o + j * LD + j].x;
-    const double2 sv = S[o + i * LD + j];
+    const double li = S[i * Sm.ld + i].x / P[i * Pm.ld + i].x, lj = S[j * Sm.ld + j].x / P[j * Pm.ld + j].x;
+    const double2 sv = S[i * Sm.ld + j];
     const double nx = sv.x - lj * p.x, ny = sv.y - lj * p.y, gap = lj - li;
     const bool far = fmax(fabs(nx), fabs(ny)) <= lim * fabs(gap) && gap != 0.0;
     const double2 v = far ? make_double2(nx / gap, ny / gap) : make_double2(-0.5 * p.x, -0.5 * p.y);
-    E[o + i * LD + j] = v;
-    E[o + j * LD + i] = make_double2(-p.x - v.x, p.y + v.y);
+    E[i * Em.ld + j] = v;
+    E[j * Em.ld + i] = make_double2(-p.x - v.x, p.y + v.y);
 }
 
 // U = L^{-H} with G = L L^H (G Hermitian positive definite, m <= JMAX), one
@@ -1715,32 +1724,33 @@ __global__ void mask_sgram_kernel(double2 *G, const int *mask, int m) {
 }
 
 // C = op(A) B, or alpha op(A) B + delta D where D is given, for small m x m
-// matrices (leading dimension LD), op = conjugate transpose when conjA; a
-// second product op(A) B2 into C2 where B2 is given.
+// matrices, op = conjugate transpose when conjA; a second product op(A) B2 into
+// C2 where B2 is given.
 // Bound by the FP64 pipe and the latency of the operands: 8 x 8 outputs per
 // CTA, so that 90 x 90 reaches every SM, the sum split over the warps of all
 // four FP64 pipes, all of A's and B's share in shared memory behind one
 // barrier.  (One thread per output on 128-thread CTAs reading both operands
 // through L2: 30 us for m = 95, now 12.)
-__global__ void __launch_bounds__(256) small_zgemm_kernel(const double2 *A, const double2 *B, double2 *C, int m, int conjA,
-                                                          const double2 *D, double alpha, double delta, const double2 *B2,
-                                                          double2 *C2) {
+__global__ void __launch_bounds__(256) small_zgemm_kernel(Mat A, Mat B, Mat C, int m, int conjA, Mat D, double alpha,
+                                                          double delta, Mat B2, Mat C2) {
     __shared__ double2 As[JMAX][9], Bs[JMAX][8], sum[3][64];
-    const size_t o = (size_t)blockIdx.z * LD * LD;
+    const int prob = blockIdx.z;
+    const double2 *a = A.of(prob);
     const int i0 = blockIdx.y * 8, j0 = blockIdx.x * 8, tid = threadIdx.x, part = tid / 64, t = tid % 64, ti = t / 8, tj = t % 8;
 #pragma unroll 4
     for (int e = tid; e < 8 * m; e += 256) {
         const int q = conjA ? e / 8 : e % m, i = conjA ? e % 8 : e / m;      // along the rows of memory
-        double2 v = i0 + i < m ? (conjA ? A[o + q * LD + i0 + i] : A[o + (i0 + i) * LD + q]) : make_double2(0.0, 0.0);
+        double2 v = i0 + i < m ? (conjA ? a[q * A.ld + i0 + i] : a[(i0 + i) * A.ld + q]) : make_double2(0.0, 0.0);
         if (conjA) v.y = -v.y;
         As[q][i] = v;
     }
     const int i = i0 + ti, j = j0 + tj;
     const bool in = part == 0 && i < m && j < m;
-    for (int pass = 0; pass < (B2 ? 2 : 1); ++pass) {
-        const double2 *b = pass ? B2 : B;
+    for (int pass = 0; pass < (B2.p ? 2 : 1); ++pass) {
+        const Mat &Bm = pass ? B2 : B, &Cm = pass ? C2 : C;
+        const double2 *b = Bm.of(prob);
 #pragma unroll 4
-        for (int e = tid; e < 8 * m; e += 256) Bs[e / 8][tj] = j < m ? b[o + (e / 8) * LD + j] : make_double2(0.0, 0.0);
+        for (int e = tid; e < 8 * m; e += 256) Bs[e / 8][tj] = j < m ? b[(e / 8) * Bm.ld + j] : make_double2(0.0, 0.0);
         __syncthreads();
         double2 s = make_double2(0.0, 0.0);
 #pragma unroll 4
@@ -1749,8 +1759,8 @@ __global__ void __launch_bounds__(256) small_zgemm_kernel(const double2 *A, cons
         __syncthreads();
         if (in) {
             s = (s + sum[0][t]) + (sum[1][t] + sum[2][t]);
-            if (D) s = rscale(alpha, s) + rscale(delta, D[o + i * LD + j]);
-            (pass ? C2 : C)[o + i * LD + j] = s;
+            if (D.p) s = rscale(alpha, s) + rscale(delta, D.of(prob)[i * D.ld + j]);
+            Cm.of(prob)[i * Cm.ld + j] = s;
         }
         __syncthreads();
     }
@@ -1926,7 +1936,6 @@ struct Solver {
     int o32X = 0, o32SX = 0, o32HX = 0, o32W = 0, o32K = 0, o32SK = 0, o32HK = 0, o32T = 0, o32T2 = 0, n32 = 0;
     double2 *d_Sg = nullptr, *d_Ub = nullptr, *d_Tb = nullptr;
     int *d_statb = nullptr;
-    float2 *d_Yf = nullptr;    // FP32 copy of a rotation's coefficients
     int oV, oHV, oSV, oVB, oHVB, oSVB, oQ, oHQ, oW, oSW, oT;
     int nvecs;
     std::vector<EigK> kd_host;
@@ -2065,9 +2074,11 @@ struct Solver {
         }
         if (F32 && mc > 8) {
             const int np = nk * nch;
-            MB_LAUNCH_E(KN_COMBINE32, to_float_kernel<<<dim3((A.count() * mc + 127) / 128, np), 128, 0, s>>>(Y, d_Yf, A.count(), mc));
+            // (in the Gram products' buffer, which is free here: 2 JMAX^2 >= LD^2)
+            float2 *Yf = reinterpret_cast<float2 *>(d_part);
+            MB_LAUNCH_E(KN_COMBINE32, to_float_kernel<<<dim3((A.count() * mc + 127) / 128, np), 128, 0, s>>>(Y, Yf, A.count(), mc));
             MB_LAUNCH_E(KN_COMBINE32, combine_tile_kernel<<<dim3(tile_grid(nmax, CT_T, mc, CT_C), np), 256, 0, s>>>(
-                                          d_k, nch, A, C, d_Yf, (float)alpha, (float)beta));
+                                          d_k, nch, A, C, Yf, (float)alpha, (float)beta));
             return;
         }
         // the widest column group (least re-reading of A) among those with the
@@ -2096,8 +2107,8 @@ struct Solver {
             MB_LAUNCH_E(KN_SMALL, cholinv_kernel<double><<<np, kCholThreads, cholinv_smem<double>(m), s>>>(G, m, U, status));
         }
     }
-    void small_gemm(const double2 *A, const double2 *B, double2 *C, int m, int conjA, int np = 0, const double2 *D = nullptr,
-                    const double2 *B2 = nullptr, double2 *C2 = nullptr, double alpha = 1.0, double delta = 1.0) {
+    void small_gemm(Mat A, Mat B, Mat C, int m, int conjA, int np = 0, Mat D = Mat(), Mat B2 = Mat(), Mat C2 = Mat(),
+                    double alpha = 1.0, double delta = 1.0) {
         const unsigned t = (unsigned)(m + 7) / 8;
         MB_LAUNCH_E(KN_SMALL, small_zgemm_kernel<<<dim3(t, t, np > 0 ? np : nk), 256, 0, s>>>(A, B, C, m, conjA, D, alpha, delta, B2, C2));
     }
@@ -2313,23 +2324,29 @@ struct Solver {
             return;
         }
         // FP32 sweeps, two refinement steps and an orthonormalization, FP64
-        // sweeps on what they leave
-        // (m = 95: 0.15 to 1.5 ms in all, 6.8 ms with FP64 sweeps throughout,
-        // which the FP64 pipe of one SM bounds at 3 ms a sweep)
-        const size_t one = (size_t)np * LD * LD;
-        double2 *b0 = d_part, *b1 = b0 + one, *b2 = b1 + one, *A = b2 + one;
+        // sweeps on what they leave (m = 95: 0.15 to 1.5 ms in all, 6.8 ms with
+        // FP64 sweeps throughout, which the FP64 pipe of one SM bounds at 3 ms
+        // a sweep).  Four matrices of every problem in the Gram products'
+        // buffer, which is free here; it is too small only for more than
+        // num_sms / 2 problems of over JMAX / 2 columns (blocks of over 50).
+        const size_t one = (size_t)np * m * m;
+        if (4 * one > part_cap) {
+            jacobi_t<double>(np, m, masked, d_G, d_Y, nullptr, true, 1e-13);
+            return;
+        }
+        const Mat b0(d_part, m), b1(b0.p + one, m), b2(b1.p + one, m), A(b2.p + one, m);
         const dim3 ge((m * m + 127) / 128, np);
-        jacobi_t<float>(np, m, masked, d_G, d_Y, A, false, 1e-6);
+        jacobi_t<float>(np, m, masked, d_G, d_Y, A.p, false, 1e-6);
         small_gemm(A, d_Y, b0, m, 0, np);                          // A X0
-        small_gemm(d_Y, b0, b1, m, 1, np, nullptr, d_Y, b2);        // S, P
+        small_gemm(d_Y, b0, b1, m, 1, np, Mat(), d_Y, b2);          // S, P
         MB_LAUNCH_E(KN_JACOBI, refine_kernel<<<ge, 128, 0, s>>>(b1, b2, b0, m, 1e-4));
         small_gemm(d_Y, b0, b1, m, 0, np, d_Y);                    // X1 = X0 + X0 E
         small_gemm(A, b1, b0, m, 0, np);
-        small_gemm(b1, b0, b2, m, 1, np, nullptr, b1, d_Y);
+        small_gemm(b1, b0, b2, m, 1, np, Mat(), b1, d_Y);
         MB_LAUNCH_E(KN_JACOBI, refine_kernel<<<ge, 128, 0, s>>>(b2, d_Y, b0, m, 1e-8));
         small_gemm(b1, b0, b2, m, 0, np, b1);                      // X2
         small_gemm(b2, b2, b0, m, 1, np);
-        small_gemm(b2, b0, b1, m, 0, np, b2, nullptr, nullptr, -0.5, 1.5);   // X3 = X2 + X2 (I - P) / 2
+        small_gemm(b2, b0, b1, m, 0, np, b2, Mat(), Mat(), -0.5, 1.5);   // X3 = X2 + X2 (I - P) / 2
         small_gemm(A, b1, b0, m, 0, np);
         small_gemm(b1, b0, d_G, m, 1, np);                         // X3^H A X3
         jacobi_t<double>(np, m, masked, d_G, b0, nullptr, true, 1e-13);
@@ -2339,7 +2356,7 @@ struct Solver {
     // would not shorten a round) and fit on the SMs, and enough for the
     // matrix and the rows to fit in shared memory
     template <typename T>
-    void jacobi_t(int np, int m, bool masked, const double2 *G, double2 *Y, double2 *full, bool sort, double tol) {
+    void jacobi_t(int np, int m, bool masked, const double2 *G, Mat Y, double2 *full, bool sort, double tol) {
         const size_t stat = 32 * sizeof(double) + LD * sizeof(int) + 256;
         int nc = std::max(1, std::min(h->num_sms / np, m / 6));
         while (nc < m && jacobi_smem<T>(m, (m + nc - 1) / nc) + stat > (size_t)h->smem_optin) ++nc;
@@ -2620,8 +2637,8 @@ int eigsolve(mb_handle *h, int nbands, double tol, int prec, double *evals, void
     S.d_U = S.alloc<double2>((size_t)S.nk * LD * LD);
     S.d_G2 = S.alloc<double2>((size_t)S.nk * LD * LD);
     S.d_T = S.alloc<double2>((size_t)S.nk * LD * LD);
-    // Gram partials; the four matrices of the FP64 refinement
-    S.part_cap = std::max((size_t)std::max(2 * h->num_sms, nprob) * JMAX * JMAX, (size_t)4 * nprob * LD * LD);
+    // partial products; what else is kept in it is gone before the next ones
+    S.part_cap = (size_t)std::max(2 * h->num_sms, nprob) * JMAX * JMAX;
     S.d_part = S.alloc<double2>(S.part_cap);
     S.d_evals = S.alloc<double>((size_t)nprob * LD);
     S.d_eps = S.alloc<double>((size_t)S.nk * S.M);
@@ -2640,7 +2657,6 @@ int eigsolve(mb_handle *h, int nbands, double tol, int prec, double *evals, void
         S.d_Ub = S.alloc<double2>((size_t)nprob * LD * LD);
         S.d_Tb = S.alloc<double2>((size_t)nprob * LD * LD);
         S.d_statb = S.alloc<int>(nprob);
-        S.d_Yf = S.alloc<float2>((size_t)nprob * LD * LD);
     }
     if (S.rc) return S.rc;
     S.cuda(cudaMemcpyAsync(S.d_k, S.kd_host.data(), sizeof(EigK) * S.nk, cudaMemcpyHostToDevice, s));
@@ -2961,7 +2977,7 @@ extern "C" int mb_debug_rayleigh_ritz(mb_handle *h, const double *A, int m, int 
     S.s = stream.s;
     S.nk = nprob;
     const size_t one = (size_t)LD * LD;
-    S.part_cap = std::max((size_t)std::max(2 * h->num_sms, nprob) * JMAX * JMAX, (size_t)4 * nprob * LD * LD);
+    S.part_cap = (size_t)std::max(2 * h->num_sms, nprob) * JMAX * JMAX;
     S.d_G = S.alloc<double2>(nprob * one);
     S.d_Y = S.alloc<double2>(nprob * one);
     S.d_part = S.alloc<double2>(S.part_cap);

@@ -63,8 +63,12 @@ size_t footprint_of(const mb_handle &h, int nbands, int prec) {
     int maxldg = 0;
     for (auto &k : h.kp) {
         tables += (size_t)k.ldg * (12 + 4) + (size_t)h.nterm * k.ldg * 24;
-        // position table of the compact planes; per-G offsets and phases of folded grids
-        tables += 16 * (size_t)h.n1 * h.n2 + (size_t)k.ldg * (4 + 4 * 24);
+        // row-space grids: the positions of a k-point's plane (four sources each
+        // where it is folded), the offset and the residues' phases of every G
+        if (rs_supported(h.n1, h.n2, h.order)) {
+            const int S = rs_fold(h.n1) * rs_fold(h.n2);
+            tables += S > 1 ? 16 * NN / S + (size_t)k.ldg * (4 + 24 * S) : 4 * (NN + (size_t)k.ldg);
+        }
         pf += (size_t)k.ldg * h.nb * h.order * 12;
         vec_bytes += (size_t)h.nb * k.ldg * 16;
         maxldg = std::max(maxldg, k.ldg);
@@ -81,8 +85,8 @@ size_t footprint_of(const mb_handle &h, int nbands, int prec) {
     if (prec != MB_FP64)
         work += (size_t)(3 * M + nc * (1 + 3 * kd) + 2 * std::max(M, nblk * b)) * vec_bytes / 2;
     const size_t LD = 128;
-    work += (size_t)h.kp.size() * nc * LD * LD * (prec != MB_FP64 ? 6 * 16 + 8 : 3 * 16) + (size_t)h.kp.size() * LD * LD * 16 * 3;
-    work += std::max((size_t)std::max<size_t>(304, h.kp.size() * nc) * 112 * 112, (size_t)4 * h.kp.size() * nc * LD * LD) * 16;
+    work += (size_t)h.kp.size() * nc * LD * LD * 16 * (prec != MB_FP64 ? 6 : 3) + (size_t)h.kp.size() * LD * LD * 16 * 3;
+    work += (size_t)std::max<size_t>(304, h.kp.size() * nc) * 112 * 112 * 16;
     // apply scratch: boundary rows + projector overlaps (generous bound)
     size_t scratch = (size_t)h.kp.size() *
                      ((size_t)M * 40 * 2 * (h.order - 1) * maxldg * 16 +

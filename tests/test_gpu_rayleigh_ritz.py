@@ -101,3 +101,14 @@ def test_bands_are_s_orthonormal(handle, nroots, prec, tol):
     handle.apply_S(0, V, SV, "fp64")
     G = V.reshape(nroots, -1).conj() @ SV.reshape(nroots, -1).T
     assert (G - torch.eye(nroots, dtype=G.dtype, device="cuda")).abs().max().item() < tol
+
+
+@pytest.mark.parametrize("n,m", [(76, 112), (77, 56), (77, 57)])
+def test_many_problems(handle, n, m):
+    """Around the number and size that the refinement's workspace holds."""
+    A = np.stack([(1 + 0.01 * p) * matrix("normal", m) for p in range(n)])
+    ev, Y = rayleigh_ritz(handle, A)
+    G = Y.conj().transpose(0, 2, 1) @ Y
+    assert np.abs(G - np.eye(m)).max() < 50 * m * U
+    tol = (1e-13 + 100 * m * U) * np.linalg.norm(A[-1])
+    assert np.abs(A @ Y - Y * ev[:, None, :]).max() < tol
