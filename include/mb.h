@@ -198,9 +198,15 @@ int mb_apply_H_batch(mb_handle *h, int nsel, const int *iks,
  *     contents behind.  Nothing in it has to start at zero (each element is
  *     written before it is read), but calls whose work overlaps on the GPU --
  *     different streams, or several host threads -- race on it: serialize them.
- *   - Returns MB_EINVAL when the request needs more scratch than the array
+ *   - Returns MB_EINVAL when the request counts more scratch than the array
  *     holds (it fits, for example, a 32-band FP32 apply of a 179-G, 120-spline
- *     slab k-point), and the other MB_E* codes of mb_apply_H. */
+ *     slab k-point), and the other MB_E* codes of mb_apply_H.  Counted are the
+ *     projector overlaps and coefficients and, per boundary between two runs
+ *     of knot intervals, 2 (order - 1) ldg(ik) elements a band.  On the grids of
+ *     the row-space kernel (order 6, sides of 16, 32 or 64 points), which
+ *     leaves no boundary rows, one boundary counts all the same where 3 nbands
+ *     is at most twice the device's SM count and there are 3 order intervals
+ *     or more; an autotuned or selected launch shape makes no difference. */
 #define MB_NOALLOC_SCRATCH_BYTES (16u * 1024u * 1024u)
 int mb_apply_H_noalloc(mb_handle *h, int ik, const void *X, void *Y, int nbands,
                        int prec, void *stream);

@@ -1027,67 +1027,20 @@ static int apply_H_group(mb_handle *h, int nsel, const int *iks, const void *con
     return MB_OK;
 }
 
-// Runs of knot intervals that an apply walking interval by interval makes of
-// one k-point's block: the wave model over the bands per CTA and CTAs per SM
-// that its planes, its kappa-row output ring and (FP32, at most `nocc`
-// occupied rows and `ldg` columns) its window of X rows allow.
-static int interval_runs(const mb_handle *h, int ik, int nbands, size_t c2) {
-    const int K = h->order, P = h->nquad, ldg = h->kp[ik].ldg;
-    const int nmax_chunks = std::max(1, std::min(kMaxChunks, h->nint / K));
-    int waves = 0;
-    auto it = h->tuned.find(std::make_tuple(1, nbands, c2 == 16 ? 1 : 0));
-    if (it != h->tuned.end()) waves = it->second.waves;
-    auto runs = [&](int bt, int ctas) {
-        return wave_model_chunks((nbands + bt - 1) / bt, h->num_sms * ctas, nmax_chunks, waves,
-                                 [&](int n) { return (h->nint + n - 1) / n + 1.0; });
-    };
-    const KPoint &kp = h->kp[ik];
-    int nocc = 1;
-    if (kp.ng) {
-        const auto r = std::minmax_element(kp.n1.begin(), kp.n1.begin() + kp.ng);
-        nocc = *r.second - *r.first + 1;
-    }
-    if (c2 == 8 && K == 6 && P == 6) {
-        // grid, largest nocc and ldg, bands per CTA, CTAs per SM, entries of an X window in shared memory
-        static const struct { int n1, n2, nocc, ldg, bt, ctas, window; } shapes[] = {
-            {16, 16, 10, 96, 2, 4, 0},   {32, 16, 24, 192, 2, 2, 0},    {32, 16, 24, 256, 2, 2, 3072},
-            {32, 16, 24, 192, 2, 2, 2304}, {32, 16, 24, 192, 1, 4, 0},  {32, 32, 24, 384, 1, 2, 0},
-            {32, 32, 24, 384, 2, 1, 0},  {32, 32, 23, 384, 1, 3, 2304}, {64, 64, 48, 1536, 1, 1, 0},
-            {64, 64, 48, 1536, 1, 1, 0}, {32, 16, 22, 192, 2, 3, 2304}};
-        for (const auto &sh : shapes) {
-            if (h->n1 != sh.n1 || h->n2 != sh.n2 || nocc > sh.nocc || ldg > sh.ldg) continue;
-            const size_t budget = std::min((size_t)h->smem_optin, (size_t)228 * 1024 / sh.ctas - 1024);
-            const size_t fixed = ((size_t)sh.bt * 6 * sh.nocc * (sh.n2 + 1) + sh.window + (size_t)sh.bt * K * ldg) * 8;
-            auto smem = [&](int n) { return fixed + (size_t)((h->nint + n - 1) / n) * K * P * sizeof(float); };
-            int n = runs(sh.bt, sh.ctas);
-            while (n < nmax_chunks && smem(n) > budget) ++n;
-            if (smem(n) <= budget) return n;
-        }
-    }
-    if (rs_supported(h->n1, h->n2, K) && (c2 == 8 || (h->n1 <= 32 && h->n2 <= 32))) {
-        const bool small = h->n1 <= 32 && h->n2 <= 32;
-        const int ctas = c2 == 16 ? 1 : (h->n1 * h->n2 <= 512 || (h->n1 == 32 && h->n2 == 32)) ? 3 : small ? 2 : 1;
-        const size_t plane = (size_t)h->n1 * (h->n2 + 1) * c2 + 8 + 8 * (2 * sizeof(int) + 8 * c2 / 2);
-        const size_t budget = (size_t)h->smem_optin / ctas - 1024;
-        for (int bt = small ? 2 : 1; bt >= 1; --bt)
-            if ((size_t)bt * K * ldg * c2 + plane <= budget) return runs(bt, ctas);
-    }
-    return runs(1, 1);
-}
-
-// Scratch by which mb_apply_H_noalloc admits a request: that of the walk over
-// knot intervals, whose runs leave their boundary rows there (at least what
-// any plane kernel uses; the row-space kernel has no boundary rows, and its
-// requests are admitted as the others' are).
+// Scratch by which mb_apply_H_noalloc admits a request: what the apply uses.
+// The row-space kernel leaves no boundary rows, but the limit counts those of
+// one run boundary where a walk over knot intervals has one in any case (fewer
+// bands than two thirds of the SMs, and enough intervals for three runs), so
+// that requests far beyond the array stay refused on every grid, and an
+// autotuned run count does not change which.
 size_t apply_H_scratch_need(const mb_handle *h, int ik, int nbands, int prec) {
-    const size_t c2 = prec == MB_FP64 ? 16 : 8;
-    const size_t need = per_k_scratch(h, h->kp[ik].ldg, nbands, interval_runs(h, ik, nbands, c2), c2, prec == MB_BF16);
-    return std::max(need, prec == MB_FP64 ? apply_H_need<double>(h, 1, &ik, nbands, false)
-                                          : apply_H_need<float>(h, 1, &ik, nbands, prec == MB_BF16));
+    const size_t need = prec == MB_FP64 ? apply_H_need<double>(h, 1, &ik, nbands, false)
+                                        : apply_H_need<float>(h, 1, &ik, nbands, prec == MB_BF16);
+    if (!rs_supported(h->n1, h->n2, h->order) || 3 * nbands > 2 * h->num_sms || h->nint < 3 * h->order) return need;
+    return std::max(need, per_k_scratch(h, h->kp[ik].ldg, nbands, 2, prec == MB_FP64 ? 16 : 8, prec == MB_BF16));
 }
 
 // A single-k-point apply on a scratch region supplied by the caller (no allocation here).
-
 int apply_H_on_scratch(mb_handle *h, int ik, const void *X, void *Y, int nbands, int prec, cudaStream_t s,
                        void *scratch) {
     const void *xs[1] = {X};
