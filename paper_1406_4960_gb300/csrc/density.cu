@@ -234,16 +234,11 @@ int density_rows(mb_handle *h, const void *evecs, int nbands, const double *occ_
     int nparts = 1, nchunks = 1;
     double best = 1e300;
     for (int c = 1; c <= std::min(nb, 64); ++c) {
-        double run = 0.0;             // the longest run of one pair
-        for (int i = 0; i < c; ++i) {
-            const int j0 = chunk_begin(i, nb, c), j1 = chunk_begin(i + 1, nb, c), ji = std::max(0, j0 - kRsHalo);
-            double t = 14.0 * (j1 - j0) * (m1 * m2 / 128);
-            for (int a0 = ji; a0 < j1; a0 += RR) {
-                const int n = std::min(RR, j1 - a0);
-                t += rounds4(n * N2) * line(m1) + rounds4(n * m1) * line(m2);
-            }
-            run = std::max(run, t);
-        }
+        // the longest run of one pair: the last, of ceil(nb / c) rows and the
+        // rows before them that they multiply
+        const int L = (nb + c - 1) / c, in = L + std::min(kRsHalo, nb - L);
+        auto lines = [&](int n) { return rounds4(n * N2) * line(m1) + rounds4(n * m1) * line(m2); };
+        const double run = 14.0 * L * (m1 * m2 / 128) + in / RR * lines(RR) + lines(in % RR);
         for (int p = 1; p <= std::min(pairs, 32); ++p) {
             const double rounds = (double)(((long long)p * c * S + h->num_sms - 1) / h->num_sms);
             const double cost = rounds * ((pairs + p - 1) / p) * run + 9.0 * 14.0 * (m1 * m2 / 128) * p;
