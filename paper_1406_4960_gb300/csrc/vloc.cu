@@ -175,43 +175,54 @@ __global__ void vloc_tables_kernel(int nq, int N1, int N2, int l1, int l2, const
 }
 
 // The row-space potential U[j][d](r) = sum_q B_j(z_q) B_{j-d}(z_q) w_q V(r, z_q) / (N1 N2),
-// d = 0 .. order - 1 (0 where j - d < 0), summed over the knot intervals both
-// splines share: one thread per (row j, grid point r), which reads every
-// plane of the row's support once.  Stored in pairs of d, each residue of the
-// folded sides contiguous: [j][d / 2][residue][point].  FP64 bound (about 100
-// FMAs per element); it runs once per potential: 0.02 ms for the slab's table.
+// d = 0 .. order - 1 (0 where j - d < 0), over the knot intervals both splines
+// share.  A CTA takes blockDim.x grid points of one row j: the products of B
+// values and weights of the row's planes are formed once in shared memory, and
+// a thread reads every plane of the row's support once at its point, a batch
+// of loads in flight together.  Stored in pairs of d, each residue of the
+// folded sides contiguous: [j][d / 2][residue][point].  Bound by the FP64 pipe:
+// 126 FMAs per element, 234 operations with a thread forming its own products.
+// It runs once per potential.
+constexpr int kMaxQuad = 16;      // setup's limit of points per interval
 __global__ void __launch_bounds__(256) rs_tables_kernel(int nb, int nint, int P, int N1, int N2, int s1, int s2,
                                                         const double *V, const double *wq, const double *Bq,
                                                         double2 *U64, float2 *U32) {
-    constexpr int K = kRsOrder;
+    constexpr int K = kRsOrder, PF = 12;
+    __shared__ double W[K * kMaxQuad][K];
     const int NN = N1 * N2, M1 = N1 / s1, NP = NN / (s1 * s2);
-    const size_t total = (size_t)(nb + kRsPad) * NN;
+    const int j = (int)blockIdx.x / (NN / blockDim.x), r = (int)blockIdx.x % (NN / blockDim.x) * blockDim.x + threadIdx.x;
+    // spline j is entry m = j + 1 - t of interval t's kappa splines
+    const int t0 = max(0, j + 2 - K), q0 = t0 * P, np = j < nb ? (min(nint - 1, j + 1) + 1 - t0) * P : 0;
     const double scale = 1.0 / NN;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(e / NN), r = (int)(e % NN);
-        double acc[K];
+    for (int e = threadIdx.x; e < np * K; e += blockDim.x) {
+        const int p = e / K, d = e % K, m = j + 1 - t0 - p / P;
+        const double *b = Bq + (size_t)(q0 + p) * K;
+        W[p][d] = d <= m ? b[m] * (wq[q0 + p] * scale) * b[m - d] : 0.0;
+    }
+    __syncthreads();
+    double acc[K];
 #pragma unroll
-        for (int d = 0; d < K; ++d) acc[d] = 0.0;
-        // spline j is entry m = j + 1 - t of interval t's kappa splines
-        for (int t = max(0, j + 2 - K); t <= min(nint - 1, j + 1) && j < nb; ++t) {
-            const int m = j + 1 - t;
-            for (int s = 0; s < P; ++s) {
-                const int q = t * P + s;
-                const double *b = Bq + (size_t)q * K;
-                const double v = b[m] * (wq[q] * scale * V[(size_t)q * NN + r]);
+    for (int d = 0; d < K; ++d) acc[d] = 0.0;
+    for (int p0 = 0; p0 < np; p0 += PF) {
+        double v[PF];
 #pragma unroll
-                for (int d = 0; d < K; ++d)
-                    if (d <= m && j - d >= 0) acc[d] = fma(b[m - d], v, acc[d]);
-            }
+        for (int i = 0; i < PF; ++i) v[i] = p0 + i < np ? V[(size_t)(q0 + p0 + i) * NN + r] : 0.0;
+#pragma unroll
+        for (int i = 0; i < PF; ++i) {
+            if (p0 + i >= np) break;
+            const int dm = min(j, j + 1 - t0 - (p0 + i) / P);        // uniform in the CTA
+#pragma unroll
+            for (int d = 0; d < K; ++d)
+                if (d <= dm) acc[d] = fma(W[p0 + i][d], v[i], acc[d]);
         }
-        const int i1 = r / N2, i2 = r % N2;
-        const int res = (i1 % s1) * s2 + i2 % s2, pt = (i2 / s2) * M1 + i1 / s1;
+    }
+    const int i1 = r / N2, i2 = r % N2;
+    const int res = (i1 % s1) * s2 + i2 % s2, pt = (i2 / s2) * M1 + i1 / s1;
 #pragma unroll
-        for (int t = 0; t < K / 2; ++t) {
-            const size_t o = ((size_t)j * (K / 2) + t) * NN + (size_t)res * NP + pt;
-            U64[o] = make_double2(acc[2 * t], acc[2 * t + 1]);
-            U32[o] = make_float2((float)acc[2 * t], (float)acc[2 * t + 1]);
-        }
+    for (int t = 0; t < K / 2; ++t) {
+        const size_t o = ((size_t)j * (K / 2) + t) * NN + (size_t)res * NP + pt;
+        U64[o] = make_double2(acc[2 * t], acc[2 * t + 1]);
+        U32[o] = make_float2((float)acc[2 * t], (float)acc[2 * t + 1]);
     }
 }
 
@@ -250,8 +261,10 @@ int vloc_derive_tables(mb_handle *h) {
     double *wq = nullptr;
     if ((rc = dev_upload(h, (void **)&wq, h->wq.data(), h->wq.size() * sizeof(double)))) return rc;
     auto blocks = [&](size_t m) { return (int)std::min<size_t>((m + 255) / 256, (size_t)h->num_sms * 8); };
+    // 64 points a CTA (256 divides NN) where 256 would leave SMs without one
+    const int T = h->nb * (NN / 256) < 2 * (size_t)h->num_sms ? 64 : 256;
     if (rs)
-        rs_tables_kernel<<<blocks((size_t)(h->nb + kRsPad) * NN), 256, 0, h->hs>>>(
+        rs_tables_kernel<<<(unsigned)((h->nb + kRsPad) * (NN / T)), T, 0, h->hs>>>(
             h->nb, h->nint, h->nquad, h->n1, h->n2, rs_fold(h->n1), rs_fold(h->n2), h->d_vloc, wq,
             (const double *)h->t64.Bq, (double2 *)h->t64.U, (float2 *)h->t32.U);
     else
