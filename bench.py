@@ -934,7 +934,7 @@ def main():
     ap.add_argument("--apply-prec", default="fp32", help="precision of --apply-only")
     ap.add_argument("--apply-tune", action="store_true", help="autotune the launch shape of --apply-only")
     ap.add_argument("--apply-kernel", type=int, default=None, help="row-space instance id for --apply-only")
-    ap.add_argument("--apply-persistent", action="store_true", help="persistent launch for --apply-kernel")
+    ap.add_argument("--apply-persistent", action="store_true", help="accepted for --apply-kernel; makes no difference")
     ap.add_argument("--no-serve", action="store_true")
     ap.add_argument("--no-scf", action="store_true")
     ap.add_argument("--scf-only", action="store_true", help="run the self-consistent loop section only")

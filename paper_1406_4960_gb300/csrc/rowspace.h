@@ -47,7 +47,10 @@ template <typename R> cudaError_t rs_launch(const RsArgs<R> &a, const RsShape &s
 template <typename R> int rs_resident(const RsShape &sh, int num_sms);
 
 // Small FP64 problems: a cluster of kRsSmallCl CTAs per (k-point, band), at most
-// kRsSmallRows rows each (rowspace64.cu), where every one has an SM to itself.
+// kRsSmallRows rows each (rowspace64.cu), up to as many CTAs as SMs.  A cluster's
+// CTAs share a GPC, and 15 clusters of 8 are resident on 152 SMs: up to 15
+// pairs take one round (40 rows: 46 us an apply, 59 to 86 by runs of rows), 16
+// to 19 two (80 us; 20 pairs by runs 71).
 constexpr int kRsSmallCl = 8, kRsSmallRows = 8;
 bool rs_small_supported(const RsShape &sh, int pairs, int nb, int num_sms);
 cudaError_t rs_launch_small(const RsArgs<double> &a, unsigned pairs, cudaStream_t s);

@@ -220,9 +220,8 @@ int build_host_tables(mb_handle *h, const mb_cell *cell, const double *kpts, int
                 }
             }
         if (gl.empty()) return MB_EINVAL;
-        // disc order: by n2, then n1 -- column by column of the grid, so that
-        // consecutive G of a warp sit one compact-plane row apart (a stride
-        // of N2 + 1 elements, free of shared-memory bank conflicts)
+        // disc order: by n2, then n1, so that consecutive G lie side by side
+        // along the contiguous axis 1 of the row-space kernel's planes
         std::sort(gl.begin(), gl.end(), [](const std::tuple<int, int, int> &x, const std::tuple<int, int, int> &y) {
             return std::make_pair(std::get<2>(x), std::get<1>(x)) < std::make_pair(std::get<2>(y), std::get<1>(y));
         });
