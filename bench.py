@@ -42,10 +42,13 @@ sys.path.insert(0, ROOT)
 os.environ.setdefault("CUDA_DEVICE_MAX_CONNECTIONS", "32")
 
 METRIC = "Hψ GB/s & eigensolves/s at 1e-6 Ha vs plain FP64 GPU; p50/p99 solve latency"
-# The plane kernel's sources: its DRAM traffic (from an ncu capture, recorded
-# in the profile summary below with the kernel instance) is reported only
-# while these are unchanged and the same instance runs.
-PLANE_SOURCES = ("rowspace.cuh", "rowspace32.cu", "fft_reg.cuh", "cplx.cuh")
+# The sources of the plane kernel and of its launch plan (which rows a CTA takes
+# decides how often halo rows and the potential are read): its DRAM traffic
+# (from an ncu capture, recorded in the profile summary below with the kernel
+# instance) is reported only while these are unchanged and the same instance
+# runs.
+PLANE_SOURCES = ("rowspace.cuh", "rowspace32.cu", "rowspace.h", "rowspace_inst.inc", "fft_reg.cuh", "cplx.cuh",
+                 "apply_common.cuh", "mb_internal.h", "apply.cu")
 PLANE_PROFILES = {
     "slab": "profiles/rowspace_kernel_slab_fp32.md",
     "graphene": "profiles/rowspace_kernel_graphene_fp32.md",
