@@ -12,19 +12,37 @@
 // transforms and 14 of products, against 43 per plane (six planes a row)
 // with a transform of every plane.
 //
-// density_rows_kernel: one CTA per (part, run of rows), a part being a
-// contiguous share of the (k-point, band) pairs; it walks its pairs one after
-// the other and adds their products to its own part of P in global memory
-// (L2).  density_planes_kernel adds the parts in order and forms the planes.
+// The quadratic form's rounding is of its largest product, so where the sum of
+// the bands nearly vanishes it loses twice the digits that |sum_j B_j x_j|^2
+// loses (the slab's one band near its nodes: 1.4e-11 of the density there for
+// 5.6e-13, and 3.2e-14 for 2.4e-15 of the largest v_xc).  Few bands therefore
+// take the planes' sums of squares themselves, formed from the same
+// transformed rows (SQUARES: 90 instructions a row).
+//
+// density_rows_kernel: one CTA per (part, run of rows or knot intervals), a
+// part being a contiguous share of the (k-point, band) pairs; it walks its
+// pairs one after the other and adds their products (or squares) to its own
+// part in global memory (L2).  density_planes_kernel adds the parts in order
+// and forms the planes (density_sum_kernel: adds them).
 // FP64 bound.  Slab, 4 k x 32 bands: 0.65 ms + 0.07 ms, against 5.1 ms (both
 // under ncu) with every plane of every band transformed and squared.
 #include <algorithm>
+#include <cmath>
 
 #include "rowspace.cuh"
 
 namespace mb {
 
 namespace {
+
+// The number of equally occupied pairs, (sum |f|)^2 / sum f^2, from which on the
+// products are taken.  The smallest of a million sums of n squares of real
+// amplitudes is about (n!! 1e-6)^(2/n) / n of their mean: 7e-4 for n = 4, 6e-3
+// for 6, where the largest error of v_xc ~ rho^(1/3) no longer comes from such
+// points (6e-16 to 8e-16 either way from 5 bands on).  The slab's 8 bands (6.1)
+// take 240 us by squares and 185 by products, 3 bands 112 and 122; the 16 x 16
+// cell's 3 bands 64 and 84 to 97.
+constexpr double kMinPairs = 6.0;
 
 struct DensRowsK {
     const double2 *X;     // nbands x nb x ldg coefficients of this k-point
@@ -33,18 +51,19 @@ struct DensRowsK {
 
 struct DensRowsArgs {
     const double *occ;    // nk x nbands
-    double *part;         // [part][nb][kappa][residue][point]
+    const double *Bq;     // nq x kappa
+    double *part;         // [part][nb][kappa][residue][point], or [part][nq][residue][point]
     const int *gpos;
     const int *pos;
     const int4 *src;
     const double2 *phase;
     size_t phase_stride;
-    int nbands, nb, nk, nparts, nchunks, s1, s2;
+    int nbands, nb, nint, nquad, nk, nparts, nchunks, s1, s2;
     int accumulate;       // 0: the parts hold nothing yet
     DensRowsK d[kMaxK];
 };
 
-template <int M1, int M2, int T, int RR, int CTAS, bool PR, bool FOLD>
+template <int M1, int M2, int T, int RR, int CTAS, bool PR, bool FOLD, bool SQUARES>
 __global__ void __launch_bounds__(T, CTAS) density_rows_kernel(const __grid_constant__ DensRowsArgs a) {
     typedef double2 C;
     typedef RsGeom<double, M1, M2, RR, PR> G;
@@ -55,11 +74,15 @@ __global__ void __launch_bounds__(T, CTAS) density_rows_kernel(const __grid_cons
     const int tid = threadIdx.x;
     const int S = FOLD ? a.s1 * a.s2 : 1, rank = FOLD ? (int)blockIdx.x % S : 0, item = (int)blockIdx.x / S;
     const int c = item % a.nchunks, p = item / a.nchunks, nb = a.nb;
-    const int j0 = chunk_begin(c, nb, a.nchunks), j1 = chunk_begin(c + 1, nb, a.nchunks), ji = max(0, j0 - H);
+    // SQUARES: knot intervals j0 .. j1 - 1, whose splines are rows j0 - 1 .. j1 + 3;
+    // row m completes interval m - 4 (rows outside the basis are zero)
+    const int n = SQUARES ? a.nint : nb;
+    const int j0 = chunk_begin(c, n, a.nchunks), j1 = chunk_begin(c + 1, n, a.nchunks);
+    const int ji = max(0, j0 - (SQUARES ? 1 : H)), mend = SQUARES ? j1 + 4 : j1, je = min(nb, mend);
     const int npair = a.nk * a.nbands;
     const int q0 = (int)((long long)p * npair / a.nparts), q1 = (int)((long long)(p + 1) * npair / a.nparts);
     const size_t prow = (size_t)S * NP;               // one product of one row
-    double *part = a.part + (size_t)p * nb * kRsOrder * prow + (size_t)rank * NP;
+    double *part = a.part + (size_t)p * (SQUARES ? a.nint * a.nquad : nb * kRsOrder) * prow + (size_t)rank * NP;
     bool fresh = !a.accumulate;
     for (int pair = q0; pair < q1; ++pair) {
         const int k = pair / a.nbands, n = pair - k * a.nbands;
@@ -67,8 +90,8 @@ __global__ void __launch_bounds__(T, CTAS) density_rows_kernel(const __grid_cons
         const double f = a.occ[(size_t)d.kg * a.nbands + n];
         if (f == 0.0) continue;                       // uniform over the CTA
         const C *X = d.X + (size_t)n * nb * d.ldg;
-        for (int a0 = ji; a0 < j1; a0 += RR) {
-            const int nin = min(RR, j1 - a0);
+        for (int a0 = ji; a0 < mend; a0 += RR) {
+            const int nin = max(0, min(RR, je - a0));
             const C *Xa = X + (size_t)a0 * d.ldg;
             __syncthreads();                          // the previous step's planes are consumed
             if constexpr (!FOLD) {
@@ -116,9 +139,33 @@ __global__ void __launch_bounds__(T, CTAS) density_rows_kernel(const __grid_cons
                 C h[H];                               // h[k]: x of row m - 5 + k
 #pragma unroll
                 for (int k2 = 0; k2 < H; ++k2) h[k2] = a0 > ji ? hist[k2 * NP + pt] : czero<C>();
+                if constexpr (SQUARES) {
+                    for (int i = 0; i < min(RR, mend - a0); ++i) {
+                        const C xm = i < nin ? x[i * G::PS] : czero<C>();
+                        const int t = a0 + i - 4;
+                        for (int s0 = 0; t >= j0 && s0 < a.nquad; s0 += 6) {      // planes, six at a time
+                            double *R = part + (size_t)(t * a.nquad + s0) * prow + pt, acc[6];
+#pragma unroll
+                            for (int s = 0; s < 6; ++s) acc[s] = !fresh && s0 + s < a.nquad ? R[s * prow] : 0.0;
+#pragma unroll
+                            for (int s = 0; s < 6; ++s) {
+                                if (s0 + s >= a.nquad) break;
+                                const double *b = a.Bq + (size_t)(t * a.nquad + s0 + s) * kRsOrder;
+                                C psi = rscale(__ldg(b), h[0]);
+#pragma unroll
+                                for (int u = 1; u < H; ++u) rfma(psi, __ldg(b + u), h[u]);
+                                rfma(psi, __ldg(b + H), xm);
+                                R[s * prow] = fma(f, fma(psi.x, psi.x, psi.y * psi.y), acc[s]);
+                            }
+                        }
+#pragma unroll
+                        for (int k2 = 0; k2 + 1 < H; ++k2) h[k2] = h[k2 + 1];
+                        h[H - 1] = xm;
+                    }
+                }
                 double *P = part + (size_t)a0 * kRsOrder * prow + pt;
                 // GR rows at a time: their sums so far are all loaded first
-                for (int i0 = 0; i0 < nin; i0 += GR, P += GR * kRsOrder * prow) {
+                for (int i0 = 0; !SQUARES && i0 < nin; i0 += GR, P += GR * kRsOrder * prow) {
                     double acc[GR][kRsOrder];
 #pragma unroll
                     for (int i = 0; i < GR; ++i)
@@ -149,10 +196,22 @@ __global__ void __launch_bounds__(T, CTAS) density_rows_kernel(const __grid_cons
         }
         fresh = false;
     }
+    const int per = SQUARES ? a.nquad : kRsOrder;
     if (fresh)                                        // no occupied pair
-        for (int m = j0; m < j1; ++m)
-            for (int e = 0; e < kRsOrder; ++e)
-                for (int pt = tid; pt < NP; pt += T) part[((size_t)m * kRsOrder + e) * prow + pt] = 0.0;
+        for (int e = j0 * per; e < j1 * per; ++e)
+            for (int pt = tid; pt < NP; pt += T) part[e * prow + pt] = 0.0;
+}
+
+// rho of the squares: the parts added in order
+__global__ void __launch_bounds__(128) density_sum_kernel(const double *part, int nparts, int nq, int N1, int N2, int s1, int s2,
+                                                          double scale, double *rho) {
+    const int NN = N1 * N2, M1 = N1 / s1, NP = NN / (s1 * s2), e = blockIdx.x % (unsigned)(NN / 128) * 128 + threadIdx.x;
+    const int q = blockIdx.x / (unsigned)(NN / 128), res = e / NP, pt = e % NP;
+    const int r = (pt % M1 * s1 + res / s2) * N2 + pt / M1 * s2 + res % s2;
+    double s = 0.0;
+#pragma unroll 8
+    for (int p = 0; p < nparts; ++p) s += part[((size_t)p * nq + q) * NN + e];
+    rho[(size_t)q * NN + r] = scale * s;
 }
 
 // rho of one knot interval's planes at one grid point: the band of P that the
@@ -199,7 +258,7 @@ __global__ void __launch_bounds__(128) density_planes_kernel(const double *part,
     }
 }
 
-template <int M1, int M2, int T, int RR, int CTAS>
+template <int M1, int M2, int T, int RR, int CTAS, bool SQUARES>
 cudaError_t launch_rows(const DensRowsArgs &a, bool pruned, int smem_limit, int device, cudaStream_t s) {
     const unsigned S = (unsigned)(a.s1 * a.s2), grid = (unsigned)(a.nparts * a.nchunks) * S;
     auto go = [&](auto kern) {
@@ -210,16 +269,24 @@ cudaError_t launch_rows(const DensRowsArgs &a, bool pruned, int smem_limit, int 
         return cudaGetLastError();
     };
     if constexpr (M1 * M2 > 256)
-        if (S > 1) return go(density_rows_kernel<M1, M2, T, RR, CTAS, false, true>);
+        if (S > 1) return go(density_rows_kernel<M1, M2, T, RR, CTAS, false, true, SQUARES>);
     if (S > 1) return cudaErrorInvalidValue;
-    return pruned ? go(density_rows_kernel<M1, M2, T, RR, CTAS, true, false>)
-                  : go(density_rows_kernel<M1, M2, T, RR, CTAS, false, false>);
+    return pruned ? go(density_rows_kernel<M1, M2, T, RR, CTAS, true, false, SQUARES>)
+                  : go(density_rows_kernel<M1, M2, T, RR, CTAS, false, false, SQUARES>);
+}
+template <bool SQUARES>
+cudaError_t launch_rows(const DensRowsArgs &a, int m1, int m2, bool pruned, int smem_limit, int device, cudaStream_t s) {
+    if (m1 == 16 && m2 == 16) return launch_rows<16, 16, 128, 16, 2, SQUARES>(a, pruned, smem_limit, device, s);
+    if (m1 == 16) return launch_rows<16, 32, 256, 16, 1, SQUARES>(a, pruned, smem_limit, device, s);
+    if (m2 == 16) return launch_rows<32, 16, 256, 16, 1, SQUARES>(a, pruned, smem_limit, device, s);
+    return launch_rows<32, 32, 256, 8, 1, SQUARES>(a, pruned, smem_limit, device, s);
 }
 
 }  // namespace
 
-// rho (device, nq x N1 x N2) on grids the row-space kernels serve.
-int density_rows(mb_handle *h, const void *evecs, int nbands, const double *occ_dev, bool nonneg, double *rho,
+// rho (device, nq x N1 x N2) on grids the row-space kernels serve; occ: the
+// occupations on the host, occ_dev: their copy on the device.
+int density_rows(mb_handle *h, const void *evecs, int nbands, const double *occ, const double *occ_dev, double *rho,
                  cudaStream_t s) {
     const int nk = (int)h->kp.size(), nb = h->nb, NN = h->n1 * h->n2;
     const int s1 = rs_fold(h->n1), s2 = rs_fold(h->n2), S = s1 * s2, m1 = h->n1 / s1, m2 = h->n2 / s2;
@@ -228,17 +295,27 @@ int density_rows(mb_handle *h, const void *evecs, int nbands, const double *occ_
     // in whole rounds of four warps, and 14 products per output row and point
     // (runs that leave a step nearly empty pay for it: 1.03 ms with 16 parts
     // of 9 runs, 18 rows each, on the slab); a part more costs its sum.
+    double sum = 0.0, sq = 0.0;
+    bool nonneg = true;
+    for (int i = 0; i < nk * nbands; ++i) {
+        sum += std::fabs(occ[i]);
+        sq += occ[i] * occ[i];
+        nonneg = nonneg && occ[i] >= 0.0;
+    }
+    const bool squares = !(sum * sum >= kMinPairs * sq);
     const int pairs = nk * nbands, RR = m1 == 32 && m2 == 32 ? 8 : 16, N2 = h->rs_pruned ? m2 * 3 / 4 : m2;
     auto line = [](int m) { return m == 32 ? 360.0 : 140.0; };
     auto rounds4 = [](int lines) { return (double)((lines + 127) / 128); };
     int nparts = 1, nchunks = 1;
     double best = 1e300;
-    for (int c = 1; c <= std::min(nb, 64); ++c) {
-        // the longest run of one pair: the last, of ceil(nb / c) rows and the
-        // rows before them that they multiply
-        const int L = (nb + c - 1) / c, in = L + std::min(kRsHalo, nb - L);
+    const int items = squares ? h->nint : nb;
+    const double per = squares ? 15.0 * h->nquad : 14.0;
+    for (int c = 1; c <= std::min(items, 64); ++c) {
+        // the longest run of one pair: the last, of ceil(items / c) rows and the
+        // rows before them that they multiply (or intervals and their rows)
+        const int L = (items + c - 1) / c, in = std::min(nb, L + std::min(kRsHalo, nb - L));
         auto lines = [&](int n) { return rounds4(n * N2) * line(m1) + rounds4(n * m1) * line(m2); };
-        const double run = 14.0 * L * (m1 * m2 / 128) + in / RR * lines(RR) + lines(in % RR);
+        const double run = per * L * (m1 * m2 / 128) + in / RR * lines(RR) + lines(in % RR);
         for (int p = 1; p <= std::min(pairs, 32); ++p) {
             const double rounds = (double)(((long long)p * c * S + h->num_sms - 1) / h->num_sms);
             const double cost = rounds * ((pairs + p - 1) / p) * run + 9.0 * 14.0 * (m1 * m2 / 128) * p;
@@ -252,9 +329,10 @@ int density_rows(mb_handle *h, const void *evecs, int nbands, const double *occ_
     cudaMemPool_t pool = mb_pool(h->device);
     if (!pool) return MB_ECUDA;
     double *part = nullptr;
-    MB_CUDA(cudaMallocFromPoolAsync((void **)&part, (size_t)nparts * nb * kRsOrder * NN * sizeof(double), pool, s));
+    MB_CUDA(cudaMallocFromPoolAsync((void **)&part, (size_t)nparts * (squares ? h->nq : nb * kRsOrder) * NN * sizeof(double), pool, s));
     DensRowsArgs a;
     a.occ = occ_dev;
+    a.Bq = (const double *)h->t64.Bq;
     a.part = part;
     a.gpos = h->d_rsgpos;
     a.pos = reinterpret_cast<const int *>(h->d_rspos);
@@ -263,6 +341,8 @@ int density_rows(mb_handle *h, const void *evecs, int nbands, const double *occ_
     a.phase_stride = (size_t)h->total_ldg;
     a.nbands = nbands;
     a.nb = nb;
+    a.nint = h->nint;
+    a.nquad = h->nquad;
     a.nparts = nparts;
     a.nchunks = nchunks;
     a.s1 = s1;
@@ -284,13 +364,15 @@ int density_rows(mb_handle *h, const void *evecs, int nbands, const double *occ_
             d.kg = k;
             off += (size_t)nbands * nb * h->kp[k].ldg;
         }
-        if (m1 == 16 && m2 == 16) e = launch_rows<16, 16, 128, 16, 2>(a, h->rs_pruned, h->smem_optin, h->device, s);
-        else if (m1 == 16) e = launch_rows<16, 32, 256, 16, 1>(a, h->rs_pruned, h->smem_optin, h->device, s);
-        else if (m2 == 16) e = launch_rows<32, 16, 256, 16, 1>(a, h->rs_pruned, h->smem_optin, h->device, s);
-        else e = launch_rows<32, 32, 256, 8, 1>(a, h->rs_pruned, h->smem_optin, h->device, s);
+        e = squares ? launch_rows<true>(a, m1, m2, h->rs_pruned, h->smem_optin, h->device, s)
+                    : launch_rows<false>(a, m1, m2, h->rs_pruned, h->smem_optin, h->device, s);
         ++h->launches;
     }
-    if (e == cudaSuccess) {
+    if (e == cudaSuccess && squares) {
+        density_sum_kernel<<<(unsigned)(h->nq * (NN / 128)), 128, 0, s>>>(part, nparts, h->nq, h->n1, h->n2, s1, s2, 1.0 / h->Ac, rho);
+        e = cudaGetLastError();
+        ++h->launches;
+    } else if (e == cudaSuccess) {
         density_planes_kernel<<<dim3((NN + 127) / 128, h->nint), 128, 0, s>>>(
             part, nparts, nb, h->nint, h->nquad, h->n1, h->n2, s1, s2, (const double *)h->t64.Bq, 1.0 / h->Ac, nonneg, rho);
         e = cudaGetLastError();

@@ -216,8 +216,8 @@ int apply_H_on_scratch(mb_handle *h, int ik, const void *X, void *Y, int nbands,
                        void *scratch);
 
 // density.cu: the electron density through row space (rs_supported handles);
-// nonneg: no occupation is negative (the result is then clamped at zero)
-int density_rows(mb_handle *h, const void *evecs, int nbands, const double *occ_dev, bool nonneg, double *rho,
+// occ: the occupations on the host, occ_dev: their copy on the device
+int density_rows(mb_handle *h, const void *evecs, int nbands, const double *occ, const double *occ_dev, double *rho,
                  cudaStream_t s);
 
 enum { BAND_S = 0, BAND_SINV = 1, BAND_PREC = 2 };

@@ -501,11 +501,10 @@ int check_tables(mb_handle *h) {
 }  // namespace
 
 // rho (device, nq x N1 x N2) from the eigenvectors evecs (the layout of
-// mb_eigsolve's) and the occupations occ_dev (device, nk x nbands).
-// nonneg: no occupation is negative.
-int scf_density(mb_handle *h, const void *evecs, int nbands, const double *occ_dev, bool nonneg, double *rho,
+// mb_eigsolve's) and the occupations occ (host, nk x nbands; occ_dev: device).
+int scf_density(mb_handle *h, const void *evecs, int nbands, const double *occ, const double *occ_dev, double *rho,
                 cudaStream_t s) {
-    if (rs_supported(h->n1, h->n2, h->order)) return density_rows(h, evecs, nbands, occ_dev, nonneg, rho, s);
+    if (rs_supported(h->n1, h->n2, h->order)) return density_rows(h, evecs, nbands, occ, occ_dev, rho, s);
     const int nk = (int)h->kp.size(), NN = h->n1 * h->n2, P = h->nquad;
     const int nmax = std::max(h->n1, h->n2);
     const int np = fft_planes(h, P);
@@ -796,8 +795,7 @@ int mb_density(mb_handle *h, const void *evecs, int nbands, const double *occ, d
     double *d_occ = B.get<double>(nocc);
     if (B.rc) return B.rc;
     MB_CUDA(cudaMemcpyAsync(d_occ, occ, sizeof(double) * nocc, cudaMemcpyHostToDevice, s));
-    const bool nonneg = std::all_of(occ, occ + nocc, [](double f) { return f >= 0.0; });
-    if ((rc = scf_density(h, evecs, nbands, d_occ, nonneg, rho, s))) return rc;
+    if ((rc = scf_density(h, evecs, nbands, occ, d_occ, rho, s))) return rc;
     MB_CUDA(cudaStreamSynchronize(s));   // the host occupations are read by the copy above
     return MB_OK;
 }
@@ -952,7 +950,7 @@ int mb_scf(mb_handle *h, const mb_scf_opts *o, double *evals, double *rho_out, m
             // output density and the mixed next input
             mu = occupations(ev, wk, nbands, nelec, o->sigma, f);
             MB_CUDA(cudaMemcpyAsync(occ, f.data(), sizeof(double) * f.size(), cudaMemcpyHostToDevice, s));
-            if ((rc = scf_density(h, evecs, nbands, occ, true, rho_o, s))) {
+            if ((rc = scf_density(h, evecs, nbands, f.data(), occ, rho_o, s))) {
                 result = rc;
                 break;
             }
