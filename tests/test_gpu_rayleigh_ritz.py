@@ -103,9 +103,10 @@ def test_bands_are_s_orthonormal(handle, nroots, prec, tol):
     assert (G - torch.eye(nroots, dtype=G.dtype, device="cuda")).abs().max().item() < tol
 
 
-@pytest.mark.parametrize("n,m", [(76, 112), (77, 56), (77, 57)])
+@pytest.mark.parametrize("n,m", [(76, 112), (77, 112), (305, 56), (305, 57)])
 def test_many_problems(handle, n, m):
-    """Around the number and size that the refinement's workspace holds."""
+    """The most that the refinement's workspace holds (max(304, n) 112^2 numbers
+    for four matrices a problem), and one more, which takes FP64 sweeps."""
     A = np.stack([(1 + 0.01 * p) * matrix("normal", m) for p in range(n)])
     ev, Y = rayleigh_ritz(handle, A)
     G = Y.conj().transpose(0, 2, 1) @ Y
